@@ -77,8 +77,18 @@ constexpr unsigned long long kEmpty = ~0ull;
 // 8 k_chunk_cost chunk counter, 9 tests of dense edges' members without a
 // dense slot (k_dense_pairs).
 constexpr int kStatSlots = 16;
-// Chunks per run a k_chunk_cost warp takes from its counter.
+// Chunks per run a k_chunk_cost warp takes from its counter, at most.
 constexpr int kCostGrab = 16;
+// Runs each warp should get to take from a counter: with fewer the work that
+// is left over at the end is a large share of a warp's time, and a call with
+// little work would leave most warps without a run (ER 2000/20000 exact:
+// k_quad 396 us with runs of 32 tasks, which is 640 runs for 9728 warps).
+constexpr int kRunsPerWarp = 8;
+// Items per run when `total` items are shared by `warps` warps.
+__device__ __forceinline__ int run_length(int64_t total, int64_t warps, int64_t most) {
+  const int64_t r = total / (warps * kRunsPerWarp);
+  return r < 1 ? 1 : (int)(r < most ? r : most);
+}
 // Filter of a dense edge's T members without a matrix slot in k_dense_pairs:
 // 2^15 bits, built when T has at most kTFilterMaxT entries.
 constexpr int kTFilterWords = 1024;
@@ -807,14 +817,16 @@ __global__ void __launch_bounds__(kThreads, kCostBlocksPerSm)
   EdgeCtx c;
   c.e = -1;
   int64_t next = -1;  // the chunk after this warp's previous run
-  // runs of kCostGrab consecutive chunks from a counter (chunks differ in
-  // cost: table answers, hub edges)
+  // runs of consecutive chunks from a counter (chunks differ in cost: table
+  // answers, hub edges)
+  const int grab =
+      run_length(groups, (int64_t)gridDim.x * (kThreads / 32), (int64_t)kCostGrab);
   for (;;) {
     unsigned long long got = 0;
-    if (lane == 0) got = atomicAdd(stats + 8, (unsigned long long)kCostGrab);
+    if (lane == 0) got = atomicAdd(stats + 8, (unsigned long long)grab);
     const int64_t g0 = (int64_t)__shfl_sync(kFull, got, 0);
     if (g0 >= groups) break;
-    const int64_t g1 = min(groups, g0 + (int64_t)kCostGrab);
+    const int64_t g1 = min(groups, g0 + grab);
     if (g0 != next) e = last_le(off, K, g0 * 32);
     next = g1;
     for (int64_t gi = g0; gi < g1; ++gi) {
@@ -964,7 +976,8 @@ __global__ void __launch_bounds__(kThreads, kQuadBlocksPerSm)
   // warps take runs of consecutive tasks from a counter: tasks differ in
   // cost (a chunk with few tests still pays a whole item set-up, tests
   // differ in latency), so fixed per-warp ranges left a long tail
-  const int64_t grab = max((int64_t)1, kQuadGrabTests / task_probes);
+  const int grab = run_length(NT, (int64_t)gridDim.x * (kThreads / 32),
+                              max((int64_t)1, kQuadGrabTests / task_probes));
   int64_t gi = 0, e = 0;
   int64_t cur = -1, cur_e = -1;
   int64_t start = 0, ctotal = 0;

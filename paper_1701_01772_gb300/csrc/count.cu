@@ -303,7 +303,7 @@ __global__ void k_compact_T(DevGraph g, const int2* __restrict__ uv, const int64
       // segment-A work of this edge in either mode: sparse = tests over the
       // shorter of N(w) above w / T above w (estimated); dense = for each
       // dense-slot member, the 128-bit groups of the T mask that hold a
-      // member and lie at or above its own (what k_dense_pairs reads), plus
+      // member and lie at or below its own (what k_dense_pairs reads), plus
       // the adjacency of the other members
       __syncwarp();  // this warp's T entries are visible to all its lanes
       const int64_t t0 = toff[e], te = pos - t0;
@@ -324,8 +324,8 @@ __global__ void k_compact_T(DevGraph g, const int2* __restrict__ uv, const int64
         sparse += min(dx / 2, te - j - 1);  // about half of N(x) lies above x
         if (xs >= 0 && xs < D) {
           const int g0 = xs >> 7;
-          groups += __popc(gb[g0 >> 5] & (~0u << (g0 & 31)));
-          for (int w = (g0 >> 5) + 1; w < kGroupWords; ++w) groups += __popc(gb[w]);
+          groups += __popc(gb[g0 >> 5] & (0xffffffffu >> (31 - (g0 & 31))));
+          for (int w = 0; w < (g0 >> 5); ++w) groups += __popc(gb[w]);
         } else {  // k_dense_pairs walks its matrix and non-matrix-above lists
           dense += g.mn_ptr != nullptr ? (__ldg(g.mn_ptr + x + 1) - __ldg(g.mn_ptr + x)) +
                                              (__ldg(g.nm_ptr + x + 1) - __ldg(g.nm_ptr + x))
@@ -387,7 +387,9 @@ __global__ void k_unit_fill(const int64_t* __restrict__ unit_off, int64_t ndense
 
 // Pairs of hub-matrix members of T in the dense edges: member w (slot s)
 // contributes popcount(w's matrix row AND the edge's T mask) over the bits
-// above s, so every adjacent pair of members counts once (k += 1, q += 2).
+// below s, so every adjacent pair of members counts once (k += 1, q += 2).
+// Slots are in decreasing degree, so T's members crowd in the low slots and
+// the groups at or below a member's own are few.
 // Work units are kDenseUnit consecutive T entries of one dense edge
 // (unit_off: exclusive scan of the units per dense edge, unit_idx: the
 // dense edge of each unit); a CTA takes one unit at a time from a counter
@@ -474,18 +476,18 @@ __global__ void __launch_bounds__(kThreads, kDenseBlocksPerSm)
         const int g0 = sl >> 7, b0 = sl & 127;
         const uint4* row = reinterpret_cast<const uint4*>(g.hm_bits + (int64_t)sl * g.hm_words);
         const int p0 = spos[g0];  // w's own group is non-zero (w is in T)
-        groups += L - p0;
-        for (int c = p0 + lane; c < L; c += 32) {
+        groups += p0 + 1;
+        for (int c = lane; c <= p0; c += 32) {
           const int gg = sgrp[c];
           const uint4 rw = ld_keep4(row + gg);
           const uint4 mk = smask[c];
           uint32_t wd[4] = {rw.x & mk.x, rw.y & mk.y, rw.z & mk.z, rw.w & mk.w};
-          if (gg == g0) {  // only the bits above w's own
+          if (gg == g0) {  // only the bits below w's own
 #pragma unroll
             for (int q4 = 0; q4 < 4; ++q4) {
               const int lo_bit = 32 * q4;
-              if (b0 >= lo_bit + 31) wd[q4] = 0u;
-              else if (b0 >= lo_bit) wd[q4] &= ~0u << (b0 - lo_bit + 1);
+              if (b0 <= lo_bit) wd[q4] = 0u;
+              else if (b0 < lo_bit + 32) wd[q4] &= (1u << (b0 - lo_bit)) - 1u;
             }
           }
           acc += __popc(wd[0]) + __popc(wd[1]) + __popc(wd[2]) + __popc(wd[3]);

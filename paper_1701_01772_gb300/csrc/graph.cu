@@ -109,8 +109,10 @@ __global__ void k_nbr_degsum(const int64_t* __restrict__ row_ptr, const int32_t*
 //            kMidMinDegree) against the top bg_count table vertices b, which
 //            answers most co-degree queries between a sampled edge's
 //            high-degree end and a low-degree neighbour.
-// Slots are assigned in increasing vertex id among vertices whose degree is
-// at least a threshold, so the index is deterministic.
+// Bitmap and table slots are assigned in increasing vertex id among the
+// vertices whose degree is at least a threshold; matrix slots and the mid x
+// big columns in decreasing degree (ties: increasing id), see k_degree_rank.
+// Both are deterministic.
 
 __global__ void k_count_deg_ge(const int64_t* __restrict__ row_ptr, int64_t n, int64_t d,
                                unsigned long long* cnt) {
@@ -139,6 +141,49 @@ __global__ void k_assign_slots(const int64_t* __restrict__ flag_scan, const int6
     int64_t s = flag_scan[v];
     slot[v] = f ? (int32_t)s : -1;
     if (f) hubs[s] = (int32_t)v;
+  }
+}
+
+// rank[s] += the number of vertices among hubs[tile] of higher (degree,
+// lower id) than hubs[s]: the slot of hubs[s] in decreasing degree. Blocks
+// (x: 256 hubs, y: one tile of kRankTile others) compare keys staged in
+// shared memory; 65,535 hubs are 4.3e9 comparisons.
+//
+// Why by degree: a hub lies in an edge's T, and is the end o of a co-degree
+// query c(w, o), the more often the higher its degree. With slots in id order
+// the members of a T mask were spread over all 256 128-bit groups of a matrix
+// row (34k group loads per dense edge of the 1M-vertex power-law graph); in
+// degree order they share the first few groups, and the hot words of a matrix
+// row or a mid x big row share sectors.
+constexpr int kRankTile = 1024;
+__global__ void k_degree_rank(const int64_t* __restrict__ row_ptr,
+                              const int32_t* __restrict__ hubs, int64_t count,
+                              unsigned int* __restrict__ rank) {
+  __shared__ uint64_t key[kRankTile];
+  auto key_of = [&](int64_t s) {
+    const int32_t v = hubs[s];
+    return ((uint64_t)(row_ptr[v + 1] - row_ptr[v]) << 32) | (uint32_t)(0x7fffffff - v);
+  };
+  const int64_t t0 = (int64_t)blockIdx.y * kRankTile;
+  const int tn = (int)min((int64_t)kRankTile, count - t0);
+  for (int i = threadIdx.x; i < tn; i += blockDim.x) key[i] = key_of(t0 + i);
+  __syncthreads();
+  const int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (s >= count) return;
+  const uint64_t mine = key_of(s);
+  unsigned int above = 0;
+  for (int i = 0; i < tn; ++i) above += key[i] > mine;
+  if (above) atomicAdd(rank + s, above);
+}
+
+__global__ void k_apply_rank(const unsigned int* __restrict__ rank,
+                             const int32_t* __restrict__ by_id, int64_t count,
+                             int32_t* __restrict__ slot, int32_t* __restrict__ hubs) {
+  for (int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; s < count;
+       s += (int64_t)gridDim.x * blockDim.x) {
+    const int32_t v = by_id[s];
+    slot[v] = (int32_t)rank[s];
+    hubs[rank[s]] = v;
   }
 }
 
@@ -841,13 +886,25 @@ static gs_status build_hub_index(gs_graph* g, uint64_t budget, cudaStream_t stre
   }
   guard.p[1] = flag;
   guard.p[2] = tmp;
-  auto assign = [&](int64_t d, int32_t** slot, int32_t** hubs, int64_t count) -> gs_status {
+  auto assign = [&](int64_t d, int32_t** slot, int32_t** hubs, int64_t count,
+                    bool by_degree) -> gs_status {
     GS_CUDA(cudaMalloc(slot, sizeof(int32_t) * (size_t)n));
     GS_CUDA(cudaMalloc(hubs, sizeof(int32_t) * (size_t)(count > 0 ? count : 1)));
     k_flag_deg_ge<<<grid_for(n, 256, 8), 256, 0, stream>>>(g->dev.row_ptr, n, d, flag);
     GS_TRY(exclusive_scan_i64(flag, flag, n, tmp, stream));
     k_assign_slots<<<grid_for(n, 256, 8), 256, 0, stream>>>(flag, g->dev.row_ptr, n, d, *slot,
                                                             *hubs);
+    if (by_degree && count > 0) {  // flag is free again: the ranks and the hubs by id
+      unsigned int* rank = reinterpret_cast<unsigned int*>(flag);
+      int32_t* by_id = reinterpret_cast<int32_t*>(flag) + count;
+      GS_CUDA(cudaMemsetAsync(rank, 0, sizeof(unsigned int) * (size_t)count, stream));
+      GS_CUDA(cudaMemcpyAsync(by_id, *hubs, sizeof(int32_t) * (size_t)count,
+                              cudaMemcpyDeviceToDevice, stream));
+      const dim3 grid((unsigned)((count + 255) / 256),
+                      (unsigned)((count + kRankTile - 1) / kRankTile));
+      k_degree_rank<<<grid, 256, 0, stream>>>(g->dev.row_ptr, by_id, count, rank);
+      k_apply_rank<<<grid_for(count, 256, 8), 256, 0, stream>>>(rank, by_id, count, *slot, *hubs);
+    }
     GS_CUDA(cudaGetLastError());
     return GS_OK;
   };
@@ -857,7 +914,7 @@ static gs_status build_hub_index(gs_graph* g, uint64_t budget, cudaStream_t stre
     GS_TRY(hub_threshold(g, bm_cap, kHubMinDegree, d_cnt, stream, &d_bm, &n_bm));
     if (n_bm > 0) {
       int32_t* hubs = nullptr;
-      GS_TRY(assign(d_bm, &g->bm_slot, &hubs, n_bm));
+      GS_TRY(assign(d_bm, &g->bm_slot, &hubs, n_bm, false));
       cudaError_t e = cudaMalloc(&g->bm_bits, sizeof(uint32_t) * (size_t)(words * n_bm));
       if (e != cudaSuccess) {
         cudaFree(hubs);
@@ -936,7 +993,7 @@ static gs_status build_hub_index(gs_graph* g, uint64_t budget, cudaStream_t stre
   if (hm_cap > 1) GS_TRY(hub_threshold(g, hm_cap, kHubMinDegree, d_cnt, stream, &d_hm, &n_hm));
   if (n_hm > 1) {
     int32_t* hubs = nullptr;
-    GS_TRY(assign(d_hm, &g->hm_slot, &hubs, n_hm));
+    GS_TRY(assign(d_hm, &g->hm_slot, &hubs, n_hm, true));
     // rows padded to a multiple of 4 words (128 bits) so that dense clique
     // counting can read a row and a T mask with aligned 16-byte loads
     const int64_t hm_words = (n_hm + 127) / 128 * 4;
@@ -997,7 +1054,7 @@ static gs_status build_hub_index(gs_graph* g, uint64_t budget, cudaStream_t stre
     GS_TRY(hub_threshold(g, tb_cap, kHubMinDegree, d_cnt, stream, &d_tb, &n_tb));
     if (n_tb > 1) {
       int32_t* hubs = nullptr;  // slot -> vertex, for the row build
-      GS_TRY(assign(d_tb, &g->tb_slot, &hubs, n_tb));
+      GS_TRY(assign(d_tb, &g->tb_slot, &hubs, n_tb, false));
       struct FreeHubs {
         int32_t* p;
         ~FreeHubs() { cudaFree(p); }
@@ -1156,7 +1213,7 @@ static gs_status build_hub_index(gs_graph* g, uint64_t budget, cudaStream_t stre
     const int64_t md_cap = n_bg > 0 ? 1 : 0;
     if (md_cap > 0 && d_md < d_hi) {
       int32_t* hubs = nullptr;
-      GS_TRY(assign(d_bg, &g->bg_slot, &hubs, n_bg));
+      GS_TRY(assign(d_bg, &g->bg_slot, &hubs, n_bg, true));
       cudaFree(hubs);
       k_flag_mid<<<grid_for(n, 256, 8), 256, 0, stream>>>(g->dev.row_ptr, g->tb_slot, n, d_md,
                                                           d_hi, flag);

@@ -160,16 +160,15 @@ extern "C" gs_status gs_batch_create(const int64_t* d_vtx_off, const int64_t* d_
         d_vtx_off, d_row_ptr, d_col, num_graphs, b->col_global, b->err);
   gs_status s = fetch_error(b->err, stream, "gs_batch_create (local vertex id out of range)");
   if (s != GS_OK) return fail(GS_EINVAL);
-  s = gs_graph_create(d_row_ptr, b->col_global, total_n, total_nnz, flags,
-                                hub_budget_bytes, stream, &b->graph);
+  // with adjacency bit matrices and co-degree blocks of the member graphs
+  // (all of them are small in the intended use): a membership test becomes
+  // one word load, a co-degree query one byte
+  s = create_graph(d_row_ptr, b->col_global, total_n, total_nnz, flags, hub_budget_bytes,
+                   hv.data(), num_graphs, stream, &b->graph);
   if (s != GS_OK) {
     b->graph = nullptr;
     return fail(s);
   }
-  // adjacency bit matrices for the member graphs (all of them are small in
-  // the intended use): every membership test becomes one word load
-  s = build_dense_blocks(b->graph, hv.data(), num_graphs, (uint64_t)24 << 30, stream);
-  if (s != GS_OK) return fail(s);
   k_batch_segments<<<grid_for(num_graphs + 1, 256, 4), 256, 0, stream>>>(
       d_vtx_off, b->graph->edge_off, num_graphs, b->seg_off);
   b->edges.resize(num_graphs + 1);

@@ -93,6 +93,10 @@ struct DevGraph {
   const uint32_t* dm_bits;
   const int64_t* dm_row;
   const int32_t* dm_first;
+  // co-degrees inside those blocks, 8 bits: c(v, x) = cg[cg_row[v] + x -
+  // dm_first[v]], 255 = not held (cg_row NULL or -1: no block)
+  const uint8_t* cg;
+  const int64_t* cg_row;
   const uint32_t* hm_bits;  // [hm_count][hm_words]
   int64_t hm_words;         // ceil(hm_count / 128) * 4
   // dense clique mode uses the first hm_dense_words * 32 slots (a multiple
@@ -273,6 +277,8 @@ struct gs_graph {
   uint32_t* dm_bits;
   int64_t* dm_row;
   int32_t* dm_first;
+  uint8_t* cg;
+  int64_t* cg_row;
   int32_t* bg_slot;
   uint16_t* md_codeg;
   int64_t* dir_at;
@@ -321,12 +327,11 @@ namespace gs {
 // Graphs (or batch members) of at most this many vertices get an adjacency
 // bit matrix (at most 32 MiB each).
 constexpr int64_t kDenseGraphMax = 16384;
-// Builds adjacency bit-matrix blocks for the vertex ranges [first[i],
-// first[i+1]) of at most kDenseGraphMax vertices (ranges = member graphs of a
-// disjoint union; a single range [0, n) for one graph). Skipped silently when
-// the blocks would exceed max_bytes or cannot be allocated.
-gs_status build_dense_blocks(gs_graph* g, const int64_t* h_first, int64_t ranges,
-                             uint64_t max_bytes, cudaStream_t stream);
+// Registration (gs_graph_create). h_first: the member graphs' vertex ranges
+// [h_first[i], h_first[i + 1]) of a disjoint union, or NULL for one graph.
+gs_status create_graph(const int64_t* d_row_ptr, const int32_t* d_col, int64_t n, int64_t nnz,
+                       uint32_t flags, uint64_t hub_budget_bytes, const int64_t* h_first,
+                       int64_t ranges, cudaStream_t stream, gs_graph** out);
 // Returns a device buffer of at least `bytes` in slot `slot` of the
 // workspace, growing it (after synchronising the stream it was last used
 // on) when needed. Previously held contents of that slot are lost on growth.

@@ -655,6 +655,17 @@ struct EdgeCtx {
   const uint32_t* tmask;  // this edge's T mask (dense edges), else NULL
 };
 
+// Rows of the endpoints in a small graph's co-degree block, shifted so that
+// the entry of vertex w is row[w] (NULL without a block).
+struct BlockRows {
+  const uint8_t *u, *v;
+};
+
+__device__ __forceinline__ const uint8_t* block_row(const DevGraph& g, int32_t o) {
+  const int64_t r = __ldg(g.cg_row + o);
+  return r >= 0 ? g.cg + (r - __ldg(g.dm_first + o)) : nullptr;
+}
+
 __device__ __forceinline__ void load_edge(const DevGraph& g, const int2* __restrict__ uv,
                                           const unsigned long long* __restrict__ t,
                                           const int64_t* __restrict__ toff,
@@ -761,9 +772,9 @@ struct ItemCost {
   bool tabled;     // a co-degree table answered segment B
 };
 
-__device__ __forceinline__ ItemCost item_cost(const DevGraph& g, const EdgeCtx& c, int64_t i,
-                                              uint32_t tword, int32_t tbase, int lane,
-                                              bool need_q) {
+__device__ __forceinline__ ItemCost item_cost(const DevGraph& g, const EdgeCtx& c,
+                                              const BlockRows& rows, int64_t i, uint32_t tword,
+                                              int32_t tbase, int lane, bool need_q) {
   ItemCost r{0, 0, 0, false};
   if (i >= c.du) return r;
   const int64_t p = c.bu + i;
@@ -786,9 +797,17 @@ __device__ __forceinline__ ItemCost item_cost(const DevGraph& g, const EdgeCtx& 
   if (need_q) {
     // segment B: -(c(w, u) - 1) for w in T, c(w, v) - 1 for w in S_u
     const int32_t o = in_t ? c.u : c.v;
-    const int32_t sw = g.col_tb != nullptr ? __ldg(g.col_tb + p)
-                       : g.tb_slot != nullptr ? __ldg(g.tb_slot + w) : -1;
-    const uint32_t tc = table_codeg_s(g, w, sw, o);
+    const uint8_t* row = in_t ? rows.u : rows.v;
+    uint32_t tc = 0;
+    if (row != nullptr) {
+      const uint32_t b = __ldg(row + w);
+      if (b < 255u) tc = b + 1u;
+    }
+    if (tc == 0) {
+      const int32_t sw = g.col_tb != nullptr ? __ldg(g.col_tb + p)
+                         : g.tb_slot != nullptr ? __ldg(g.tb_slot + w) : -1;
+      tc = table_codeg_s(g, w, sw, o);
+    }
     r.tabled = tc != 0;
     if (tc != 0) {
       r.qconst = in_t ? 1 - (int64_t)(tc - 1u) : (int64_t)(tc - 1u) - 1;
@@ -818,6 +837,7 @@ __global__ void __launch_bounds__(kThreads, kCostBlocksPerSm)
   int64_t e = 0;
   EdgeCtx c;
   c.e = -1;
+  BlockRows rows{nullptr, nullptr};
   int64_t next = -1;  // the chunk after this warp's previous run
   // runs of consecutive chunks from a counter (chunks differ in cost: table
   // answers, hub edges)
@@ -833,8 +853,14 @@ __global__ void __launch_bounds__(kThreads, kCostBlocksPerSm)
     next = g1;
     for (int64_t gi = g0; gi < g1; ++gi) {
       while (e + 1 < K && __ldg(off + e + 1) <= gi * 32) ++e;
-      if (e != c.e) load_edge(g, uv, t, toff, mask_idx, tmask, e, c);
-      const ItemCost it = item_cost(g, c, gi * 32 + lane - __ldg(off + e), __ldg(tbits + gi),
+      if (e != c.e) {
+        load_edge(g, uv, t, toff, mask_idx, tmask, e, c);
+        if (g.cg_row != nullptr) {
+          rows.u = block_row(g, c.u);
+          rows.v = block_row(g, c.v);
+        }
+      }
+      const ItemCost it = item_cost(g, c, rows, gi * 32 + lane - __ldg(off + e), __ldg(tbits + gi),
                                     __ldg(tpre + gi), lane, need_q);
       const unsigned live = __ballot_sync(kFull, it.a + it.b > 0);
       const unsigned tabled = __ballot_sync(kFull, it.tabled);
@@ -1367,6 +1393,8 @@ DevGraph graph_view(const gs_graph* gr, const Tuning& tu) {
     g.dir_at = nullptr;
     g.dir = nullptr;
     g.col_tb = nullptr;
+    g.cg = nullptr;
+    g.cg_row = nullptr;
   }
   return g;
 }

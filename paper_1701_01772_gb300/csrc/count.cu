@@ -35,12 +35,11 @@
 //            count of each item (iterate the shorter list, test in the
 //            longer); constant terms (the -1s, table co-degrees) added
 //            directly; two ballots per chunk (items with tests, items a table
-//            answered) for the 4-node pass.
-//   quad     chunks are cut into tasks of task_probes tests; warps take
+//            answered) for the 4-node pass; consecutive chunks with at most
+//            32 items with tests in all form a pack.
+//   quad     packs are cut into tasks of task_probes tests; warps take
 //            runs of consecutive tasks from a counter; inside a task lanes
-//            take consecutive tests (two per lane per iteration) and find
-//            their item by a search over the warp's scanned costs
-//            (load-balanced search).
+//            take consecutive tests (two per lane per iteration).
 //   dense    in a dense edge segment A is counted by k_dense_pairs, in work
 //            units of kDenseUnit T entries: pairs of dense-slot members by
 //            matrix rows ANDed with the T mask, 128 bits at a time; for the
@@ -77,7 +76,8 @@ constexpr unsigned long long kEmpty = ~0ull;
 // 8 k_chunk_cost chunk counter, 9 tests of dense edges' members without a
 // dense slot (k_dense_pairs).
 constexpr int kStatSlots = 16;
-// Chunks per run a k_chunk_cost warp takes from its counter, at most.
+// Chunks per run a k_chunk_cost warp takes from its counter, at most; also
+// the most chunks a pack of k_quad spans (packs do not cross runs), at most 32.
 constexpr int kCostGrab = 16;
 // Runs each warp should get to take from a counter: with fewer the work that
 // is left over at the end is a large share of a warp's time, and a call with
@@ -711,13 +711,6 @@ __device__ __forceinline__ uint32_t table_codeg_s(const DevGraph& g, int32_t a, 
   return 0;
 }
 
-// What the cost pass learnt about an item, for the 4-node pass: it has
-// tests, and a co-degree table answered its segment B (so the 4-node pass
-// needs neither the table nor the item when it has no tests). The constant
-// q terms are added by the cost pass alone.
-constexpr int kHintLive = 1;
-constexpr int kHintTabled = 2;
-
 // sslot value marking a searched vertex whose adjacency is a dense bit-matrix
 // row: sl then points at the row and sbm holds the first vertex of the block.
 constexpr int32_t kDenseRow = -3;
@@ -851,6 +844,11 @@ __global__ void __launch_bounds__(kThreads, kCostBlocksPerSm)
     const int64_t g1 = min(groups, g0 + grab);
     if (g0 != next) e = last_le(off, K, g0 * 32);
     next = g1;
+    // packs: consecutive chunks of the run with at most 32 live items in all,
+    // so that k_quad sets up a warp's worth of items at a time; a pack's
+    // tasks are counted at its first chunk
+    int64_t head = g0, pcost = 0;
+    int plive = 0;
     for (int64_t gi = g0; gi < g1; ++gi) {
       while (e + 1 < K && __ldg(off + e + 1) <= gi * 32) ++e;
       if (e != c.e) {
@@ -865,14 +863,23 @@ __global__ void __launch_bounds__(kThreads, kCostBlocksPerSm)
       const unsigned live = __ballot_sync(kFull, it.a + it.b > 0);
       const unsigned tabled = __ballot_sync(kFull, it.tabled);
       if (lane == 0) reinterpret_cast<uint2*>(cbits)[gi] = make_uint2(live, tabled);
-      int64_t cost = warp_sum<int64_t>((int64_t)it.a + it.b);
-      int64_t qc = warp_sum<int64_t>(it.qconst);
+      const int64_t cost = live ? warp_sum<int64_t>((int64_t)it.a + it.b) : 0;
+      const int64_t qc = warp_sum<int64_t>(it.qconst);
+      if (plive + __popc(live) > 32) {
+        if (lane == 0) task_cnt[head] = (pcost + task_probes - 1) / task_probes;
+        head = gi;
+        pcost = 0;
+        plive = 0;
+      }
+      pcost += cost;
+      plive += __popc(live);
       if (lane == 0) {
-        task_cnt[gi] = (cost + task_probes - 1) / task_probes;
+        if (gi != head) task_cnt[gi] = 0;
         if (qc != 0) atomicAdd(q + e, (unsigned long long)qc);
         tests += cost;
       }
     }
+    if (lane == 0) task_cnt[head] = (pcost + task_probes - 1) / task_probes;
   }
   if (lane == 0 && tests) atomicAdd(stats + 1, (unsigned long long)tests);
 }
@@ -895,68 +902,72 @@ __device__ __forceinline__ bool bucket_contains(const int32_t* __restrict__ p, i
   return sorted_contains(p, len, x);
 }
 
-// Kept to 64 bytes: eight CTAs of 256 items then take 128 KB of shared
-// memory, which leaves the rest of the SM's 256 KB to the L1 cache that the
-// membership tests depend on. The matrix slots of an iterated list are found
-// beside it (col_hm for adjacency lists, T_hm for T) and the segment-B sign
-// is stored in one word.
-struct SharedItem {
-  const int32_t* it[2];
-  const int32_t* sl[2];
-  int32_t sbm[2];
-  int32_t slen[2];
-  int16_t sslot[2];
-  int32_t ca;
-  int32_t mode;  // (bsign + 1) << 8
+// The items of the pack a warp works on, field by field so that lanes that
+// read different items hit different banks (60 bytes per item: eight CTAs of
+// 256 items take 120 KB of shared memory, which leaves the rest of the SM's
+// 256 KB to the L1 cache that the membership tests depend on). Only items
+// with tests are kept, in order of position. [0] is segment A, [1] segment B.
+// The matrix slots of an iterated list are found beside it (col_hm for
+// adjacency lists, T_hm for T).
+struct WarpItems {
+  const int32_t* it[2][32];
+  const int32_t* sl[2][32];
+  int32_t sbm[2][32];
+  int32_t slen[2][32];
+  int32_t ca[32];       // tests of segment A; its hits count +1 in k, +2 in q
+  int16_t sslot[2][32];
+  int16_t bsign[32];    // segment B adds it to q per hit
+  uint16_t who[32];     // chunk of the pack (high bits) and bit of each item
 };
-static_assert(sizeof(SharedItem) == 64, "SharedItem size");
+static_assert(sizeof(WarpItems) == 60 * 32, "WarpItems size");
 
-// Item set-up of k_quad, out of line: it runs once per chunk and its
+// Item set-up of k_quad, out of line: it runs once per pack and its
 // temporaries would otherwise raise the register count of the test loop.
-// Derives the same segments as item_cost counts, with the cost pass's hint
-// in place of the table reads, and stores each field to the lane's
-// shared-memory descriptor as soon as it is known (only the segments that
-// have tests are written; a segment with no tests is never read). Returns
-// the item's test count.
+// Derives the same segments as item_cost counts for position i of edge e
+// (bit `bit` of its chunk, an item with tests), with the cost pass's word on
+// whether a table answered segment B in place of the table reads, and stores each field to place `at` of the
+// warp's item arrays as soon as it is known (only the segments that have
+// tests are written; a segment with no tests is never read). Returns the
+// item's test count.
 __device__ __noinline__ int64_t setup_item(const DevGraph& g, const int2* __restrict__ uv,
                                            const unsigned long long* __restrict__ t,
                                            const int64_t* __restrict__ toff,
                                            const int32_t* __restrict__ mask_idx,
                                            const uint32_t* __restrict__ tmask, int64_t e,
                                            const int32_t* __restrict__ T, int64_t i,
-                                           uint32_t tword, int32_t tbase, int lane, bool need_q,
-                                           int hint, SharedItem* si) {
+                                           uint32_t tword, int32_t tbase, int bit, bool need_q,
+                                           bool tabled, WarpItems* wi, int at) {
   EdgeCtx c;
   load_edge(g, uv, t, toff, mask_idx, tmask, e, c);
   int32_t ca = 0, cb = 0, bsign = 0;
-  if (i < c.du && (hint & kHintLive)) {
+  if (i < c.du) {
     const int32_t w = __ldg(g.col + c.bu + i);
     if (w != c.v) {
-      const bool in_t = (tword >> lane) & 1u;
+      const bool in_t = (tword >> bit) & 1u;
       int64_t bw;
       const int64_t dw = deg_of(g.row_ptr, w, &bw);
       if (in_t && c.tmask != nullptr) {
         // dense edge: segment A is done by k_dense_pairs
       } else if (in_t) {
-        const int64_t iw = tbase + __popc(tword & ((1u << lane) - 1u));
+        const int64_t iw = tbase + __popc(tword & ((1u << bit) - 1u));
         const int64_t tg = c.te - iw - 1;
         const int64_t upw = __ldg(g.up_ptr + w);
         const int64_t dup = bw + dw - upw;
         if (dup <= tg) {
-          si->it[0] = g.col + upw;
-          si->sl[0] = T + c.toff + iw + 1;
-          si->slen[0] = (int32_t)tg;
-          si->sslot[0] = -1;
-          si->sbm[0] = -1;
+          wi->it[0][at] = g.col + upw;
+          wi->sl[0][at] = T + c.toff + iw + 1;
+          wi->slen[0][at] = (int32_t)tg;
+          wi->sslot[0][at] = -1;
+          wi->sbm[0][at] = -1;
           ca = (int32_t)dup;
         } else {
           Seg sa;
           set_search(g, w, bw, dw, sa);
-          si->it[0] = T + c.toff + iw + 1;
-          si->sl[0] = sa.sl;
-          si->slen[0] = sa.slen;
-          si->sslot[0] = (int16_t)sa.sslot;
-          si->sbm[0] = sa.sbm;
+          wi->it[0][at] = T + c.toff + iw + 1;
+          wi->sl[0][at] = sa.sl;
+          wi->slen[0][at] = sa.slen;
+          wi->sslot[0][at] = (int16_t)sa.sslot;
+          wi->sbm[0][at] = sa.sbm;
           ca = (int32_t)tg;
         }
       }
@@ -964,27 +975,103 @@ __device__ __noinline__ int64_t setup_item(const DevGraph& g, const int2* __rest
         // segment B: c(w, u) for w in T (q -= 1 per hit), c(w, v) for w in
         // S_u (q += 1 per hit), unless a co-degree table answered it
         bsign = in_t ? -1 : 1;
-        if (!(hint & kHintTabled)) {
+        if (!tabled) {
           Seg sb;
           if (in_t) codeg_segment(g, w, bw, dw, c.u, c.bu, c.du, sb);
           else codeg_segment(g, w, bw, dw, c.v, c.bv, c.dv, sb);
-          si->it[1] = sb.it;
-          si->sl[1] = sb.sl;
-          si->slen[1] = sb.slen;
-          si->sslot[1] = (int16_t)sb.sslot;
-          si->sbm[1] = sb.sbm;
+          wi->it[1][at] = sb.it;
+          wi->sl[1][at] = sb.sl;
+          wi->slen[1][at] = sb.slen;
+          wi->sslot[1][at] = (int16_t)sb.sslot;
+          wi->sbm[1][at] = sb.sbm;
           cb = sb.cnt;
         }
       }
     }
   }
-  si->ca = ca;
-  // per-hit weights: segment A adds one 4-clique pair (k += 1, q += 2 when q
-  // is wanted); segment B adds bsign to q
-  si->mode = (bsign + 1) << 8;
+  wi->ca[at] = ca;
+  wi->bsign[at] = bsign;
   return (int64_t)ca + cb;
 }
 
+// One side of a membership test, as loaded so far: a word and a bit to test
+// (matrix, bitmap, dense row), the bounds of a directory bucket, or nothing
+// yet (a halving search is left).
+struct Probe {
+  uint32_t word, bit;
+  int how;  // 0 search, 1 word, 2 bucket
+};
+
+// First loads of the test "x in the searched set". xs: x's matrix slot, -1
+// when it has none; kMayMatrix false: the set has no matrix row (sslot < 0).
+template <bool kMayMatrix>
+__device__ __forceinline__ Probe probe_begin(const DevGraph& g, int sslot, int32_t sbm,
+                                             const int32_t* sl, int32_t slen, int32_t x,
+                                             int32_t xs) {
+  Probe p{0u, 0u, 0};
+  if (kMayMatrix && sslot >= 0 && xs >= 0) {
+    p.word = ld_keep(g.hm_bits + (int64_t)sslot * g.hm_words + (xs >> 5));
+    p.bit = xs & 31;
+    p.how = 1;
+  } else if (sslot == kDenseRow) {
+    const int32_t lx = x - sbm;
+    p.word = __ldg(reinterpret_cast<const uint32_t*>(sl) + (lx >> 5));
+    p.bit = lx & 31;
+    p.how = 1;
+  } else if (sbm >= 0) {
+    p.word = __ldg(g.bm_bits + (int64_t)sbm * g.bm_words + (x >> 5));
+    p.bit = x & 31;
+    p.how = 1;
+  } else if (sbm < -1) {
+    const uint32_t* d = g.dir + (uint32_t)slen + (uint32_t)(x >> (-2 - sbm));
+    p.word = __ldg(d);
+    p.bit = __ldg(d + 1);
+    p.how = 2;
+  }
+  return p;
+}
+
+__device__ __forceinline__ bool probe_end(const Probe& p, const int32_t* sl, int32_t slen,
+                                          int32_t x) {
+  return p.how == 1   ? ((p.word >> p.bit) & 1u) != 0
+         : p.how == 2 ? bucket_contains(sl + p.word, (int32_t)(p.bit - p.word), x)
+                      : sorted_contains(sl, slen, x);
+}
+
+// Matrix slots beside an iterated list: col_hm for an adjacency list, T_hm
+// for a T list (NULL without a matrix).
+__device__ __forceinline__ const int16_t* slots_beside(const DevGraph& g, const int32_t* it,
+                                                       const int32_t* T, const int16_t* T_hm) {
+  if (T_hm == nullptr) return nullptr;
+  const size_t pc = (size_t)(it - g.col);
+  return pc < (size_t)g.nnz ? g.col_hm + pc : T_hm + (it - T);
+}
+
+// Bits [0, x) of a word, x clamped to 0..32.
+__device__ __forceinline__ unsigned bits_below(int32_t x) {
+  return x <= 0 ? 0u : x >= 32 ? kFull : (1u << x) - 1u;
+}
+
+// The 4-node membership tests. A pack is up to 32 items with tests from
+// consecutive chunks (of one edge or several); its tests (the items' segments
+// A and B in order) are one index space, cut into tasks of task_probes tests.
+// A warp walks a task from test r on in one of two ways:
+//   run   the next 64 or more tests belong to one segment: its descriptor is
+//         the same in every lane, so the set searched and the way it answers
+//         are chosen once per run, and lanes take consecutive elements, two
+//         each per step;
+//   mixed otherwise, 64 tests of several items: each lane finds the item of
+//         its two tests from bit masks of the item starts among those 64
+//         (one warp reduction per 32), and reads its descriptor.
+// Lane i owns item i: it counts the item's hits from the hit ballots, whose
+// bits [start, end) are the item's tests, and adds them to the item's edge.
+//
+// Why packs: a chunk of 32 positions has few items left after the tables
+// (3.8 on the 1M-vertex power-law graph, 11 on R-MAT 24), so setting up one
+// chunk at a time left most lanes idle in the set-up, which was most of the
+// work there (850 of 1390 warp instructions per chunk). Eight CTAs per SM at
+// 32 registers, some spilled, hide more latency than six at 40 (R-MAT 24
+// 0.1%: 151 against 160 ms; 1M-vertex power-law exact 456 against 457 ms).
 __global__ void __launch_bounds__(kThreads, kQuadBlocksPerSm)
     k_quad(const __grid_constant__ DevGraph g, const int2* __restrict__ uv, const int64_t* __restrict__ off, int64_t K,
            const unsigned long long* __restrict__ t, const int64_t* __restrict__ toff,
@@ -997,169 +1084,204 @@ __global__ void __launch_bounds__(kThreads, kQuadBlocksPerSm)
            unsigned long long* __restrict__ k_out,
            unsigned long long* __restrict__ q,
            unsigned long long* __restrict__ task_counter) {
-  __shared__ SharedItem items[kThreads / 32][32];
+  __shared__ WarpItems items[kThreads / 32];
   const int lane = threadIdx.x & 31;
-  SharedItem* my = items[threadIdx.x >> 5];
-  const int64_t NT = __ldg(task_off + groups);
+  const unsigned upto = kFull >> (31 - lane);
+  WarpItems* my = items + (threadIdx.x >> 5);
   // warps take runs of consecutive tasks from a counter: tasks differ in
-  // cost (a chunk with few tests still pays a whole item set-up, tests
+  // cost (a pack with few tests still pays a whole item set-up, tests
   // differ in latency), so fixed per-warp ranges left a long tail
-  const int grab = run_length(NT, (int64_t)gridDim.x * (kThreads / 32),
+  const int grab = run_length(__ldg(task_off + groups), (int64_t)gridDim.x * (kThreads / 32),
                               max((int64_t)1, kQuadGrabTests / task_probes));
-  int64_t gi = 0, e = 0;
-  int64_t cur = -1, cur_e = -1;
-  int64_t start = 0, ctotal = 0;
-  unsigned acc_k = 0;
-  int acc_q = 0;
-  int64_t next = -1;  // the task after this warp's previous run
   for (;;) {
     unsigned long long got = 0;
     if (lane == 0) got = atomicAdd(task_counter, (unsigned long long)grab);
-    const int64_t t0 = (int64_t)__shfl_sync(kFull, got, 0);
-    if (t0 >= NT) break;
-    const int64_t t1 = min(NT, t0 + grab);
-    if (t0 != next) {
-      gi = last_le(task_off, groups, t0);
-      e = last_le(off, K, gi * 32);
-    }
-    next = t1;
-    for (int64_t task = t0; task < t1; ++task) {
-      while (gi + 1 < groups && __ldg(task_off + gi + 1) <= task) ++gi;
-      if (gi != cur) {
-        // flush the previous chunk's counts to its edge
-        const unsigned long long sk = warp_sum<unsigned long long>(acc_k);
-        const long long sq = warp_sum<long long>(acc_q);
-        if (lane == 0 && cur >= 0) {
-          if (sk) atomicAdd(k_out + cur_e, sk);
-          if (sq) atomicAdd(q + cur_e, (unsigned long long)sq);
-        }
-        acc_k = 0;
-        acc_q = 0;
-        while (e + 1 < K && __ldg(off + e + 1) <= gi * 32) ++e;
-        __syncwarp();
-        const uint2 cb = __ldg(reinterpret_cast<const uint2*>(cbits) + gi);
-        const int hint = (int)((cb.x >> lane) & 1u) * kHintLive +
-                         (int)((cb.y >> lane) & 1u) * kHintTabled;
-        const int64_t mine =
-            setup_item(g, uv, t, toff, mask_idx, tmask, e, T, gi * 32 + lane - __ldg(off + e),
-                       __ldg(tbits + gi), __ldg(tpre + gi), lane, need_q, hint, my + lane);
-        __syncwarp();
-        int64_t incl = mine;
-#pragma unroll
-        for (int d = 1; d < 32; d <<= 1) {
-          int64_t y = __shfl_up_sync(kFull, incl, d);
-          if (lane >= d) incl += y;
-        }
-        start = incl - mine;
-        ctotal = __shfl_sync(kFull, incl, 31);
-        cur = gi;
-        cur_e = e;
+    int64_t task = (int64_t)__shfl_sync(kFull, got, 0);
+    int left = (int)min((int64_t)grab, __ldg(task_off + groups) - task);
+    if (left <= 0) break;
+    int64_t gi = last_le(task_off, groups, task);
+    int64_t e0 = last_le(off, K, gi * 32);
+    while (left > 0) {
+      // the tasks of this run that lie in the pack at chunk gi
+      while (__ldg(task_off + gi + 1) <= task) ++gi;
+      while (e0 + 1 < K && __ldg(off + e0 + 1) <= gi * 32) ++e0;
+      int here = (int)min((int64_t)left, __ldg(task_off + gi + 1) - task);
+      left -= here;
+      // lane c: chunk gi + c of the pack (up to the next chunk with tasks of
+      // its own) and the items with tests in it
+      uint2 cb = make_uint2(0u, 0u);
+      bool own = false;
+      if (lane < kCostGrab && gi + lane < groups) {
+        cb = __ldg(reinterpret_cast<const uint2*>(cbits) + gi + lane);
+        own = lane > 0 && __ldg(task_off + gi + lane + 1) > __ldg(task_off + gi + lane);
       }
-      const int64_t lo = (task - __ldg(task_off + gi)) * task_probes;
-      const int32_t len = (int32_t)min(ctotal - lo, task_probes);
-      // item starts relative to the task's first test, in 32 bits: clamping
-      // keeps their order and never touches the item that holds a test of
-      // this task (it starts less than one item's tests before lo)
-      const int32_t srel = (int32_t)max(min(start - lo, task_probes), (int64_t)INT32_MIN + 1);
-      // Two independent tests per lane per iteration (r and r + 32): their
-      // loads are issued together so each warp keeps more requests in flight.
-      for (int32_t r = lane; r - lane < len; r += 64) {
-        int32_t x[2], xs[2], seg[2], o[2];
-        const SharedItem* it[2];
-        bool act[2];
+      const unsigned heads = __ballot_sync(kFull, own);
+      if (heads && lane >= __ffs(heads) - 1) cb.x = 0u;
+      int upto_c = __popc(cb.x);
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          const int32_t rr = r + 32 * h;  // test index within the task
-          int j = 0;  // item = last lane whose start <= rr
+      for (int d = 1; d < 32; d <<= 1) {
+        const int y = __shfl_up_sync(kFull, upto_c, d);
+        if (lane >= d) upto_c += y;
+      }
+      const int live = __shfl_sync(kFull, upto_c, 31);
+      __syncwarp();  // the previous pack's descriptors are no longer read
+      for (unsigned bits = cb.x, k = upto_c - __popc(cb.x); bits; bits &= bits - 1, ++k) {
+        const int b = __ffs(bits) - 1;
+        my->who[k] = (uint16_t)((lane << 6) | (((cb.y >> b) & 1u) << 5) | b);
+      }
+      __syncwarp();
+      // lane i: the set-up of item i
+      int64_t e = e0, mine = 0;
+      if (lane < live) {
+        const int who = my->who[lane];
+        const int64_t gc = gi + (who >> 6);
+        while (e + 1 < K && __ldg(off + e + 1) <= gc * 32) ++e;
+        mine = setup_item(g, uv, t, toff, mask_idx, tmask, e, T,
+                          gc * 32 + (who & 31) - __ldg(off + e), __ldg(tbits + gc),
+                          __ldg(tpre + gc), who & 31, need_q, ((who >> 5) & 1) != 0, my, lane);
+      }
+      __syncwarp();
+      int64_t start = mine;  // first test of the item; the total past the items
 #pragma unroll
-          for (int step = 16; step > 0; step >>= 1) {
-            const int32_t sv = __shfl_sync(kFull, srel, j + step);
-            if (sv <= rr) j += step;
-          }
-          const int32_t sj = __shfl_sync(kFull, srel, j);
-          act[h] = rr < len;
-          it[h] = &my[j];
-          o[h] = rr - sj;
-          seg[h] = o[h] < it[h]->ca ? 0 : 1;
-          if (seg[h]) o[h] -= it[h]->ca;
-          x[h] = 0;
-          xs[h] = -1;
-          if (act[h]) {
-            const int32_t* ip = it[h]->it[seg[h]] + o[h];
-            x[h] = __ldg(ip);
-            xs[h] = kNoSlotInfo;
-            if (T_hm != nullptr) {  // matrix slots stored beside the list
-              const size_t pc = (size_t)(ip - g.col);
-              xs[h] = pc < (size_t)g.nnz ? (int32_t)__ldg(g.col_hm + pc)
-                                         : (int32_t)__ldg(T_hm + (ip - T));
+      for (int d = 1; d < 32; d <<= 1) {
+        int64_t y = __shfl_up_sync(kFull, start, d);
+        if (lane >= d) start += y;
+      }
+      const int64_t ctotal = __shfl_sync(kFull, start, 31);
+      start -= mine;
+      unsigned long long acc_a = 0, acc_b = 0;  // hits of the lane's item
+      for (; here > 0; --here, ++task) {
+        const int64_t lo = (task - __ldg(task_off + gi)) * task_probes;
+        const int32_t len = (int32_t)min(ctotal - lo, task_probes);
+        // item starts relative to the task's first test, in 32 bits: clamping
+        // keeps their order and never touches the item that holds a test of
+        // this task (it starts less than one item's tests before lo)
+        const int32_t srel = (int32_t)max(min(start - lo, task_probes), (int64_t)INT32_MIN + 1);
+        // segment B of the item starts at sb, the item ends at se
+        const int32_t sb =
+            (int32_t)max(min(start - lo + (lane < live ? my->ca[lane] : 0), task_probes),
+                         (int64_t)INT32_MIN + 1);
+        const int32_t sd = __shfl_down_sync(kFull, srel, 1);
+        const int32_t se = lane < 31 ? min(sd, len) : len;
+        for (int32_t r = 0; r < len;) {
+          // item of test r: the last one that starts at or before it (lanes
+          // past the items hold the total, which is at or past len)
+          const int j0 = 31 - __clz(__ballot_sync(kFull, srel <= r));
+          const int32_t sj = __shfl_sync(kFull, srel, j0);
+          const int32_t sbj = __shfl_sync(kFull, sb, j0);
+          const int32_t sej = __shfl_sync(kFull, se, j0);
+          const int sg = r >= sbj ? 1 : 0;
+          const int32_t end = sg ? sej : min(sbj, len);
+          if (end - r >= 64) {
+            const int32_t* it = my->it[sg][j0] + (r - (sg ? sbj : sj)) + lane;
+            const int32_t* sl = my->sl[sg][j0];
+            const int32_t sbm = my->sbm[sg][j0], slen = my->slen[sg][j0];
+            const int sslot = my->sslot[sg][j0];
+            unsigned hits = 0;
+            const int32_t n = (end - r) & ~63;
+            r += n;
+            if (sslot >= 0) {
+              const int16_t* hs = slots_beside(g, it, T, T_hm);
+              for (int32_t i = 0; i < n; i += 64) {
+                const int32_t x0 = __ldg(it + i), x1 = __ldg(it + i + 32);
+                int32_t s0, s1;
+                if (hs != nullptr) {
+                  s0 = __ldg(hs + i);
+                  s1 = __ldg(hs + i + 32);
+                } else {
+                  s0 = __ldg(g.hm_slot + x0);
+                  s1 = __ldg(g.hm_slot + x1);
+                }
+                const Probe p0 = probe_begin<true>(g, sslot, sbm, sl, slen, x0, s0);
+                const Probe p1 = probe_begin<true>(g, sslot, sbm, sl, slen, x1, s1);
+                hits += probe_end(p0, sl, slen, x0);
+                hits += probe_end(p1, sl, slen, x1);
+              }
+            } else {
+              for (int32_t i = 0; i < n; i += 64) {
+                const int32_t x0 = __ldg(it + i), x1 = __ldg(it + i + 32);
+                const Probe p0 = probe_begin<false>(g, sslot, sbm, sl, slen, x0, -1);
+                const Probe p1 = probe_begin<false>(g, sslot, sbm, sl, slen, x1, -1);
+                hits += probe_end(p0, sl, slen, x0);
+                hits += probe_end(p1, sl, slen, x1);
+              }
             }
-          }
-        }
-        // constant-time word for matrix / bitmap answers, or the bucket bounds
-        // of a directory, issued for both
-        uint32_t word[2], bitpos[2];
-        bool direct[2], bucket[2];
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          direct[h] = false;
-          bucket[h] = false;
-          word[h] = 0;
-          bitpos[h] = 0;
-          if (!act[h]) continue;
-          const int sslot = it[h]->sslot[seg[h]];
-          if (sslot == kDenseRow) {
-            const int32_t lx = x[h] - it[h]->sbm[seg[h]];
-            word[h] = __ldg(reinterpret_cast<const uint32_t*>(it[h]->sl[seg[h]]) + (lx >> 5));
-            bitpos[h] = lx & 31;
-            direct[h] = true;
+            hits = __reduce_add_sync(kFull, hits);
+            if (lane == j0) {
+              if (sg) acc_b += hits;
+              else acc_a += hits;
+            }
             continue;
           }
-          if (sslot >= 0) {
-            if (xs[h] == kNoSlotInfo) xs[h] = __ldg(g.hm_slot + x[h]);
-            if (xs[h] >= 0) {
-              word[h] = ld_keep(g.hm_bits + (int64_t)sslot * g.hm_words + (xs[h] >> 5));
-              bitpos[h] = xs[h] & 31;
-              direct[h] = true;
-              continue;
-            }
-          }
-          const int sbm = it[h]->sbm[seg[h]];
-          if (sbm >= 0) {
-            word[h] = __ldg(g.bm_bits + (int64_t)sbm * g.bm_words + (x[h] >> 5));
-            bitpos[h] = x[h] & 31;
-            direct[h] = true;
-          } else if (sbm < -1) {
-            const uint32_t* d =
-                g.dir + (uint32_t)it[h]->slen[seg[h]] + (uint32_t)(x[h] >> (-2 - sbm));
-            word[h] = __ldg(d);
-            bitpos[h] = __ldg(d + 1);
-            bucket[h] = true;
-          }
-        }
+          // item starts among the next 64 tests: bit b of m0 / m1 = test r + b
+          // / r + 32 + b begins an item (items have tests, so starts differ)
+          const int32_t ds = srel - r;
+          const unsigned m0 = __reduce_or_sync(kFull, ds > 0 && ds < 32 ? 1u << ds : 0u);
+          const unsigned m1 =
+              __reduce_or_sync(kFull, ds >= 32 && ds < 64 ? 1u << (ds - 32) : 0u);
+          int j[2], seg[2];
+          int32_t x[2], xs[2];
+          bool act[2];
+          j[0] = min(j0 + __popc(m0 & upto), 31);
+          j[1] = min(j0 + __popc(m0) + __popc(m1 & upto), 31);
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          if (!act[h]) continue;
-          bool hit = direct[h]   ? ((word[h] >> bitpos[h]) & 1u) != 0
-                     : bucket[h] ? bucket_contains(it[h]->sl[seg[h]] + word[h],
-                                                   (int32_t)(bitpos[h] - word[h]), x[h])
-                                 : sorted_contains(it[h]->sl[seg[h]], it[h]->slen[seg[h]], x[h]);
-          if (hit) {
-            if (seg[h] == 0) {
-              ++acc_k;
-              acc_q += need_q ? 2 : 0;
-            } else {
-              acc_q += (it[h]->mode >> 8) - 1;
+          for (int h = 0; h < 2; ++h) {
+            const int32_t rr = r + 32 * h + lane;
+            const int32_t bj = __shfl_sync(kFull, sb, j[h]);
+            int32_t o = rr - __shfl_sync(kFull, srel, j[h]);
+            act[h] = rr < len;
+            seg[h] = 0;
+            x[h] = 0;
+            xs[h] = -1;
+            if (act[h]) {
+              if (rr >= bj) {
+                seg[h] = 1;
+                o = rr - bj;
+              }
+              const int32_t* it = my->it[seg[h]][j[h]] + o;
+              x[h] = __ldg(it);
+              if (my->sslot[seg[h]][j[h]] >= 0) {
+                const int16_t* hs = slots_beside(g, it, T, T_hm);
+                xs[h] = hs != nullptr ? (int32_t)__ldg(hs) : __ldg(g.hm_slot + x[h]);
+              }
             }
           }
+          Probe p[2];
+#pragma unroll
+          for (int h = 0; h < 2; ++h)
+            if (act[h])
+              p[h] = probe_begin<true>(g, my->sslot[seg[h]][j[h]], my->sbm[seg[h]][j[h]],
+                                       my->sl[seg[h]][j[h]], my->slen[seg[h]][j[h]], x[h], xs[h]);
+          unsigned hit[2];
+#pragma unroll
+          for (int h = 0; h < 2; ++h)
+            hit[h] = __ballot_sync(
+                kFull,
+                act[h] && probe_end(p[h], my->sl[seg[h]][j[h]], my->slen[seg[h]][j[h]], x[h]));
+#pragma unroll
+          for (int h = 0; h < 2; ++h) {
+            const int32_t rh = r + 32 * h;
+            const unsigned below_b = bits_below(sb - rh);
+            acc_a += __popc(hit[h] & below_b & ~bits_below(srel - rh));
+            acc_b += __popc(hit[h] & bits_below(se - rh) & ~below_b);
+          }
+          r += 64;
         }
       }
+      // the lanes' counts to their edges: one addition when the pack lies in
+      // one edge
+      long long dq = 0;
+      if (lane < live)
+        dq = (need_q ? 2 * (long long)acc_a : 0) + (long long)my->bsign[lane] * (long long)acc_b;
+      const int64_t e_last = __shfl_sync(kFull, e, live - 1);
+      if (e_last == e0) {
+        acc_a = warp_sum<unsigned long long>(acc_a);
+        dq = warp_sum<long long>(dq);
+        if (lane != 0) acc_a = 0, dq = 0;
+      }
+      if (acc_a) atomicAdd(k_out + e, acc_a);
+      if (dq) atomicAdd(q + e, (unsigned long long)dq);
     }
-  }
-  const unsigned long long sk = warp_sum<unsigned long long>(acc_k);
-  const long long sq = warp_sum<long long>(acc_q);
-  if (lane == 0 && cur >= 0) {
-    if (sk) atomicAdd(k_out + cur_e, sk);
-    if (sq) atomicAdd(q + cur_e, (unsigned long long)sq);
   }
 }
 

@@ -103,8 +103,15 @@ __device__ __forceinline__ uint32_t tfilter_hash(int32_t x) {
 #define GS_QUAD_GRAB_TESTS 16384
 #endif
 constexpr int64_t kQuadGrabTests = GS_QUAD_GRAB_TESTS;
-// Resident CTAs per SM of k_dense_pairs (at most 40 registers).
-constexpr int kDenseBlocksPerSm = 6;
+// Threads of a k_dense_pairs CTA and resident CTAs per SM.
+#ifndef GS_DENSE_THREADS
+#define GS_DENSE_THREADS 256
+#endif
+#ifndef GS_DENSE_BLOCKS
+#define GS_DENSE_BLOCKS 6
+#endif
+constexpr int kDenseThreads = GS_DENSE_THREADS;
+constexpr int kDenseBlocksPerSm = GS_DENSE_BLOCKS;
 // T entries per k_dense_pairs work unit (a heavy dense edge is split into
 // several units so that small samples still fill the GPU).
 constexpr int64_t kDenseUnit = 4 * kThreads;
@@ -126,6 +133,11 @@ __device__ __forceinline__ T warp_sum(T v) {
   return v;
 }
 
+
+// Bits [0, x) of a word, x clamped to 0..32.
+__device__ __forceinline__ unsigned bits_below(int32_t x) {
+  return x <= 0 ? 0u : x >= 32 ? kFull : (1u << x) - 1u;
+}
 
 __device__ __forceinline__ int64_t deg_of(const int64_t* __restrict__ row_ptr, int32_t v,
                                           int64_t* base) {
@@ -385,19 +397,24 @@ __global__ void k_unit_fill(const int64_t* __restrict__ unit_off, int64_t ndense
       unit_idx[u] = (int32_t)idx;
 }
 
-// Pairs of hub-matrix members of T in the dense edges: member w (slot s)
-// contributes popcount(w's matrix row AND the edge's T mask) over the bits
-// below s, so every adjacent pair of members counts once (k += 1, q += 2).
-// Slots are in decreasing degree, so T's members crowd in the low slots and
-// the groups at or below a member's own are few.
-// Work units are kDenseUnit consecutive T entries of one dense edge
-// (unit_off: exclusive scan of the units per dense edge, unit_idx: the
-// dense edge of each unit); a CTA takes one unit at a time from a counter
-// and stages the edge's mask (at most 2 KB) in shared memory; each warp
-// takes 32 of the unit's entries at a time and walks the rows of the
-// members among them with lanes over 128-bit groups (coalesced 512-byte
-// reads of the L2-resident matrix).
-__global__ void __launch_bounds__(kThreads, kDenseBlocksPerSm)
+// Pairs of dense-slot members of T in the dense edges, and the pairs of T's
+// other members, per work unit of kDenseUnit T entries (unit_off: exclusive
+// scan of the units per dense edge, unit_idx: the dense edge of each unit); a
+// CTA takes one unit at a time from a counter.
+//   dense-slot pairs: the member of rank r in slot order (slot s) contributes
+//   popcount(its matrix row AND the edge's T mask) over the bits below s, so
+//   every adjacent pair of members counts once (k += 1, q += 2). Slots are in
+//   decreasing degree, so T's members crowd in the low slots and the mask's
+//   non-zero 128-bit groups at or below a member's own are few. A unit takes
+//   the members of its kDenseUnit ranks, listed in slot order in shared
+//   memory; eight lanes walk one member's groups (128 coalesced bytes of the
+//   L2-resident matrix at a time), so a warp has four members of nearly equal
+//   length in flight, eight with the second set.
+//   other members (w without a dense slot among the unit's T entries): w's
+//   matrix neighbours (a bit of the mask, or, past the dense slots, a search
+//   of T when above w) and w's neighbours above w without a matrix slot (a
+//   search of T behind a hashed filter).
+__global__ void __launch_bounds__(kDenseThreads, kDenseBlocksPerSm)
     k_dense_pairs(const __grid_constant__ DevGraph g, const int64_t* __restrict__ toff,
                   const unsigned long long* __restrict__ t, const int32_t* __restrict__ T,
                   const int16_t* __restrict__ T_hm, const uint32_t* __restrict__ tmask,
@@ -407,200 +424,232 @@ __global__ void __launch_bounds__(kThreads, kDenseBlocksPerSm)
                   unsigned long long* __restrict__ counter,
                   unsigned long long* __restrict__ tests,
                   unsigned long long* __restrict__ rest_tests) {
-  // the edge's T mask, whole (fmask) and compacted to its non-zero 128-bit
-  // groups: smask[c] is group sgrp[c]; spos[g] = number of non-zero groups
-  // below g
-  __shared__ uint4 fmask[kHubMatrixMaxGroups];
+  constexpr int kWarps = kDenseThreads / 32;
+  // the edge's T mask compacted to its non-zero 128-bit groups: smask[c] is
+  // group sgrp[c], with sbase[c] members in the groups before it
   __shared__ uint4 smask[kHubMatrixMaxGroups];
   __shared__ uint16_t sgrp[kHubMatrixMaxGroups];
-  __shared__ uint16_t spos[kHubMatrixMaxGroups + 1];
-  __shared__ int wcnt[kThreads / 32], wlen[kThreads / 32];
-  // members without a dense slot among kThreads T entries: vertex, list
-  // offsets and lengths, first position in the concatenation of their lists
-  __shared__ int64_t ra[kThreads], rb[kThreads];
-  __shared__ int32_t rw[kThreads], rna[kThreads], rst[kThreads];
+  __shared__ uint16_t sbase[kHubMatrixMaxGroups];
+  __shared__ int wcnt[kWarps], wlen[kWarps];
+  // the unit's dense-slot members in slot order: slot and compact group
+  __shared__ uint16_t mslot[kDenseUnit];
+  __shared__ uint8_t mgrp[kDenseUnit];
+  // members without a dense slot among a warp's 32 T entries: vertex, list
+  // offsets, matrix-neighbour count, start in the concatenation of the lists
+  __shared__ int64_t ra[kDenseThreads], rb[kDenseThreads];
+  __shared__ int32_t rw[kDenseThreads], rna[kDenseThreads], rst[kDenseThreads];
   // hashed filter of T's members without a matrix slot (what the
   // non-matrix lists search for): a clear bit means "not in T"
   __shared__ uint32_t tfilt[kTFilterWords];
-  __shared__ unsigned long long part[kThreads / 32][3];
+  __shared__ unsigned long long part[kWarps][3];
   __shared__ int64_t cur;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const int64_t dense_words = g.hm_dense_words;
   const int G = (int)(dense_words / 4);  // 128-bit groups of the dense slots
   const int D = (int)(dense_words * 32);
-  const uint32_t* fmask32 = reinterpret_cast<const uint32_t*>(fmask);
+  const unsigned below = (1u << lane) - 1u, upto = kFull >> (31 - lane);
+  const int64_t units = __ldg(unit_off + ndense);
+  if (threadIdx.x == 0) cur = (int64_t)atomicAdd(counter, 1ull);
+  __syncthreads();
   for (;;) {
-    if (threadIdx.x == 0) cur = (int64_t)atomicAdd(counter, 1ull);
-    __syncthreads();
     const int64_t unit = cur;
-    if (unit >= __ldg(unit_off + ndense)) break;
+    if (unit >= units) break;
+    // the next unit's number, stored at the end of this one
+    unsigned long long following = 0;
+    if (threadIdx.x == 0) following = atomicAdd(counter, 1ull);
     const int64_t idx = __ldg(unit_idx + unit);
     const int64_t e = dense_e[idx];
     const uint4* m = reinterpret_cast<const uint4*>(tmask + idx * dense_words);
-    int L = 0;  // non-zero groups so far (the same in every thread)
-    for (int i0 = 0; i0 < G; i0 += kThreads) {
+    const int64_t b = toff[e], te = (int64_t)t[e];
+    const int64_t r0 = (unit - __ldg(unit_off + idx)) * kDenseUnit;
+    const int32_t* Te = T + b;
+    const int16_t* Ts = T_hm + b;
+    int L = 0, M = 0;  // non-zero groups and members so far (the same in every thread)
+    for (int i0 = 0; i0 < G; i0 += kDenseThreads) {
       const int i = i0 + threadIdx.x;
       const uint4 mv = i < G ? m[i] : make_uint4(0u, 0u, 0u, 0u);
-      if (i < G) fmask[i] = mv;
-      const bool nz = (mv.x | mv.y | mv.z | mv.w) != 0u;
-      const unsigned bal = __ballot_sync(kFull, nz);
-      if (lane == 0) wcnt[wid] = __popc(bal);
-      __syncthreads();
-      int before = L, total = L;
-      for (int w = 0; w < kThreads / 32; ++w) {
-        before += w < wid ? wcnt[w] : 0;
-        total += wcnt[w];
+      const int pc = __popc(mv.x) + __popc(mv.y) + __popc(mv.z) + __popc(mv.w);
+      const unsigned bal = __ballot_sync(kFull, pc != 0);
+      int incl = pc;
+#pragma unroll
+      for (int k = 1; k < 32; k <<= 1) {
+        const int y = __shfl_up_sync(kFull, incl, k);
+        if (lane >= k) incl += y;
       }
-      const int at = before + __popc(bal & ((1u << lane) - 1u));
-      if (i < G) spos[i] = (uint16_t)at;
-      if (nz) {
+      if (lane == 31) {
+        wcnt[wid] = __popc(bal);
+        wlen[wid] = incl;
+      }
+      __syncthreads();
+      int at = L + __popc(bal & below), mb = M + incl - pc;
+#pragma unroll
+      for (int w = 0; w < kWarps; ++w) {
+        at += w < wid ? wcnt[w] : 0;
+        mb += w < wid ? wlen[w] : 0;
+        L += wcnt[w];
+        M += wlen[w];
+      }
+      if (pc) {
         smask[at] = mv;
         sgrp[at] = (uint16_t)i;
+        sbase[at] = (uint16_t)mb;
       }
-      L = total;
-      __syncthreads();  // wcnt is rewritten by the next round
+      __syncthreads();  // wcnt and wlen are rewritten by the next round
     }
-    if (threadIdx.x == 0) spos[G] = (uint16_t)L;
+    const bool others = (int64_t)M < te;
+    const bool filt = others && te <= kTFilterMaxT;
+    if (filt)
+      for (int i = threadIdx.x; i < kTFilterWords; i += kDenseThreads) tfilt[i] = 0u;
+    // members of rank [r0, r0 + kDenseUnit), a mask word per thread
+    const int nmem = (int)min((int64_t)kDenseUnit, max((int64_t)0, (int64_t)M - r0));
+    if (nmem > 0)
+      for (int i = threadIdx.x; i < 4 * L; i += kDenseThreads) {
+        const int c = i >> 2, w4 = i & 3;
+        const uint4 mv = smask[c];
+        uint32_t bits = w4 == 0 ? mv.x : w4 == 1 ? mv.y : w4 == 2 ? mv.z : mv.w;
+        int64_t rank = (int64_t)sbase[c] - r0 + (w4 > 0 ? __popc(mv.x) : 0) +
+                       (w4 > 1 ? __popc(mv.y) : 0) + (w4 > 2 ? __popc(mv.z) : 0);
+        const int s0 = sgrp[c] * 128 + w4 * 32;
+        for (; bits; bits &= bits - 1, ++rank)
+          if (rank >= 0 && rank < nmem) {
+            mslot[rank] = (uint16_t)(s0 + __ffs(bits) - 1);
+            mgrp[rank] = (uint8_t)c;
+          }
+      }
     __syncthreads();
-    const int64_t b = toff[e];
-    const int64_t r0 = (unit - __ldg(unit_off + idx)) * kDenseUnit;
-    const int64_t len = min((int64_t)t[e], r0 + kDenseUnit);
-    unsigned long long acc = 0, groups = 0;
-    for (int64_t c0 = r0 + (int64_t)wid * 32; c0 < len; c0 += kThreads) {
-      const int xs = c0 + lane < len ? (int)__ldg(T_hm + b + c0 + lane) : -1;
-      unsigned members = __ballot_sync(kFull, xs >= 0 && xs < D);
-      while (members) {
-        const int src = __ffs(members) - 1;
-        members &= members - 1;
-        const int sl = __shfl_sync(kFull, xs, src);
-        const int g0 = sl >> 7, b0 = sl & 127;
-        const uint4* row = reinterpret_cast<const uint4*>(g.hm_bits + (int64_t)sl * g.hm_words);
-        const int p0 = spos[g0];  // w's own group is non-zero (w is in T)
-        groups += p0 + 1;
-        for (int c = lane; c <= p0; c += 32) {
-          const int gg = sgrp[c];
-          const uint4 rw = ld_keep4(row + gg);
-          const uint4 mk = smask[c];
-          uint32_t wd[4] = {rw.x & mk.x, rw.y & mk.y, rw.z & mk.z, rw.w & mk.w};
-          if (gg == g0) {  // only the bits below w's own
+    if (filt)
+      for (int64_t i = threadIdx.x; i < te; i += kDenseThreads)
+        if (__ldg(Ts + i) < 0) {
+          const uint32_t h = tfilter_hash(__ldg(Te + i));
+          atomicOr(tfilt + (h >> 5), 1u << (h & 31u));
+        }
+    // dense-slot pairs: eight lanes per member, eight members per warp
+    unsigned acc = 0, groups = 0;
+    const int sub = lane >> 3, l8 = lane & 7;
+    for (int m0 = wid * 8; m0 < nmem; m0 += kWarps * 8) {
+      int p0[2], b0[2];
+      const uint4* row[2];
 #pragma unroll
-            for (int q4 = 0; q4 < 4; ++q4) {
-              const int lo_bit = 32 * q4;
-              if (b0 <= lo_bit) wd[q4] = 0u;
-              else if (b0 < lo_bit + 32) wd[q4] &= (1u << (b0 - lo_bit)) - 1u;
-            }
+      for (int h = 0; h < 2; ++h) {
+        const int r = m0 + 2 * sub + h;
+        const int s = r < nmem ? (int)mslot[r] : 0;
+        p0[h] = r < nmem ? (int)mgrp[r] : -1;
+        b0[h] = s & 127;
+        row[h] = reinterpret_cast<const uint4*>(g.hm_bits + (int64_t)s * g.hm_words);
+        groups += p0[h] + 1;  // the same in the eight lanes
+      }
+      const int last = max(p0[0], p0[1]);
+      for (int c = l8; c <= last; c += 8) {
+        const int gg = sgrp[c];
+        const uint4 mk = smask[c];
+        uint4 rv[2];
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+          rv[h] = c <= p0[h] ? ld_keep4(row[h] + gg) : make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          uint32_t wd[4] = {rv[h].x & mk.x, rv[h].y & mk.y, rv[h].z & mk.z, rv[h].w & mk.w};
+          if (c == p0[h]) {  // the member's own group: only the bits below its own
+#pragma unroll
+            for (int q4 = 0; q4 < 4; ++q4) wd[q4] &= bits_below(b0[h] - 32 * q4);
           }
           acc += __popc(wd[0]) + __popc(wd[1]) + __popc(wd[2]) + __popc(wd[3]);
         }
       }
     }
+    groups = l8 == 0 ? groups : 0u;
     // members without a dense slot: w's matrix neighbours x (a bit of the
     // mask below D; past D, x = hm_vertex[s] counts when above w and in T)
     // and w's neighbours above w without a matrix slot (counted when in T).
-    // The block walks the concatenation of these lists, 32 positions per
-    // warp at a time.
-    unsigned long long rhits = 0, rtested = 0;
-    const int64_t te = (int64_t)t[e];
-    const int32_t* Te = T + b;
-    const bool filt = te <= kTFilterMaxT;
-    if (filt) {
-      for (int i = threadIdx.x; i < kTFilterWords; i += kThreads) tfilt[i] = 0u;
-      __syncthreads();
-      for (int64_t i = threadIdx.x; i < te; i += kThreads)
-        if (__ldg(T_hm + b + i) < 0) {
-          const uint32_t h = tfilter_hash(__ldg(Te + i));
-          atomicOr(tfilt + (h >> 5), 1u << (h & 31u));
-        }
-      __syncthreads();
-    }
-    for (int64_t c0 = r0; c0 < len; c0 += kThreads) {
-      const int64_t j = c0 + threadIdx.x;
-      int32_t w = -1, na = 0, nb = 0;
-      int64_t a0 = 0, b0 = 0;
-      if (j < len) {
-        const int xs = __ldg(T_hm + b + j);
-        if (!(xs >= 0 && xs < D)) {
-          w = __ldg(Te + j);
-          a0 = __ldg(g.mn_ptr + w);
-          na = (int32_t)(__ldg(g.mn_ptr + w + 1) - a0);
-          b0 = __ldg(g.nm_ptr + w);
-          nb = (int32_t)(__ldg(g.nm_ptr + w + 1) - b0);
-        }
-      }
-      const int32_t mine = na + nb;
-      const unsigned nz = __ballot_sync(kFull, mine > 0);
-      int32_t incl = mine;
-#pragma unroll
-      for (int k = 1; k < 32; k <<= 1) {
-        const int32_t y = __shfl_up_sync(kFull, incl, k);
-        if (lane >= k) incl += y;
-      }
-      if (lane == 31) {
-        wcnt[wid] = __popc(nz);
-        wlen[wid] = incl;
-      }
-      __syncthreads();
-      int32_t bn = 0, bl = 0, cnt = 0, total = 0;
-      for (int k = 0; k < kThreads / 32; ++k) {
-        if (k < wid) {
-          bn += wcnt[k];
-          bl += wlen[k];
-        }
-        cnt += wcnt[k];
-        total += wlen[k];
-      }
-      if (mine > 0) {
-        const int at = bn + __popc(nz & ((1u << lane) - 1u));
-        rw[at] = w;
-        ra[at] = a0;
-        rna[at] = na;
-        rb[at] = b0;
-        rst[at] = bl + incl - mine;
-      }
-      __syncthreads();
-      for (int32_t q0 = wid * 32; q0 < total; q0 += kThreads) {
-        int k0 = 0;  // last entry starting at or before q0
-        for (int step = kThreads / 2; step > 0; step >>= 1)
-          if (k0 + step < cnt && rst[k0 + step] <= q0) k0 += step;
-        const int32_t qq = q0 + lane;
-        int k = k0;  // last entry starting at or before qq (within 32)
-#pragma unroll
-        for (int step = 16; step > 0; step >>= 1)
-          if (k + step < cnt && rst[k + step] <= qq) k += step;
-        if (qq < total) {
-          const int32_t o = qq - rst[k];
-          bool hit;
-          if (o < rna[k]) {
-            const int sx = __ldg(g.mn_slot + ra[k] + o);
-            if (sx < D) {
-              hit = ((fmask32[sx >> 5] >> (sx & 31)) & 1u) != 0;
-            } else {
-              const int32_t x = __ldg(g.hm_vertex + sx);
-              hit = x > rw[k] && sorted_contains(Te, te, x);
-            }
-          } else {
-            const int32_t x = __ldg(g.nm_col + rb[k] + (o - rna[k]));
-            const uint32_t h = tfilter_hash(x);
-            hit = (!filt || ((tfilt[h >> 5] >> (h & 31u)) & 1u) != 0) && sorted_contains(Te, te, x);
+    // A warp walks the concatenation of these lists for 32 T entries.
+    unsigned long long rtested = 0;
+    if (others) {
+      __syncthreads();  // the filter is complete
+      const uint32_t* mask32 = tmask + idx * dense_words;
+      const int64_t len = min(te, r0 + kDenseUnit);
+      int64_t* wa = ra + wid * 32;
+      int64_t* wb = rb + wid * 32;
+      int32_t* wv = rw + wid * 32;
+      int32_t* wna = rna + wid * 32;
+      int32_t* wst = rst + wid * 32;
+      for (int64_t c0 = r0 + (int64_t)wid * 32; c0 < len; c0 += kDenseThreads) {
+        int32_t w = -1, na = 0, nb = 0;
+        int64_t a0 = 0, n0 = 0;
+        const int64_t j = c0 + lane;
+        if (j < len) {
+          const int xs = __ldg(Ts + j);
+          if (!(xs >= 0 && xs < D)) {
+            w = __ldg(Te + j);
+            a0 = __ldg(g.mn_ptr + w);
+            na = (int32_t)(__ldg(g.mn_ptr + w + 1) - a0);
+            n0 = __ldg(g.nm_ptr + w);
+            nb = (int32_t)(__ldg(g.nm_ptr + w + 1) - n0);
           }
-          rhits += hit ? 1 : 0;
-          ++rtested;
         }
+        const unsigned nz = __ballot_sync(kFull, na + nb > 0);
+        if (nz == 0) continue;
+        // start of the list in the concatenation; lane i then keeps the start
+        // of the i-th list (the total past the lists)
+        int32_t start = na + nb;
+#pragma unroll
+        for (int k = 1; k < 32; k <<= 1) {
+          const int32_t y = __shfl_up_sync(kFull, start, k);
+          if (lane >= k) start += y;
+        }
+        const int32_t total = __shfl_sync(kFull, start, 31);
+        __syncwarp();  // the previous entries are no longer read
+        if (na + nb > 0) {
+          const int at = __popc(nz & below);
+          wa[at] = a0;
+          wb[at] = n0;
+          wv[at] = w;
+          wna[at] = na;
+          wst[at] = start - (na + nb);
+        }
+        __syncwarp();
+        const int cnt = __popc(nz);
+        start = lane < cnt ? wst[lane] : total;
+        for (int32_t p = 0; p < total; p += 32) {
+          const int j0 = __popc(__ballot_sync(kFull, start <= p)) - 1;
+          const int32_t ds = start - p;
+          const unsigned marks = __reduce_or_sync(kFull, ds > 0 && ds < 32 ? 1u << ds : 0u);
+          const int k = min(j0 + __popc(marks & upto), cnt - 1);
+          const int32_t o = p + lane - __shfl_sync(kFull, start, k);
+          if (p + lane < total) {
+            bool hit;
+            if (o < wna[k]) {
+              const int sx = __ldg(g.mn_slot + wa[k] + o);
+              if (sx < D) {
+                hit = ((__ldg(mask32 + (sx >> 5)) >> (sx & 31)) & 1u) != 0;
+              } else {
+                const int32_t x = __ldg(g.hm_vertex + sx);
+                hit = x > wv[k] && sorted_contains(Te, te, x);
+              }
+            } else {
+              const int32_t x = __ldg(g.nm_col + wb[k] + (o - wna[k]));
+              const uint32_t h = tfilter_hash(x);
+              hit = (!filt || ((tfilt[h >> 5] >> (h & 31u)) & 1u) != 0) &&
+                    sorted_contains(Te, te, x);
+            }
+            acc += hit ? 1u : 0u;
+          }
+        }
+        rtested += lane == 0 ? total : 0;
       }
-      __syncthreads();  // rw, ra, rb, rna, rst, wcnt and wlen are reused
     }
-    acc += rhits;
-    acc = warp_sum<unsigned long long>(acc);
+    unsigned long long acc64 = warp_sum<unsigned long long>(acc);
     rtested = warp_sum<unsigned long long>(rtested);
+    const unsigned long long gsum = warp_sum<unsigned long long>(groups);
     if (lane == 0) {
-      part[wid][0] = acc;
-      part[wid][1] = groups;  // the same on every lane
+      part[wid][0] = acc64;
+      part[wid][1] = gsum;
       part[wid][2] = rtested;
     }
+    if (threadIdx.x == 0) cur = (int64_t)following;
     __syncthreads();
     if (threadIdx.x == 0) {
       unsigned long long sk = 0, sg = 0, sr = 0;
-      for (int w = 0; w < kThreads / 32; ++w) {
+      for (int w = 0; w < kWarps; ++w) {
         sk += part[w][0];
         sg += part[w][1];
         sr += part[w][2];
@@ -612,7 +661,8 @@ __global__ void __launch_bounds__(kThreads, kDenseBlocksPerSm)
       if (sg) atomicAdd(tests, sg);
       if (sr) atomicAdd(rest_tests, sr);
     }
-    __syncthreads();  // the masks, part and cur are reused for the next unit
+    // the masks, lists and part are reused for the next unit, whose first
+    // writes to them follow a barrier or are this thread's own
   }
 }
 
@@ -1045,11 +1095,6 @@ __device__ __forceinline__ const int16_t* slots_beside(const DevGraph& g, const 
   if (T_hm == nullptr) return nullptr;
   const size_t pc = (size_t)(it - g.col);
   return pc < (size_t)g.nnz ? g.col_hm + pc : T_hm + (it - T);
-}
-
-// Bits [0, x) of a word, x clamped to 0..32.
-__device__ __forceinline__ unsigned bits_below(int32_t x) {
-  return x <= 0 ? 0u : x >= 32 ? kFull : (1u << x) - 1u;
 }
 
 // The 4-node membership tests. A pack is up to 32 items with tests from
@@ -1649,7 +1694,7 @@ int64_t launch_tmask(const DevGraph& g, CountBufs& b, cudaStream_t stream) {
 // No host sync.
 int64_t launch_dense(const DevGraph& g, bool need_q, CountBufs& b, cudaStream_t stream) {
   if (b.ndense <= 0 || g.col_hm == nullptr) return 0;
-  k_dense_pairs<<<sm_count() * kDenseBlocksPerSm, kThreads, 0, stream>>>(
+  k_dense_pairs<<<sm_count() * kDenseBlocksPerSm, kDenseThreads, 0, stream>>>(
       g, b.toff, b.t, b.T, b.T_hm, b.tmask, b.dense_e, b.unit_off, b.unit_idx, b.ndense,
       need_q ? 1 : 0, b.k2, b.q, b.stats + 7, b.stats + 4, b.stats + 9);
   return 1;

@@ -288,27 +288,56 @@ __global__ void k_compact_T(DevGraph g, const int2* __restrict__ uv, const int64
     int2 pr = uv[e];
     int64_t bu;
     int64_t du = deg_of(g.row_ptr, pr.x, &bu);
-    int64_t words = (du + 31) >> 5, w0 = off[e] >> 5, pos = toff[e];
+    const int64_t words = (du + 31) >> 5, w0 = off[e] >> 5, t0 = toff[e];
+    int64_t pos = t0;
     long long dsum = 0;
     int thm = 0;
-    for (int64_t w = 0; w < words; ++w) {
-      uint32_t word = __ldg(tbits + w0 + w);
-      if (lane == 0) tpre[w0 + w] = (int32_t)(pos - toff[e]);
-      bool hm_member = false;
-      if ((word >> lane) & 1u) {
-        int32_t x = __ldg(g.col + bu + w * 32 + lane);
-        const int64_t at = pos + __popc(word & ((1u << lane) - 1u));
-        T[at] = x;
-        if (T_hm != nullptr) {
-          const int16_t xs = __ldg(g.col_hm + bu + w * 32 + lane);
-          T_hm[at] = xs;
-          hm_member = xs >= 0 && xs < g.hm_dense_words * 32;
-        }
-        dsum += __ldg(g.row_ptr + x + 1) - __ldg(g.row_ptr + x);
+    // 32 words of T bits at a time, one per lane; then the words that have
+    // members, four at a time so that their loads are in flight together
+    for (int64_t wb = 0; wb < words; wb += 32) {
+      const uint32_t word = wb + lane < words ? __ldg(tbits + w0 + wb + lane) : 0u;
+      int before = __popc(word);
+#pragma unroll
+      for (int d = 1; d < 32; d <<= 1) {
+        const int y = __shfl_up_sync(kFull, before, d);
+        if (lane >= d) before += y;
       }
-      thm += __popc(__ballot_sync(kFull, hm_member));
-      pos += __popc(word);
+      const int all = __shfl_sync(kFull, before, 31);
+      before -= __popc(word);
+      if (wb + lane < words) tpre[w0 + wb + lane] = (int32_t)(pos - t0) + before;
+      const int64_t c0 = bu + wb * 32 + lane;
+      for (unsigned nz = __ballot_sync(kFull, word != 0u); nz;) {
+        int32_t x[4];
+        int at[4];
+        int16_t xs[4];
+#pragma unroll
+        for (int h = 0; h < 4; ++h) {
+          const int k = nz ? __ffs(nz) - 1 : 0;
+          const uint32_t wd = nz ? __shfl_sync(kFull, word, k) : 0u;
+          const int bk = __shfl_sync(kFull, before, k);
+          nz &= nz - 1;
+          x[h] = -1;
+          xs[h] = -1;
+          at[h] = bk + __popc(wd & ((1u << lane) - 1u));
+          if ((wd >> lane) & 1u) {
+            x[h] = __ldg(g.col + c0 + k * 32);
+            if (T_hm != nullptr) xs[h] = __ldg(g.col_hm + c0 + k * 32);
+          }
+        }
+#pragma unroll
+        for (int h = 0; h < 4; ++h) {
+          if (x[h] < 0) continue;
+          T[pos + at[h]] = x[h];
+          if (T_hm != nullptr) {
+            T_hm[pos + at[h]] = xs[h];
+            thm += xs[h] >= 0 && xs[h] < g.hm_dense_words * 32;
+          }
+          dsum += __ldg(g.row_ptr + x[h] + 1) - __ldg(g.row_ptr + x[h]);
+        }
+      }
+      pos += all;
     }
+    thm = __reduce_add_sync(kFull, thm);
     for (int o = 16; o > 0; o >>= 1) dsum += __shfl_xor_sync(kFull, dsum, o);
     bool dense_mode = false;
     if (T_hm != nullptr && thm >= kDenseMin) {
@@ -318,7 +347,7 @@ __global__ void k_compact_T(DevGraph g, const int2* __restrict__ uv, const int64
       // member and lie at or below its own (what k_dense_pairs reads), plus
       // the adjacency of the other members
       __syncwarp();  // this warp's T entries are visible to all its lanes
-      const int64_t t0 = toff[e], te = pos - t0;
+      const int64_t te = pos - t0;
       const int D = (int)(g.hm_dense_words * 32);
       uint32_t* gb = gbits[threadIdx.x >> 5];
       for (int w = lane; w < kGroupWords; w += 32) gb[w] = 0u;
@@ -328,16 +357,24 @@ __global__ void k_compact_T(DevGraph g, const int2* __restrict__ uv, const int64
         if (xs >= 0 && xs < D) atomicOr(gb + (xs >> 12), 1u << ((xs >> 7) & 31));
       }
       __syncwarp();
+      int gpre = lane < kGroupWords ? __popc(gb[lane]) : 0;  // groups in words <= lane
+#pragma unroll
+      for (int d = 1; d < kGroupWords; d <<= 1) {
+        const int y = __shfl_up_sync(kFull, gpre, d);
+        if (lane >= d) gpre += y;
+      }
       long long sparse = 0, dense = 0, groups = 0;
-      for (int64_t j = lane; j < te; j += 32) {
+      for (int64_t j0 = 0; j0 < te; j0 += 32) {
+        const int64_t j = j0 + lane;
+        const int xs = j < te ? (int)T_hm[t0 + j] : -1;
+        const int gw = __shfl_sync(kFull, gpre, xs >= 4096 ? (xs >> 12) - 1 : 0);
+        if (j >= te) continue;
         const int32_t x = T[t0 + j];
-        const int xs = T_hm[t0 + j];
         const int64_t dx = __ldg(g.row_ptr + x + 1) - __ldg(g.row_ptr + x);
         sparse += min(dx / 2, te - j - 1);  // about half of N(x) lies above x
         if (xs >= 0 && xs < D) {
           const int g0 = xs >> 7;
-          groups += __popc(gb[g0 >> 5] & (0xffffffffu >> (31 - (g0 & 31))));
-          for (int w = 0; w < (g0 >> 5); ++w) groups += __popc(gb[w]);
+          groups += (xs >= 4096 ? gw : 0) + __popc(gb[g0 >> 5] & (kFull >> (31 - (g0 & 31))));
         } else {  // k_dense_pairs walks its matrix and non-matrix-above lists
           dense += g.mn_ptr != nullptr ? (__ldg(g.mn_ptr + x + 1) - __ldg(g.mn_ptr + x)) +
                                              (__ldg(g.nm_ptr + x + 1) - __ldg(g.nm_ptr + x))

@@ -742,10 +742,17 @@ struct EdgeCtx {
   const uint32_t* tmask;  // this edge's T mask (dense edges), else NULL
 };
 
-// Rows of the endpoints in a small graph's co-degree block, shifted so that
-// the entry of vertex w is row[w] (NULL without a block).
-struct BlockRows {
-  const uint8_t *u, *v;
+// What the cost pass keeps of an edge: the endpoints' lists, and for each end
+// o of its co-degree queries c(w, o) (o = u for w in T, o = v for w in S_u)
+// the row of a small graph's co-degree block shifted so that w's entry is
+// row[w] (NULL without a block), the table slot and the mid x big column.
+struct CostEdge {
+  int64_t e, first, end;  // edge, its positions [first, end)
+  int64_t bu, te;
+  int32_t v, du, dv;
+  bool dense;
+  const uint8_t *row_u, *row_v;
+  int32_t slot_u, slot_v, col_u, col_v;
 };
 
 __device__ __forceinline__ const uint8_t* block_row(const DevGraph& g, int32_t o) {
@@ -771,16 +778,14 @@ __device__ __forceinline__ void load_edge(const DevGraph& g, const int2* __restr
   c.toff = toff[e];
 }
 
-// c(a, b) + 1 from the co-degree table when both are table hubs or from the
+// c(w, o) + 1 from the co-degree table when both are table hubs or from the
 // mid x big table when one is a mid vertex and the other a big hub; 0 when
-// neither can answer (the +1 marks a present entry).
-// sa is a's table slot (tb_slot[a], -1 without a table).
-__device__ __forceinline__ uint32_t table_codeg_s(const DevGraph& g, int32_t a, int32_t sa,
-                                                  int32_t b) {
-  if (g.tb_slot == nullptr) return 0;
-  const int32_t sb = __ldg(g.tb_slot + b);
-  if (sa >= 0 && sb >= 0) {
-    const int32_t lo = min(sa, sb), hi = max(sa, sb);
+// neither can answer (the +1 marks a present entry). sw, so: table slots (-1
+// none, <= -2 a mid row); co: o's mid x big column (-1 none).
+__device__ __forceinline__ uint32_t table_codeg(const DevGraph& g, int32_t w, int32_t sw,
+                                                int32_t so, int32_t co) {
+  if (sw >= 0 && so >= 0) {
+    const int32_t lo = min(sw, so), hi = max(sw, so);
     const uint16_t c = ld_once16(g.tb_codeg + tb_index(lo, hi, g.tb_count));
     if (c != 0xFFFFu) return (uint32_t)c + 1u;
     if (g.tb_giant != nullptr) {  // a pair of giants
@@ -789,11 +794,11 @@ __device__ __forceinline__ uint32_t table_codeg_s(const DevGraph& g, int32_t a, 
     }
     return 0;  // a true co-degree of 65,535 is left to the tests
   }
-  if (g.md_codeg != nullptr && (sa < -1 || sb < -1) && (sa >= 0 || sb >= 0)) {
+  if (g.md_codeg != nullptr && (sw < -1 || so < -1) && (sw >= 0 || so >= 0)) {
     // one mid vertex (slot -2 - row), one table vertex that may be big
-    const int32_t row = -2 - min(sa, sb);
-    const int32_t col = __ldg(g.bg_slot + (sa >= 0 ? a : b));
-    if (col >= 0) return (uint32_t)ld_once16(g.md_codeg + (int64_t)row * g.bg_count + col) + 1u;
+    const int32_t col = sw >= 0 ? __ldg(g.bg_slot + w) : co;
+    if (col >= 0)
+      return (uint32_t)ld_once16(g.md_codeg + (int64_t)(-2 - min(sw, so)) * g.bg_count + col) + 1u;
   }
   return 0;
 }
@@ -848,65 +853,61 @@ __device__ __forceinline__ void codeg_segment(const DevGraph& g, int32_t w, int6
 // the graph has it, so the table read does not wait for a gather.
 struct ItemCost {
   int32_t a, b;    // tests of segments A and B
-  int64_t qconst;  // constant q contribution
+  int32_t qconst;  // constant q contribution (a co-degree is below n < 2^31)
   bool tabled;     // a co-degree table answered segment B
 };
 
-__device__ __forceinline__ ItemCost item_cost(const DevGraph& g, const EdgeCtx& c,
-                                              const BlockRows& rows, int64_t i, uint32_t tword,
-                                              int32_t tbase, int lane, bool need_q) {
+// Most items are in S_u and answered by a table: for those only the element,
+// its table slot and the table entry are read; degrees are read by the rest.
+__device__ __forceinline__ ItemCost item_cost(const DevGraph& g, const CostEdge& c, int64_t i,
+                                              uint32_t tword, const int32_t* __restrict__ tpre,
+                                              int lane, bool need_q) {
   ItemCost r{0, 0, 0, false};
   if (i >= c.du) return r;
   const int64_t p = c.bu + i;
   const int32_t w = __ldg(g.col + p);
   if (w == c.v) return r;
   const bool in_t = (tword >> lane) & 1u;
-  const int64_t dw = __ldg(g.row_ptr + w + 1) - __ldg(g.row_ptr + w);
-  if (in_t) {
-    if (c.tmask != nullptr) {
-      // dense edge: segment A is k_dense_pairs' work (pairs of dense-slot
-      // members; the other members' matrix and non-matrix neighbours)
-    } else {
-      // |N(w) above w cap T above w|: the shorter side is iterated
-      const int64_t iw = tbase + __popc(tword & ((1u << lane) - 1u));
-      const int64_t tg = c.te - iw - 1;
-      const int64_t dup = __ldg(g.row_ptr + w + 1) - __ldg(g.up_ptr + w);
-      r.a = (int32_t)min(dup, tg);
-    }
-  }
   if (need_q) {
     // segment B: -(c(w, u) - 1) for w in T, c(w, v) - 1 for w in S_u
-    const int32_t o = in_t ? c.u : c.v;
-    const uint8_t* row = in_t ? rows.u : rows.v;
+    const uint8_t* row = in_t ? c.row_u : c.row_v;
     uint32_t tc = 0;
     if (row != nullptr) {
       const uint32_t b = __ldg(row + w);
       if (b < 255u) tc = b + 1u;
     }
-    if (tc == 0) {
-      const int32_t sw = g.col_tb != nullptr ? __ldg(g.col_tb + p)
-                         : g.tb_slot != nullptr ? __ldg(g.tb_slot + w) : -1;
-      tc = table_codeg_s(g, w, sw, o);
+    if (tc == 0 && g.tb_slot != nullptr) {
+      const int32_t sw = __ldg(g.col_tb != nullptr ? g.col_tb + p : g.tb_slot + w);
+      tc = table_codeg(g, w, sw, in_t ? c.slot_u : c.slot_v, in_t ? c.col_u : c.col_v);
     }
     r.tabled = tc != 0;
     if (tc != 0) {
-      r.qconst = in_t ? 1 - (int64_t)(tc - 1u) : (int64_t)(tc - 1u) - 1;
+      r.qconst = in_t ? 2 - (int32_t)tc : (int32_t)tc - 2;
     } else {
       r.qconst = in_t ? 1 : -1;
-      r.b = (int32_t)min(dw, in_t ? c.du : c.dv);
+      r.b = (int32_t)min(__ldg(g.row_ptr + w + 1) - __ldg(g.row_ptr + w),
+                         (int64_t)(in_t ? c.du : c.dv));
     }
+  }
+  if (in_t && !c.dense) {
+    // |N(w) above w cap T above w|: the shorter side is iterated (in a dense
+    // edge segment A is k_dense_pairs' work)
+    const int64_t tg = c.te - (__ldg(tpre) + __popc(tword & ((1u << lane) - 1u))) - 1;
+    if (tg > 0) r.a = (int32_t)min(__ldg(g.row_ptr + w + 1) - __ldg(g.up_ptr + w), tg);
   }
   return r;
 }
 
 
 // Chunk costs: membership tests per chunk and the number of tasks it needs.
-// Also adds the constant part of q. Same warp partition as k_tri.
+// Also adds the constant part of q. Bound by the latency of the table reads
+// (two bytes of a random sector per item); cost phase of the 1M-vertex
+// power-law graph exact: 131 -> 116 ms when the items a table answers stopped
+// reading their degrees and the sums went to 32-bit warp reductions.
 __global__ void __launch_bounds__(kThreads, kCostBlocksPerSm)
     k_chunk_cost(DevGraph g, const int2* __restrict__ uv, const int64_t* __restrict__ off, int64_t K,
-                 const unsigned long long* __restrict__ t, const int64_t* __restrict__ toff,
-                 const uint32_t* __restrict__ tbits, const int32_t* __restrict__ tpre,
-                 const int32_t* __restrict__ mask_idx, const uint32_t* __restrict__ tmask,
+                 const unsigned long long* __restrict__ t, const uint32_t* __restrict__ tbits,
+                 const int32_t* __restrict__ tpre, const int32_t* __restrict__ mask_idx,
                  int need_q, int64_t task_probes, int64_t* __restrict__ task_cnt,
                  uint32_t* __restrict__ cbits, unsigned long long* __restrict__ q,
                  unsigned long long* __restrict__ stats) {
@@ -914,11 +915,11 @@ __global__ void __launch_bounds__(kThreads, kCostBlocksPerSm)
   const int lane = threadIdx.x & 31;
   const int64_t P = __ldg(off + K);
   const int64_t groups = P >> 5;  // padded: P is a multiple of 32
-  int64_t e = 0;
-  EdgeCtx c;
+  CostEdge c;
   c.e = -1;
-  BlockRows rows{nullptr, nullptr};
-  int64_t next = -1;  // the chunk after this warp's previous run
+  c.first = c.end = 0;
+  c.row_u = c.row_v = nullptr;
+  c.slot_u = c.slot_v = c.col_u = c.col_v = -1;
   // runs of consecutive chunks from a counter (chunks differ in cost: table
   // answers, hub edges)
   const int grab =
@@ -929,29 +930,53 @@ __global__ void __launch_bounds__(kThreads, kCostBlocksPerSm)
     const int64_t g0 = (int64_t)__shfl_sync(kFull, got, 0);
     if (g0 >= groups) break;
     const int64_t g1 = min(groups, g0 + grab);
-    if (g0 != next) e = last_le(off, K, g0 * 32);
-    next = g1;
     // packs: consecutive chunks of the run with at most 32 live items in all,
     // so that k_quad sets up a warp's worth of items at a time; a pack's
     // tasks are counted at its first chunk
     int64_t head = g0, pcost = 0;
     int plive = 0;
     for (int64_t gi = g0; gi < g1; ++gi) {
-      while (e + 1 < K && __ldg(off + e + 1) <= gi * 32) ++e;
-      if (e != c.e) {
-        load_edge(g, uv, t, toff, mask_idx, tmask, e, c);
+      const int64_t p0 = gi * 32;
+      if (p0 < c.first || p0 >= c.end) {  // another edge: the next one, or a search
+        c.e = p0 == c.end && c.e >= 0 ? c.e + 1 : last_le(off, K, p0);
+        c.first = __ldg(off + c.e);
+        c.end = __ldg(off + c.e + 1);
+        const int2 pr = uv[c.e];
+        c.v = pr.y;
+        c.du = (int32_t)deg_of(g.row_ptr, pr.x, &c.bu);
+        c.dv = (int32_t)(__ldg(g.row_ptr + pr.y + 1) - __ldg(g.row_ptr + pr.y));
+        c.te = (int64_t)t[c.e];
+        c.dense = mask_idx != nullptr && mask_idx[c.e] >= 0;
         if (g.cg_row != nullptr) {
-          rows.u = block_row(g, c.u);
-          rows.v = block_row(g, c.v);
+          c.row_u = block_row(g, pr.x);
+          c.row_v = block_row(g, pr.y);
+        }
+        if (g.tb_slot != nullptr) {
+          c.slot_u = __ldg(g.tb_slot + pr.x);
+          c.slot_v = __ldg(g.tb_slot + pr.y);
+        }
+        if (g.bg_slot != nullptr) {
+          c.col_u = __ldg(g.bg_slot + pr.x);
+          c.col_v = __ldg(g.bg_slot + pr.y);
         }
       }
-      const ItemCost it = item_cost(g, c, rows, gi * 32 + lane - __ldg(off + e), __ldg(tbits + gi),
-                                    __ldg(tpre + gi), lane, need_q);
-      const unsigned live = __ballot_sync(kFull, it.a + it.b > 0);
+      const ItemCost it =
+          item_cost(g, c, p0 + lane - c.first, __ldg(tbits + gi), tpre + gi, lane, need_q);
+      const unsigned live = __ballot_sync(kFull, (it.a | it.b) != 0);
       const unsigned tabled = __ballot_sync(kFull, it.tabled);
       if (lane == 0) reinterpret_cast<uint2*>(cbits)[gi] = make_uint2(live, tabled);
-      const int64_t cost = live ? warp_sum<int64_t>((int64_t)it.a + it.b) : 0;
-      const int64_t qc = warp_sum<int64_t>(it.qconst);
+      // sums over the warp, in 32 bits while every term is far from them
+      constexpr int32_t kSmall = 1 << 24;
+      const bool wide = __any_sync(kFull, it.a > kSmall || it.b > kSmall || it.qconst > kSmall ||
+                                              it.qconst < -kSmall);
+      int64_t cost, qc;
+      if (wide) {
+        cost = warp_sum<int64_t>((int64_t)it.a + it.b);
+        qc = warp_sum<int64_t>(it.qconst);
+      } else {
+        cost = __reduce_add_sync(kFull, it.a + it.b);
+        qc = __reduce_add_sync(kFull, it.qconst);
+      }
       if (plive + __popc(live) > 32) {
         if (lane == 0) task_cnt[head] = (pcost + task_probes - 1) / task_probes;
         head = gi;
@@ -962,7 +987,7 @@ __global__ void __launch_bounds__(kThreads, kCostBlocksPerSm)
       plive += __popc(live);
       if (lane == 0) {
         if (gi != head) task_cnt[gi] = 0;
-        if (qc != 0) atomicAdd(q + e, (unsigned long long)qc);
+        if (qc != 0) atomicAdd(q + c.e, (unsigned long long)qc);
         tests += cost;
       }
     }
@@ -1743,8 +1768,8 @@ int64_t launch_cost(const DevGraph& g, bool need_k, bool need_q, const Tuning& t
   (void)need_k;  // every item's segment A feeds both k and q
   const int32_t* mi = g.col_hm != nullptr ? b.mask_idx : nullptr;
   k_chunk_cost<<<sm_count() * kCostBlocksPerSm, kThreads, 0, stream>>>(
-      g, b.uv, b.off, b.K, b.t, b.toff, b.tbits, b.tpre, mi, b.tmask, need_q, tu.task_probes,
-      b.task_off, b.cbits, b.q, b.stats);
+      g, b.uv, b.off, b.K, b.t, b.tbits, b.tpre, mi, need_q, tu.task_probes, b.task_off, b.cbits,
+      b.q, b.stats);
   exclusive_scan_i64(b.task_off, b.task_off, b.groups, b.tmp1, stream);
   return 4;
 }

@@ -29,11 +29,9 @@
 //           classifies its positions (T, S_u, S_v or none) with one
 //           membership test each, counts t and the chunk's probes, and
 //           turns them into tasks of kTaskProbes probes.
-//   probe   tasks are split evenly over all warps; lanes take consecutive
-//           probes of a task and find their item by a search over the
-//           warp's scanned probe counts (item descriptors in shared
-//           memory); a probe costs one or two membership tests (in N(u),
-//           in N(v)).
+//   probe   warps take runs of tasks from a counter; lanes take consecutive
+//           probes of a task (item descriptors in shared memory); a probe
+//           costs up to two membership tests (in N(v), in N(u)).
 //   final   one thread per edge writes the 15 statistics and keeps the
 //           column maxima (the extremal statistics of Sec. 7).
 // Weighted hits are accumulated exactly: weight d_w / c_w = q + f / 2^64
@@ -59,8 +57,12 @@ namespace {
 
 constexpr int kThreads = 256;
 constexpr unsigned kFull = 0xffffffffu;
-constexpr int kProbeBlocksPerSm = 4;
+#ifndef GS_PROBE_BLOCKS
+#define GS_PROBE_BLOCKS 5
+#endif
+constexpr int kProbeBlocksPerSm = GS_PROBE_BLOCKS;
 constexpr int64_t kTaskProbes = 512;
+constexpr int kRunTasks = 8;  // tasks a probe warp takes from the counter, at most
 constexpr int kCats = 4;   // x7, x9, x10, omega
 constexpr int kCols = 15;  // x3 .. x17
 constexpr int kNone = 0, kT = 1, kSu = 2, kSv = 3;
@@ -192,10 +194,13 @@ __global__ void __launch_bounds__(kThreads)
   if (lane == 0 && probes) atomicAdd(stats, probes);
 }
 
-struct ItemDesc {  // one lane's item, in shared memory for the probe loop
-  int64_t bw, dw, o;
-  uint64_t q, f;
-  int32_t w, cls;
+// The items of the chunk a warp works on (live positions only, in order),
+// field by field so that lanes that read different items hit different banks.
+struct WarpItems {
+  int64_t bw[32];  // start of N(w)
+  int32_t dw[32], o[32], w[32];
+  uint16_t who[32];  // position in the chunk
+  uint8_t cls[32];
 };
 
 // Adds a 64-bit integer part and a 128-bit fraction to an edge's
@@ -217,145 +222,240 @@ __device__ __forceinline__ u128 shfl_xor_u128(u128 v, int o) {
   return ((u128)hi << 64) | lo;
 }
 
-struct Hits {
-  unsigned long long I[kCats];
-  u128 F[kCats];
+// How "x in N(y)" is answered for an endpoint y, looked up once per chunk
+// instead of once per probe: a row of words (dense row or bitmap, bit
+// x - first), the matrix row (for an x with a matrix slot), a bucket
+// directory, or a halving search of the list.
+struct EndSet {
+  const uint32_t* words;
+  const uint32_t* mrow;
+  const uint32_t* dir;
+  const int32_t* list;
+  int32_t first, deg, shift;
 };
 
-__device__ __forceinline__ void flush_hits(Hits& h, unsigned long long* __restrict__ acc_e,
-                                           int lane) {
-#pragma unroll
-  for (int k = 0; k < kCats; ++k) {
-    unsigned long long I = h.I[k];
-    u128 F = h.F[k];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      I += __shfl_xor_sync(kFull, I, o);
-      F += shfl_xor_u128(F, o);
+// A bitmap row of at most this many words (32 KB) stays in the L1 cache, so
+// it answers every x and the matrix slots need not be read.
+constexpr int64_t kShortRowWords = 8192;
+
+__device__ __forceinline__ EndSet end_set(const DevGraph& g, int32_t y, int64_t by, int64_t dy) {
+  EndSet s{nullptr, nullptr, nullptr, g.col + by, 0, (int32_t)dy, 0};
+  if (g.dm_row != nullptr) {
+    const int64_t r = __ldg(g.dm_row + y);
+    if (r >= 0) {
+      s.words = g.dm_bits + r;
+      s.first = __ldg(g.dm_first + y);
+      return s;
     }
-    if (lane == 0 && (I || F)) acc_add(acc_e + 3 * k, I, F);
-    h.I[k] = 0;
-    h.F[k] = 0;
   }
+  const int32_t b = bitmap_slot(g, y);
+  if (b >= 0) s.words = g.bm_bits + (int64_t)b * g.bm_words;
+  if (b >= 0 && g.bm_words <= kShortRowWords) return s;
+  const int32_t h = table_slot(g, y);
+  if (h >= 0) s.mrow = g.hm_bits + (int64_t)h * g.hm_words;
+  if (b < 0 && g.dir_at != nullptr) {
+    const int64_t at = __ldg(g.dir_at + y);
+    if (at >= 0) {
+      s.dir = g.dir + at;
+      s.shift = g.id_bits - dir_log2(dy, g.id_bits);
+    }
+  }
+  return s;
 }
 
+// xs: x's matrix slot (-1 if none; not looked at without a matrix row).
+__device__ __forceinline__ bool set_has(const EndSet& s, int32_t x, int32_t xs) {
+  if (s.mrow != nullptr && xs >= 0) return (__ldg(s.mrow + (xs >> 5)) >> (xs & 31)) & 1u;
+  if (s.words != nullptr) {
+    const int32_t lx = x - s.first;
+    return (__ldg(s.words + (lx >> 5)) >> (lx & 31)) & 1u;
+  }
+  if (s.dir != nullptr) {
+    const uint32_t* d = s.dir + (uint32_t)(x >> s.shift);
+    const uint32_t lo = __ldg(d), hi = __ldg(d + 1);
+    return sorted_contains(s.list + lo, (int64_t)(hi - lo), x);
+  }
+  return sorted_contains(s.list, s.deg, x);
+}
+
+// Statistic (0: x7, 1: x9, 2: x10, 3: omega, -1: none) of a probe that read x
+// from N(w). v is tested first; u only where its answer matters.
+__device__ __forceinline__ int probe_cat(const EndSet& su, const EndSet& sv, int32_t u, int32_t v,
+                                         int cls, int32_t w, int32_t x, int32_t xs) {
+  const bool above = x > w;
+  if (cls == kT) return above && set_has(sv, x, xs) && set_has(su, x, xs) ? 0 : -1;
+  if (x == u || x == v) return -1;
+  const bool in_v = set_has(sv, x, xs);
+  if (!in_v && !(cls == kSu && above)) return -1;
+  const bool in_u = set_has(su, x, xs);
+  if (!in_v) return in_u ? 1 : -1;                  // S_u pair
+  if (in_u) return 3;                               // omega
+  return cls == kSu ? 2 : above ? 1 : -1;           // 4-cycle; S_v pair
+}
+
+// Bits [0, x) of a word, x clamped to 0..32.
+__device__ __forceinline__ unsigned bits_below(int32_t x) {
+  return x <= 0 ? 0u : x >= 32 ? kFull : (1u << x) - 1u;
+}
+
+// Probes. A chunk's probes (its items in order) are one index space cut into
+// tasks; warps take runs of tasks from a counter. From probe r on a warp walks
+// either a run of 32 or more probes of one item (its descriptor is the same in
+// every lane) or 32 probes of several items, found from a bit mask of the item
+// starts among them. Lane i owns item i: it counts the item's hits per
+// statistic (from the hit ballots, whose bits [start, end) are the item's
+// probes), and the item's weight d_w / c_w multiplies the counts once per
+// chunk. Issue bound before: five shuffles to find the item, two general
+// membership look-ups and 4 x 192-bit predicated additions per probe. 20,000
+// edges of the 100k-vertex power-law graph at p_e = 0.1 (2.1e9 probes): 29.2
+// -> 19.1 ms for the whole call (20.8 / 20.2 / 19.1 / 19.3 ms at 3 / 4 / 5 / 6
+// CTAs per SM).
 __global__ void __launch_bounds__(kThreads, kProbeBlocksPerSm)
     k_micro_probe(const __grid_constant__ DevGraph g, const int2* __restrict__ uv,
                   const int64_t* __restrict__ choff, const int64_t* __restrict__ chunk_e,
                   const uint32_t* __restrict__ tmask, const int64_t* __restrict__ task_off,
-                  int64_t C, double pe, uint64_t seed, unsigned long long* __restrict__ acc) {
-  __shared__ ItemDesc items[kThreads / 32][32];
+                  int64_t C, double pe, uint64_t seed, unsigned long long* __restrict__ acc,
+                  unsigned long long* __restrict__ counter) {
+  __shared__ WarpItems items[kThreads / 32];
   const int lane = threadIdx.x & 31;
-  ItemDesc* my = items[threadIdx.x >> 5];
-  const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  const unsigned upto = kFull >> (31 - lane);
+  WarpItems* my = items + (threadIdx.x >> 5);
   const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
-  const int64_t NT = __ldg(task_off + C);
-  const int64_t per = (NT + warps - 1) / warps;
-  const int64_t t0 = warp * per, t1 = min(NT, t0 + per);
-  if (t0 >= t1) return;
-  int64_t c = last_le64(task_off, C, t0);
-  int64_t cur = -1, cur_e = -1;
-  int64_t start = 0, ctotal = 0;
-  int32_t u = 0, v = 0;
-  int64_t bu = 0, du = 0, bv = 0, dv = 0;
-  Hits h;
-#pragma unroll
-  for (int k = 0; k < kCats; ++k) {
-    h.I[k] = 0;
-    h.F[k] = 0;
-  }
-  for (int64_t task = t0; task < t1; ++task) {
-    while (c + 1 < C && __ldg(task_off + c + 1) <= task) ++c;
-    if (c != cur) {
+  // at least eight runs per warp, at most kRunTasks tasks each
+  const int64_t share = __ldg(task_off + C) / (warps * 8);
+  const int grab = share < 1 ? 1 : share < kRunTasks ? (int)share : kRunTasks;
+  for (;;) {
+    unsigned long long got = 0;
+    if (lane == 0) got = atomicAdd(counter, (unsigned long long)grab);
+    int64_t task = (int64_t)__shfl_sync(kFull, got, 0);
+    int left = (int)min((int64_t)grab, __ldg(task_off + C) - task);
+    if (left <= 0) break;
+    int64_t c = last_le64(task_off, C, task);
+    while (left > 0) {
+      while (__ldg(task_off + c + 1) <= task) ++c;
+      int here = (int)min((int64_t)left, __ldg(task_off + c + 1) - task);
+      left -= here;
       const int64_t e = chunk_e[c];
-      if (cur >= 0 && e != cur_e) flush_hits(h, acc + cur_e * 3 * kCats, lane);
       const ChunkAt a = chunk_at(g, uv, choff, e, c);
-      u = a.u;
-      v = a.v;
-      bu = a.bu;
-      du = a.du;
-      bv = a.bv;
-      dv = a.dv;
-      const uint32_t inT = tmask[2 * c], live = tmask[2 * c + 1];
+      const EndSet su = end_set(g, a.u, a.bu, a.du), sv = end_set(g, a.v, a.bv, a.dv);
+      const bool slots = su.mrow != nullptr || sv.mrow != nullptr;
+      const uint32_t inT = tmask[2 * c], alive = tmask[2 * c + 1];
+      const int live = __popc(alive);
+      __syncwarp();  // the previous chunk's items are no longer read
+      if ((alive >> lane) & 1u) my->who[__popc(alive & ((1u << lane) - 1u))] = (uint16_t)lane;
+      __syncwarp();
       int64_t mine = 0;
-      __syncwarp();
-      ItemDesc d;
-      d.cls = kNone;
-      d.w = 0;
-      d.bw = 0;
-      d.dw = 1;
-      d.o = 0;
-      d.q = 0;
-      d.f = 0;
-      const int64_t i = a.first + lane;
-      if ((live >> lane) & 1u) {
-        d.w = __ldg(g.col + a.bo + i);
-        d.cls = a.vside ? kSv : (((inT >> lane) & 1u) ? kT : kSu);
-        d.bw = __ldg(g.row_ptr + d.w);
-        d.dw = __ldg(g.row_ptr + d.w + 1) - d.bw;
-        mine = probes_of(d.dw, pe);
-        const uint64_t key = ((uint64_t)(uint32_t)min(u, v) << 32) | (uint32_t)max(u, v);
-        const uint64_t hh = splitmix(splitmix(seed ^ splitmix(key)) ^ (uint64_t)(uint32_t)d.w);
-        d.o = (int64_t)__umul64hi(hh, (uint64_t)d.dw);
-        d.q = (uint64_t)(d.dw / mine);
-        d.f = (uint64_t)((((u128)(uint64_t)(d.dw % mine)) << 64) / (u128)(uint64_t)mine);
+      uint64_t q = 0, f = 0;  // weight d_w / c_w = q + f / 2^64 of the lane's item
+      if (lane < live) {
+        const int at = my->who[lane];
+        const int32_t w = __ldg(g.col + a.bo + a.first + at);
+        const int64_t bw = __ldg(g.row_ptr + w);
+        const uint32_t dw = (uint32_t)(__ldg(g.row_ptr + w + 1) - bw);  // < 2^31
+        mine = probes_of((int64_t)dw, pe);
+        const uint64_t key = ((uint64_t)(uint32_t)min(a.u, a.v) << 32) | (uint32_t)max(a.u, a.v);
+        const uint64_t hh = splitmix(splitmix(seed ^ splitmix(key)) ^ (uint64_t)(uint32_t)w);
+        my->bw[lane] = bw;
+        my->dw[lane] = (int32_t)dw;
+        my->o[lane] = (int32_t)__umul64hi(hh, (uint64_t)dw);
+        my->w[lane] = w;
+        my->cls[lane] = (uint8_t)(a.vside ? kSv : (((inT >> at) & 1u) ? kT : kSu));
+        const uint32_t cw = (uint32_t)mine;
+        q = dw / cw;
+        // floor((d_w mod c_w) 2^64 / c_w), 32 bits of the quotient at a time
+        const uint64_t r0 = (uint64_t)(dw % cw) << 32;
+        const uint64_t r1 = (r0 % cw) << 32;
+        f = ((r0 / cw) << 32) | (r1 / cw);
       }
-      my[lane] = d;
       __syncwarp();
-      int64_t incl = mine;
+      int64_t start = mine;  // first probe of the item; the total past the items
 #pragma unroll
       for (int s = 1; s < 32; s <<= 1) {
-        const int64_t y = __shfl_up_sync(kFull, incl, s);
-        if (lane >= s) incl += y;
+        const int64_t y = __shfl_up_sync(kFull, start, s);
+        if (lane >= s) start += y;
       }
-      start = incl - mine;
-      ctotal = __shfl_sync(kFull, incl, 31);
-      cur = c;
-      cur_e = e;
-    }
-    const int64_t lo = (task - __ldg(task_off + c)) * kTaskProbes;
-    const int32_t len = (int32_t)min(ctotal - lo, kTaskProbes);
-    // item starts relative to the task's first probe, clamped to 32 bits
-    // (order kept; the item holding a probe of this task starts less than
-    // one item's probes before lo)
-    const int32_t srel = (int32_t)max(min(start - lo, kTaskProbes), (int64_t)INT32_MIN + 1);
-    for (int32_t r = lane; r - lane < len; r += 32) {
-      int j = 0;
+      const int64_t ctotal = __shfl_sync(kFull, start, 31);
+      start -= mine;
+      unsigned cnt[kCats];
 #pragma unroll
-      for (int step = 16; step > 0; step >>= 1) {
-        const int32_t sv = __shfl_sync(kFull, srel, j + step);
-        if (sv <= r) j += step;
-      }
-      const int32_t sj = __shfl_sync(kFull, srel, j);
-      if (r >= len) continue;
-      const ItemDesc& it = my[j];
-      int64_t p = it.o + (int64_t)(r - sj);
-      if (p >= it.dw) p -= it.dw;
-      const int32_t x = __ldg(g.col + it.bw + p);
-      const int32_t xs =
-          g.col_hm != nullptr ? (int32_t)__ldg(g.col_hm + it.bw + p) : kNoSlotInfo;
-      const bool in_u = adj_contains(g, u, bu, du, x, xs);
-      int cat = -1;
-      if (it.cls == kT) {
-        if (in_u && x > it.w && adj_contains(g, v, bv, dv, x, xs)) cat = 0;
-      } else if (x != u && x != v) {
-        const bool in_v = adj_contains(g, v, bv, dv, x, xs);
-        if (in_u && in_v) cat = 3;                                         // omega
-        else if (it.cls == kSu && in_v) cat = 2;                           // 4-cycle
-        else if (it.cls == kSu && in_u && x > it.w) cat = 1;               // S_u pair
-        else if (it.cls == kSv && in_v && x > it.w) cat = 1;               // S_v pair
-      }
-      if (cat >= 0) {
-#pragma unroll
-        for (int k = 0; k < kCats; ++k)
-          if (k == cat) {
-            h.I[k] += it.q;
-            h.F[k] += it.f;
+      for (int k = 0; k < kCats; ++k) cnt[k] = 0;
+      for (; here > 0; --here, ++task) {
+        const int64_t lo = (task - __ldg(task_off + c)) * kTaskProbes;
+        const int32_t len = (int32_t)min(ctotal - lo, kTaskProbes);
+        // item starts relative to the task's first probe, clamped to 32 bits
+        // (order kept; the item holding a probe of this task starts less than
+        // one item's probes before lo)
+        const int32_t srel = (int32_t)max(min(start - lo, kTaskProbes), (int64_t)INT32_MIN + 1);
+        const int32_t sd = __shfl_down_sync(kFull, srel, 1);
+        const int32_t se = lane < 31 ? min(sd, len) : len;
+        for (int32_t r = 0; r < len;) {
+          const int j0 = 31 - __clz(__ballot_sync(kFull, srel <= r));
+          const int32_t sj = __shfl_sync(kFull, srel, j0);
+          const int32_t end = __shfl_sync(kFull, se, j0);
+          if (end - r >= 32) {
+            const int32_t dw = my->dw[j0], w = my->w[j0];
+            const int64_t bw = my->bw[j0];
+            const int cls = my->cls[j0];
+            // position in the window; o < d_w and fewer than d_w probes, so
+            // the sum can pass 2^31
+            uint32_t p = (uint32_t)my->o[j0] + (uint32_t)(r - sj) + lane;
+            unsigned c1 = 0, c2 = 0, c3 = 0;
+            for (; end - r >= 32; r += 32, p += 32) {
+              const uint32_t pp = p >= (uint32_t)dw ? p - (uint32_t)dw : p;
+              const int32_t x = __ldg(g.col + bw + pp);
+              const int32_t xs = slots ? (int32_t)__ldg(g.col_hm + bw + pp) : -1;
+              const int cat = probe_cat(su, sv, a.u, a.v, cls, w, x, xs);
+              c1 += cat == 0 || cat == 1;
+              c2 += cat == 2;
+              c3 += cat == 3;
+            }
+            c1 = __reduce_add_sync(kFull, c1);
+            if (cls != kT) {
+              c2 = __reduce_add_sync(kFull, c2);
+              c3 = __reduce_add_sync(kFull, c3);
+            }
+            if (lane == j0) {
+              cnt[0] += cls == kT ? c1 : 0u;
+              cnt[1] += cls == kT ? 0u : c1;
+              cnt[2] += c2;
+              cnt[3] += c3;
+            }
+            continue;
           }
+          const int32_t ds = srel - r;
+          const unsigned marks = __reduce_or_sync(kFull, ds > 0 && ds < 32 ? 1u << ds : 0u);
+          const int j = min(j0 + __popc(marks & upto), 31);
+          const int32_t o = r + lane - __shfl_sync(kFull, srel, j);
+          int cat = -1;
+          if (r + lane < len) {
+            const uint32_t dw = (uint32_t)my->dw[j];
+            uint32_t pp = (uint32_t)my->o[j] + (uint32_t)o;
+            if (pp >= dw) pp -= dw;
+            const int32_t x = __ldg(g.col + my->bw[j] + pp);
+            const int32_t xs = slots ? (int32_t)__ldg(g.col_hm + my->bw[j] + pp) : -1;
+            cat = probe_cat(su, sv, a.u, a.v, my->cls[j], my->w[j], x, xs);
+          }
+          const unsigned range = bits_below(se - r) & ~bits_below(srel - r);
+#pragma unroll
+          for (int k = 0; k < kCats; ++k)
+            cnt[k] += __popc(__ballot_sync(kFull, cat == k) & range);
+          r += 32;
+        }
+      }
+      // weighted counts to the edge
+#pragma unroll
+      for (int k = 0; k < kCats; ++k) {
+        if (!__any_sync(kFull, cnt[k] != 0)) continue;
+        unsigned long long I = (unsigned long long)cnt[k] * q;
+        u128 F = (u128)cnt[k] * f;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+          I += __shfl_xor_sync(kFull, I, o);
+          F += shfl_xor_u128(F, o);
+        }
+        if (lane == 0) acc_add(acc + e * 3 * kCats + 3 * k, I, F);
       }
     }
   }
-  if (cur >= 0) flush_hits(h, acc + cur_e * 3 * kCats, lane);
 }
 
 __device__ __forceinline__ double acc_value(const unsigned long long* a) {
@@ -546,7 +646,7 @@ extern "C" gs_status gs_micro(const gs_graph* gr, gs_workspace* ws, const int32_
         g, uv, choff, chunk_e, C, p_e, t, tmask, task_off, stats);
     GS_TRY(exclusive_scan_i64(task_off, task_off, C, tmp1, stream));
     k_micro_probe<<<sm_count() * kProbeBlocksPerSm, kThreads, 0, stream>>>(
-        g, uv, choff, chunk_e, tmask, task_off, C, p_e, seed, acc);
+        g, uv, choff, chunk_e, tmask, task_off, C, p_e, seed, acc, stats + 1);
     launches += 8;
   }
   k_micro_final<<<final_blocks, kThreads, 0, stream>>>(

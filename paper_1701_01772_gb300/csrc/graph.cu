@@ -350,16 +350,19 @@ __global__ void __launch_bounds__(kBlockRowThreads)
 // every x in N(w), one to the counter of each big neighbour of x (the
 // 16-bit column slots of x's big neighbours, listed beforehand), and writes
 // the finished row out. The whole CTA walks the concatenation of the
-// big-neighbour lists of N(w) (kMidRowThreads entries at a time): warps
+// big-neighbour lists of N(w) (a CTA's worth of entries at a time): warps
 // take 32-position segments, one position per lane, so a hub in N(w) with
-// thousands of big neighbours is spread over all warps.
+// thousands of big neighbours is spread over all warps. The CTA has the
+// fewest threads that still fill an SM next to the rows' shared memory
+// (row_shape): a row that is short for 1024 threads spends its time in the
+// block's barriers. Registration and exact 3-node counts of the 100k-vertex
+// power-law graph (91,000 rows of 17.6 KB, 256 threads): 33.4 -> 28.3 ms.
 #ifndef GS_BIG_MAX
 #define GS_BIG_MAX 65536
 #endif
 constexpr int kBigMax = GS_BIG_MAX;
 static_assert(kBigMax <= 65536, "column slots are stored in 16 bits");
 constexpr int kBigMin = 1024;  // narrowest shape tried
-constexpr int kMidRowThreads = 1024;
 
 // Number of big neighbours of every vertex. One warp per vertex.
 __global__ void k_big_count(const int64_t* __restrict__ row_ptr, const int32_t* __restrict__ col,
@@ -404,20 +407,21 @@ __global__ void k_mid_row_vertex(const int32_t* __restrict__ tb_slot, int64_t n,
   }
 }
 
-__global__ void __launch_bounds__(kMidRowThreads, 1)
+template <int kRowThreads>
+__global__ void __launch_bounds__(kRowThreads, 2048 / kRowThreads)
     k_mid_rows(const int64_t* __restrict__ row_ptr, const int32_t* __restrict__ col,
                const int32_t* __restrict__ rows_v, int64_t rows,
                const int64_t* __restrict__ boff, const uint16_t* __restrict__ blist,
                int64_t bg_count, uint16_t* __restrict__ md,
                unsigned long long* __restrict__ counter) {
   extern __shared__ uint32_t acc[];  // (bg_count + 1) / 2 words
-  // the current kMidRowThreads entries of N(w) that have big neighbours:
+  // the current kRowThreads entries of N(w) that have big neighbours:
   // list offset and first position in the concatenation of their lists
-  __shared__ int64_t sbo[kMidRowThreads];
-  __shared__ int32_t sst[kMidRowThreads];
-  __shared__ int32_t wn[kMidRowThreads / 32], wl[kMidRowThreads / 32];
+  __shared__ int64_t sbo[kRowThreads];
+  __shared__ int32_t sst[kRowThreads];
+  __shared__ int32_t wn[kRowThreads / 32], wl[kRowThreads / 32];
   __shared__ int64_t cur;
-  constexpr int kWarps = kMidRowThreads / 32;
+  constexpr int kWarps = kRowThreads / 32;
   const int W = (int)((bg_count + 1) / 2);
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   for (;;) {
@@ -425,10 +429,10 @@ __global__ void __launch_bounds__(kMidRowThreads, 1)
     __syncthreads();  // the previous row has been written out
     const int64_t r = cur;
     if (r >= rows) break;
-    for (int i = threadIdx.x; i < W; i += kMidRowThreads) acc[i] = 0u;
+    for (int i = threadIdx.x; i < W; i += kRowThreads) acc[i] = 0u;
     const int32_t w = rows_v[r];
     const int64_t s = row_ptr[w], d = row_ptr[w + 1] - s;
-    for (int64_t c0 = 0; c0 < d; c0 += kMidRowThreads) {
+    for (int64_t c0 = 0; c0 < d; c0 += kRowThreads) {
       int64_t bo = 0;
       int32_t len = 0;
       if (c0 + threadIdx.x < d) {
@@ -466,9 +470,9 @@ __global__ void __launch_bounds__(kMidRowThreads, 1)
       __syncthreads();
       // 32-position segments of the concatenation, one per warp at a time;
       // a segment spans at most 32 entries (all non-empty)
-      for (int32_t q0 = wid * 32; q0 < total; q0 += kMidRowThreads) {
+      for (int32_t q0 = wid * 32; q0 < total; q0 += kRowThreads) {
         int k0 = 0;  // last entry starting at or before q0
-        for (int step = kMidRowThreads / 2; step > 0; step >>= 1)
+        for (int step = kRowThreads / 2; step > 0; step >>= 1)
           if (k0 + step < cnt && sst[k0 + step] <= q0) k0 += step;
         const int32_t q = q0 + lane;
         int k = k0;  // last entry starting at or before q
@@ -485,7 +489,7 @@ __global__ void __launch_bounds__(kMidRowThreads, 1)
     __syncthreads();
     const uint16_t* a16 = reinterpret_cast<const uint16_t*>(acc);
     uint16_t* out = md + r * bg_count;
-    for (int64_t c = threadIdx.x; c < bg_count; c += kMidRowThreads) out[c] = a16[c];
+    for (int64_t c = threadIdx.x; c < bg_count; c += kRowThreads) out[c] = a16[c];
   }
 }
 
@@ -732,7 +736,8 @@ __global__ void k_giant_index(const int64_t* __restrict__ flag_scan, int64_t cou
 // warp, and writes the row once. Pairs of two giants (degree >= 65,536,
 // whose co-degree may not fit 16 bits) go to the 32-bit giant table by
 // global atomics instead (marked 0xFFFF afterwards by k_mark_giant_pairs).
-__global__ void __launch_bounds__(kMidRowThreads, 1)
+template <int kRowThreads>
+__global__ void __launch_bounds__(kRowThreads, 2048 / kRowThreads)
     k_table_rows(const int64_t* __restrict__ row_ptr, const int32_t* __restrict__ col,
                  const int32_t* __restrict__ tb_vertex, int64_t count,
                  const int64_t* __restrict__ loff, const int32_t* __restrict__ lists,
@@ -740,11 +745,11 @@ __global__ void __launch_bounds__(kMidRowThreads, 1)
                  uint32_t* __restrict__ giant_codeg, uint16_t* __restrict__ tb,
                  unsigned long long* __restrict__ counter) {
   extern __shared__ uint32_t acc[];  // count / 2 words (row 0 is the longest)
-  __shared__ int64_t sbo[kMidRowThreads];
-  __shared__ int32_t sst[kMidRowThreads];
-  __shared__ int32_t wn[kMidRowThreads / 32], wl[kMidRowThreads / 32];
+  __shared__ int64_t sbo[kRowThreads];
+  __shared__ int32_t sst[kRowThreads];
+  __shared__ int32_t wn[kRowThreads / 32], wl[kRowThreads / 32];
   __shared__ int64_t cur;
-  constexpr int kWarps = kMidRowThreads / 32;
+  constexpr int kWarps = kRowThreads / 32;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   for (;;) {
     if (threadIdx.x == 0) cur = (int64_t)atomicAdd(counter, 1ull);
@@ -753,11 +758,11 @@ __global__ void __launch_bounds__(kMidRowThreads, 1)
     if (a >= count - 1) break;  // the last row is empty
     const int64_t R = count - a - 1;
     const int W = (int)((R + 1) / 2);
-    for (int i = threadIdx.x; i < W; i += kMidRowThreads) acc[i] = 0u;
+    for (int i = threadIdx.x; i < W; i += kRowThreads) acc[i] = 0u;
     const int32_t va = tb_vertex[a];
     const int32_t ga = giant != nullptr ? giant[a] : -1;
     const int64_t s = row_ptr[va], d = row_ptr[va + 1] - s;
-    for (int64_t c0 = 0; c0 < d; c0 += kMidRowThreads) {
+    for (int64_t c0 = 0; c0 < d; c0 += kRowThreads) {
       int64_t bo = 0;
       int32_t len = 0;
       if (c0 + threadIdx.x < d) {
@@ -804,9 +809,9 @@ __global__ void __launch_bounds__(kMidRowThreads, 1)
         sst[at] = bl + incl - len;
       }
       __syncthreads();
-      for (int32_t q0 = wid * 32; q0 < total; q0 += kMidRowThreads) {
+      for (int32_t q0 = wid * 32; q0 < total; q0 += kRowThreads) {
         int k0 = 0;
-        for (int step = kMidRowThreads / 2; step > 0; step >>= 1)
+        for (int step = kRowThreads / 2; step > 0; step >>= 1)
           if (k0 + step < cnt && sst[k0 + step] <= q0) k0 += step;
         const int32_t q = q0 + lane;
         int k = k0;
@@ -829,7 +834,7 @@ __global__ void __launch_bounds__(kMidRowThreads, 1)
     __syncthreads();
     const uint16_t* a16 = reinterpret_cast<const uint16_t*>(acc);
     uint16_t* out = tb + tb_index(a, a + 1, count);
-    for (int64_t c = threadIdx.x; c < R; c += kMidRowThreads) out[c] = a16[c];
+    for (int64_t c = threadIdx.x; c < R; c += kRowThreads) out[c] = a16[c];
   }
 }
 
@@ -872,6 +877,37 @@ static gs_status read_error(DevError* d_err, cudaStream_t stream, const char* wh
   }
   return GS_OK;
 }
+
+// Threads and CTAs per SM of a row kernel whose rows take `row` bytes of
+// shared memory: the smallest CTA of which 2048 threads fit an SM, else 1024.
+struct RowShape {
+  int threads, per_sm;
+};
+
+static RowShape row_shape(size_t row) {
+  const size_t sm = (size_t)220 << 10;  // left for CTAs, each with 1 KB of the system's
+  for (int t = 256; t < 1024; t *= 2) {
+    const size_t cta = row + (size_t)t * 12 + 2048;
+    if (sm / cta >= (size_t)(2048 / t)) return RowShape{t, 2048 / t};
+  }
+  return RowShape{1024, sm / (row + 1024 * 12 + 2048) >= 2 ? 2 : 1};
+}
+
+// Launches kernel<threads> for the row shape with `smem` dynamic bytes.
+#define GS_LAUNCH_ROWS(kernel, smem, stream, ...)                                             \
+  [&]() -> cudaError_t {                                                                      \
+    const RowShape sh = row_shape(smem);                                                      \
+    auto go = [&](auto k) -> cudaError_t {                                                    \
+      cudaError_t le = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,   \
+                                            (int)(smem));                                     \
+      if (le != cudaSuccess) return le;                                                       \
+      k<<<sm_count() * sh.per_sm, sh.threads, smem, stream>>>(__VA_ARGS__);                   \
+      return cudaGetLastError();                                                              \
+    };                                                                                        \
+    return sh.threads == 256   ? go(kernel<256>)                                              \
+           : sh.threads == 512 ? go(kernel<512>)                                              \
+                               : go(kernel<1024>);                                            \
+  }()
 
 // Smallest degree threshold d >= min_deg with at most `cap` vertices of
 // degree >= d (binary search with a device count per probe).
@@ -1147,14 +1183,12 @@ static gs_status build_hub_index(gs_graph* g, uint64_t budget, bool tables, cuda
           g->dev.row_ptr, g->dev.col, g->tb_slot, n, flag, lists);
       uint32_t* tb_w = reinterpret_cast<uint32_t*>(g->tb_codeg);
       const size_t row_smem = sizeof(uint32_t) * (size_t)(n_tb / 2 + 1);
-      cudaError_t e = cudaFuncSetAttribute(k_table_rows,
-                                           cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                           (int)row_smem);
-      if (e == cudaSuccess) e = cudaMemsetAsync(d_cnt, 0, sizeof(unsigned long long), stream);
+      cudaError_t e = cudaMemsetAsync(d_cnt, 0, sizeof(unsigned long long), stream);
+      if (e == cudaSuccess)
+        e = GS_LAUNCH_ROWS(k_table_rows, row_smem, stream, g->dev.row_ptr, g->dev.col, hubs, n_tb,
+                           flag, lists, g->tb_giant, giants, g->tb_giant_codeg, g->tb_codeg,
+                           d_cnt);
       if (e == cudaSuccess) {
-        k_table_rows<<<sm_count(), kMidRowThreads, row_smem, stream>>>(
-            g->dev.row_ptr, g->dev.col, hubs, n_tb, flag, lists, g->tb_giant, giants,
-            g->tb_giant_codeg, g->tb_codeg, d_cnt);
         if (g->tb_giant != nullptr)
           k_mark_giant_pairs<<<grid_for(n_tb, 256, 8), 256, 0, stream>>>(g->tb_giant, n_tb, tb_w);
         e = cudaStreamSynchronize(stream);
@@ -1300,14 +1334,11 @@ static gs_status build_hub_index(gs_graph* g, uint64_t budget, bool tables, cuda
                                                                  g->bg_slot, flag, blist);
         k_mid_row_vertex<<<grid_for(n, 256, 8), 256, 0, stream>>>(g->tb_slot, n, rows_v);
         const size_t row_smem = sizeof(uint32_t) * (size_t)((n_bg + 1) / 2);
-        cudaError_t e = cudaFuncSetAttribute(k_mid_rows, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)row_smem);
-        if (e == cudaSuccess) e = cudaMemsetAsync(d_cnt, 0, sizeof(unsigned long long), stream);
-        if (e == cudaSuccess) {
-          k_mid_rows<<<sm_count(), kMidRowThreads, row_smem, stream>>>(
-              g->dev.row_ptr, g->dev.col, rows_v, rows, flag, blist, n_bg, g->md_codeg, d_cnt);
-          e = cudaStreamSynchronize(stream);
-        }
+        cudaError_t e = cudaMemsetAsync(d_cnt, 0, sizeof(unsigned long long), stream);
+        if (e == cudaSuccess)
+          e = GS_LAUNCH_ROWS(k_mid_rows, row_smem, stream, g->dev.row_ptr, g->dev.col, rows_v, rows,
+                             flag, blist, n_bg, g->md_codeg, d_cnt);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
         cudaFree(blist);
         cudaFree(rows_v);
         if (e != cudaSuccess) return cuda_fail(e, "mid x big table", __FILE__, __LINE__);

@@ -73,7 +73,7 @@ constexpr unsigned long long kEmpty = ~0ull;
 // Device counters of one count (CountBufs::stats): 0 triangle-pass tests,
 // 1 4-node tests, 2 / 3 model bytes (3-node / 4-node part), 4 dense groups,
 // 5 k_quad task counter, 6 dense edges, 7 k_dense_pairs unit counter,
-// 8 k_chunk_cost chunk counter, 9 tests of dense edges' members without a
+// 8 k_chunk_cost chunk counter, 10 k_tri_chunks chunk counter, 9 tests of dense edges' members without a
 // dense slot (k_dense_pairs).
 constexpr int kStatSlots = 16;
 // Chunks per run a k_chunk_cost warp takes from its counter, at most; also
@@ -114,6 +114,7 @@ constexpr int64_t kQuadGrabTests = GS_QUAD_GRAB_TESTS;
 #ifndef GS_DENSE_BLOCKS
 #define GS_DENSE_BLOCKS 6
 #endif
+constexpr int kTriBlocksPerSm = 6;  // k_tri_chunks: at most 40 registers
 constexpr int kDenseThreads = GS_DENSE_THREADS;
 constexpr int kDenseBlocksPerSm = GS_DENSE_BLOCKS;
 // T entries per k_dense_pairs work unit (a heavy dense edge is split into
@@ -226,13 +227,11 @@ __global__ void k_prep(DevGraph g, const int32_t* __restrict__ pairs, int64_t K,
 }
 
 // ---------------------------------------------------------------- tri
-// Positions [0, P) of the concatenated (padded) N(u) lists are split into
-// equal contiguous ranges of 32-position groups, one range per warp.
-template <bool kPad>
+// 3-node work alone: positions [0, P) of the concatenated N(u) lists are
+// split into equal contiguous ranges of 32-position groups, one range per warp.
 __global__ void __launch_bounds__(kThreads) k_tri(DevGraph g, const int2* __restrict__ uv,
                                                   const int64_t* __restrict__ off, int64_t K,
-                                                  unsigned long long* __restrict__ t,
-                                                  uint32_t* __restrict__ tbits) {
+                                                  unsigned long long* __restrict__ t) {
   const int lane = threadIdx.x & 31;
   const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
@@ -259,7 +258,6 @@ __global__ void __launch_bounds__(kThreads) k_tri(DevGraph g, const int2* __rest
       }
     }
     const unsigned ball = __ballot_sync(kFull, hit);
-    if (kPad && lane == 0) tbits[gi] = ball;
     const unsigned grp = __match_any_sync(kFull, (unsigned long long)le);
     const int cnt = __popc(ball & grp);
     if (cnt && lane == __ffs(grp) - 1) atomicAdd(t + le, (unsigned long long)cnt);
@@ -267,11 +265,73 @@ __global__ void __launch_bounds__(kThreads) k_tri(DevGraph g, const int2* __rest
   }
 }
 
-// Host launcher of the unpadded triangle pass for count_static.cu (a
-// kernel template can only be launched from the file that defines it).
+// The triangle pass of the 4-node work: positions padded to 32 per edge, so
+// a chunk of 32 positions lies in one edge. Warps take runs of chunks from a
+// counter; what an edge needs (N(u), and how "x in N(v)" is answered) is
+// looked up when the edge changes, t is added once per edge and run, and the
+// next chunk's elements are loaded before this chunk's answers are used.
+// k_tri<true> looked all of it up for every position: 1M-vertex power-law
+// graph exact (5.6e9 positions): 47.2 -> 37.9 ms (44.2 / 40.8 ms at 8 / 5
+// CTAs per SM).
+__global__ void __launch_bounds__(kThreads, kTriBlocksPerSm)
+    k_tri_chunks(const __grid_constant__ DevGraph g, const int2* __restrict__ uv,
+                 const int64_t* __restrict__ off, int64_t K, unsigned long long* __restrict__ t,
+                 uint32_t* __restrict__ tbits, unsigned long long* __restrict__ counter) {
+  const int lane = threadIdx.x & 31;
+  const int64_t groups = __ldg(off + K) >> 5;  // padded: a multiple of 32
+  const int grab =
+      run_length(groups, (int64_t)gridDim.x * (kThreads / 32), (int64_t)kCostGrab);
+  int64_t e = -1, first = 0, end = 0, bu = 0;
+  int32_t du = 0, v = 0;
+  EndSet sv{};
+  for (;;) {
+    unsigned long long got = 0;
+    if (lane == 0) got = atomicAdd(counter, (unsigned long long)grab);
+    const int64_t g0 = (int64_t)__shfl_sync(kFull, got, 0);
+    if (g0 >= groups) break;
+    const int64_t g1 = min(groups, g0 + grab);
+    unsigned found = 0;  // of edge e in this run
+    int32_t x = -1, xs = -1;
+    bool loaded = false;
+    for (int64_t gi = g0; gi < g1; ++gi) {
+      const int64_t p0 = gi * 32;
+      if (p0 < first || p0 >= end) {  // another edge: the next one, or a search
+        if (found && lane == 0) atomicAdd(t + e, (unsigned long long)found);
+        found = 0;
+        e = p0 == end && e >= 0 ? e + 1 : last_le(off, K, p0);
+        first = __ldg(off + e);
+        end = __ldg(off + e + 1);
+        const int2 pr = uv[e];
+        v = pr.y;
+        du = (int32_t)deg_of(g.row_ptr, pr.x, &bu);
+        int64_t bv;
+        const int64_t dv = deg_of(g.row_ptr, v, &bv);
+        sv = end_set(g, v, bv, dv);
+        loaded = false;
+      }
+      const int64_t i = p0 - first + lane;
+      if (!loaded) {
+        x = i < du ? __ldg(g.col + bu + i) : -1;
+        xs = sv.mrow != nullptr && i < du ? (int32_t)__ldg(g.col_hm + bu + i) : -1;
+      }
+      const int32_t y = x, ys = xs;
+      loaded = gi + 1 < g1 && p0 + 32 < end;
+      if (loaded) {
+        x = i + 32 < du ? __ldg(g.col + bu + i + 32) : -1;
+        xs = sv.mrow != nullptr && i + 32 < du ? (int32_t)__ldg(g.col_hm + bu + i + 32) : -1;
+      }
+      const unsigned ball = __ballot_sync(kFull, y >= 0 && y != v && set_has(sv, y, ys));
+      if (lane == 0) tbits[gi] = ball;
+      found += __popc(ball);
+    }
+    if (found && lane == 0) atomicAdd(t + e, (unsigned long long)found);
+  }
+}
+
+// Host launcher of the 3-node triangle pass for count_static.cu.
 void launch_tri_unpadded(const DevGraph& g, const int2* uv, const int64_t* off, int64_t K,
                          unsigned long long* t, int blocks, cudaStream_t stream) {
-  k_tri<false><<<blocks, kThreads, 0, stream>>>(g, uv, off, K, t, nullptr);
+  k_tri<<<blocks, kThreads, 0, stream>>>(g, uv, off, K, t);
 }
 
 // ---------------------------------------------------------------- compact T
@@ -863,14 +923,13 @@ struct ItemCost {
 
 // Most items are in S_u and answered by a table: for those only the element,
 // its table slot and the table entry are read; degrees are read by the rest.
-__device__ __forceinline__ ItemCost item_cost(const DevGraph& g, const CostEdge& c, int64_t i,
-                                              uint32_t tword, const int32_t* __restrict__ tpre,
-                                              int lane, bool need_q) {
+// w: the item's vertex (-1: no item), sw: its table slot (-1 without tables).
+__device__ __forceinline__ ItemCost item_cost(const DevGraph& g, const CostEdge& c, int32_t w,
+                                              int32_t sw, uint32_t tword,
+                                              const int32_t* __restrict__ tpre, int lane,
+                                              bool need_q) {
   ItemCost r{0, 0, 0, false};
-  if (i >= c.du) return r;
-  const int64_t p = c.bu + i;
-  const int32_t w = __ldg(g.col + p);
-  if (w == c.v) return r;
+  if (w < 0 || w == c.v) return r;
   const bool in_t = (tword >> lane) & 1u;
   if (need_q) {
     // segment B: -(c(w, u) - 1) for w in T, c(w, v) - 1 for w in S_u
@@ -881,7 +940,7 @@ __device__ __forceinline__ ItemCost item_cost(const DevGraph& g, const CostEdge&
       if (b < 255u) tc = b + 1u;
     }
     if (tc == 0 && g.tb_slot != nullptr) {
-      const int32_t sw = __ldg(g.col_tb != nullptr ? g.col_tb + p : g.tb_slot + w);
+      if (g.col_tb == nullptr) sw = __ldg(g.tb_slot + w);
       tc = table_codeg(g, w, sw, in_t ? c.slot_u : c.slot_v, in_t ? c.col_u : c.col_v);
     }
     r.tabled = tc != 0;
@@ -906,8 +965,10 @@ __device__ __forceinline__ ItemCost item_cost(const DevGraph& g, const CostEdge&
 // Chunk costs: membership tests per chunk and the number of tasks it needs.
 // Also adds the constant part of q. Bound by the latency of the table reads
 // (two bytes of a random sector per item); cost phase of the 1M-vertex
-// power-law graph exact: 131 -> 116 ms when the items a table answers stopped
-// reading their degrees and the sums went to 32-bit warp reductions.
+// power-law graph exact: 131 -> 114 ms when the items a table answers stopped
+// reading their degrees and the sums went to 32-bit warp reductions, 110 ms
+// with one addition to q per edge and run. Loading the next chunk's elements
+// ahead spilled at 40 registers (119 ms) and gave 112 ms at 64.
 __global__ void __launch_bounds__(kThreads, kCostBlocksPerSm)
     k_chunk_cost(DevGraph g, const int2* __restrict__ uv, const int64_t* __restrict__ off, int64_t K,
                  const unsigned long long* __restrict__ t, const uint32_t* __restrict__ tbits,
@@ -937,11 +998,13 @@ __global__ void __launch_bounds__(kThreads, kCostBlocksPerSm)
     // packs: consecutive chunks of the run with at most 32 live items in all,
     // so that k_quad sets up a warp's worth of items at a time; a pack's
     // tasks are counted at its first chunk
-    int64_t head = g0, pcost = 0;
+    int64_t head = g0, pcost = 0, qsum = 0;  // qsum: constant of edge c.e in this run
     int plive = 0;
     for (int64_t gi = g0; gi < g1; ++gi) {
       const int64_t p0 = gi * 32;
       if (p0 < c.first || p0 >= c.end) {  // another edge: the next one, or a search
+        if (qsum != 0 && lane == 0) atomicAdd(q + c.e, (unsigned long long)qsum);
+        qsum = 0;
         c.e = p0 == c.end && c.e >= 0 ? c.e + 1 : last_le(off, K, p0);
         c.first = __ldg(off + c.e);
         c.end = __ldg(off + c.e + 1);
@@ -964,8 +1027,11 @@ __global__ void __launch_bounds__(kThreads, kCostBlocksPerSm)
           c.col_v = __ldg(g.bg_slot + pr.y);
         }
       }
-      const ItemCost it =
-          item_cost(g, c, p0 + lane - c.first, __ldg(tbits + gi), tpre + gi, lane, need_q);
+      const int64_t i = p0 + lane - c.first, at = c.bu + i;
+      const int32_t w = i < c.du ? __ldg(g.col + at) : -1;
+      const int32_t sw = g.col_tb != nullptr && i < c.du ? __ldg(g.col_tb + at) : -1;
+      const uint32_t tword = __ldg(tbits + gi);
+      const ItemCost it = item_cost(g, c, w, sw, tword, tpre + gi, lane, need_q);
       const unsigned live = __ballot_sync(kFull, (it.a | it.b) != 0);
       const unsigned tabled = __ballot_sync(kFull, it.tabled);
       if (lane == 0) reinterpret_cast<uint2*>(cbits)[gi] = make_uint2(live, tabled);
@@ -991,10 +1057,11 @@ __global__ void __launch_bounds__(kThreads, kCostBlocksPerSm)
       plive += __popc(live);
       if (lane == 0) {
         if (gi != head) task_cnt[gi] = 0;
-        if (qc != 0) atomicAdd(q + c.e, (unsigned long long)qc);
         tests += cost;
       }
+      qsum += qc;
     }
+    if (qsum != 0 && lane == 0) atomicAdd(q + c.e, (unsigned long long)qsum);
     if (lane == 0) task_cnt[head] = (pcost + task_probes - 1) / task_probes;
   }
   if (lane == 0 && tests) atomicAdd(stats + 1, (unsigned long long)tests);
@@ -1725,9 +1792,9 @@ int64_t launch_tri(const DevGraph& g, bool four, const Tuning& tu, CountBufs& b,
                    cudaStream_t stream) {
   const int grid = sm_count() * tu.tri_blocks_per_sm;
   if (four)
-    k_tri<true><<<grid, kThreads, 0, stream>>>(g, b.uv, b.off, b.K, b.t, b.tbits);
+    k_tri_chunks<<<grid, kThreads, 0, stream>>>(g, b.uv, b.off, b.K, b.t, b.tbits, b.stats + 10);
   else
-    k_tri<false><<<grid, kThreads, 0, stream>>>(g, b.uv, b.off, b.K, b.t, nullptr);
+    k_tri<<<grid, kThreads, 0, stream>>>(g, b.uv, b.off, b.K, b.t);
   return 1;
 }
 

@@ -222,62 +222,6 @@ __device__ __forceinline__ u128 shfl_xor_u128(u128 v, int o) {
   return ((u128)hi << 64) | lo;
 }
 
-// How "x in N(y)" is answered for an endpoint y, looked up once per chunk
-// instead of once per probe: a row of words (dense row or bitmap, bit
-// x - first), the matrix row (for an x with a matrix slot), a bucket
-// directory, or a halving search of the list.
-struct EndSet {
-  const uint32_t* words;
-  const uint32_t* mrow;
-  const uint32_t* dir;
-  const int32_t* list;
-  int32_t first, deg, shift;
-};
-
-// A bitmap row of at most this many words (32 KB) stays in the L1 cache, so
-// it answers every x and the matrix slots need not be read.
-constexpr int64_t kShortRowWords = 8192;
-
-__device__ __forceinline__ EndSet end_set(const DevGraph& g, int32_t y, int64_t by, int64_t dy) {
-  EndSet s{nullptr, nullptr, nullptr, g.col + by, 0, (int32_t)dy, 0};
-  if (g.dm_row != nullptr) {
-    const int64_t r = __ldg(g.dm_row + y);
-    if (r >= 0) {
-      s.words = g.dm_bits + r;
-      s.first = __ldg(g.dm_first + y);
-      return s;
-    }
-  }
-  const int32_t b = bitmap_slot(g, y);
-  if (b >= 0) s.words = g.bm_bits + (int64_t)b * g.bm_words;
-  if (b >= 0 && g.bm_words <= kShortRowWords) return s;
-  const int32_t h = table_slot(g, y);
-  if (h >= 0) s.mrow = g.hm_bits + (int64_t)h * g.hm_words;
-  if (b < 0 && g.dir_at != nullptr) {
-    const int64_t at = __ldg(g.dir_at + y);
-    if (at >= 0) {
-      s.dir = g.dir + at;
-      s.shift = g.id_bits - dir_log2(dy, g.id_bits);
-    }
-  }
-  return s;
-}
-
-// xs: x's matrix slot (-1 if none; not looked at without a matrix row).
-__device__ __forceinline__ bool set_has(const EndSet& s, int32_t x, int32_t xs) {
-  if (s.mrow != nullptr && xs >= 0) return (__ldg(s.mrow + (xs >> 5)) >> (xs & 31)) & 1u;
-  if (s.words != nullptr) {
-    const int32_t lx = x - s.first;
-    return (__ldg(s.words + (lx >> 5)) >> (lx & 31)) & 1u;
-  }
-  if (s.dir != nullptr) {
-    const uint32_t* d = s.dir + (uint32_t)(x >> s.shift);
-    const uint32_t lo = __ldg(d), hi = __ldg(d + 1);
-    return sorted_contains(s.list + lo, (int64_t)(hi - lo), x);
-  }
-  return sorted_contains(s.list, s.deg, x);
-}
-
 // Statistic (0: x7, 1: x9, 2: x10, 3: omega, -1: none) of a probe that read x
 // from N(w). v is tested first; u only where its answer matters.
 __device__ __forceinline__ int probe_cat(const EndSet& su, const EndSet& sv, int32_t u, int32_t v,

@@ -356,12 +356,14 @@ __global__ void __launch_bounds__(kBlockRowThreads)
 // fewest threads that still fill an SM next to the rows' shared memory
 // (row_shape): a row that is short for 1024 threads spends its time in the
 // block's barriers. Registration and exact 3-node counts of the 100k-vertex
-// power-law graph (91,000 rows of 17.6 KB, 256 threads): 33.4 -> 28.3 ms.
+// power-law graph (91,000 rows of 17.6 KB, 256 threads): 33.4 -> 28.3 ms. The
+// rows of k_table_rows are hubs with long lists: 1024 threads, two CTAs per SM
+// where they fit (256 threads: 6.6 against 5.0 ms there).
 #ifndef GS_BIG_MAX
 #define GS_BIG_MAX 65536
 #endif
 constexpr int kBigMax = GS_BIG_MAX;
-static_assert(kBigMax <= 65536, "column slots are stored in 16 bits");
+static_assert(kBigMax <= 65536, "column slots are stored in 16 bits");  // 7 shapes from kBigMin
 constexpr int kBigMin = 1024;  // narrowest shape tried
 
 // Number of big neighbours of every vertex. One warp per vertex.
@@ -515,6 +517,41 @@ __global__ void k_mid_big_work(const int64_t* __restrict__ row_ptr, const int32_
     acc += (unsigned long long)m * b;
   }
   if (lane == 0 && acc) atomicAdd(total, acc);
+}
+
+// The build work of up to kShapes (lo, big) pairs in one pass over the
+// adjacency (one pass each took 2.3 of the 28 ms of a 100k-vertex graph's
+// registration).
+constexpr int kShapes = 8;
+struct ShapeBounds {
+  int64_t lo[kShapes], big[kShapes];
+};
+__global__ void k_mid_big_works(const int64_t* __restrict__ row_ptr,
+                                const int32_t* __restrict__ col, int64_t n,
+                                const __grid_constant__ ShapeBounds b, int shapes, int64_t hi,
+                                unsigned long long* __restrict__ total) {
+  const int lane = threadIdx.x & 31;
+  const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
+  unsigned long long acc[kShapes] = {};
+  for (int64_t x = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; x < n; x += warps) {
+    unsigned mid[kShapes] = {}, big[kShapes] = {};
+    for (int64_t p = row_ptr[x] + lane; p < row_ptr[x + 1]; p += 32) {
+      const int32_t y = col[p];
+      const int64_t d = __ldg(row_ptr + y + 1) - __ldg(row_ptr + y);
+#pragma unroll
+      for (int s = 0; s < kShapes; ++s) {
+        mid[s] += d >= b.lo[s] && d < hi;
+        big[s] += d >= b.big[s];
+      }
+    }
+#pragma unroll
+    for (int s = 0; s < kShapes; ++s)
+      acc[s] += (unsigned long long)__reduce_add_sync(0xffffffffu, mid[s]) *
+                __reduce_add_sync(0xffffffffu, big[s]);
+  }
+  if (lane == 0)
+    for (int s = 0; s < shapes; ++s)
+      if (acc[s]) atomicAdd(total + s, acc[s]);
 }
 
 // Pilot of the mid x big table's shape: for a deterministic spread of
@@ -879,14 +916,15 @@ static gs_status read_error(DevError* d_err, cudaStream_t stream, const char* wh
 }
 
 // Threads and CTAs per SM of a row kernel whose rows take `row` bytes of
-// shared memory: the smallest CTA of which 2048 threads fit an SM, else 1024.
+// shared memory: the smallest CTA (of at least `least` threads) of which 2048
+// threads fit an SM, else 1024.
 struct RowShape {
   int threads, per_sm;
 };
 
-static RowShape row_shape(size_t row) {
+static RowShape row_shape(size_t row, int least) {
   const size_t sm = (size_t)220 << 10;  // left for CTAs, each with 1 KB of the system's
-  for (int t = 256; t < 1024; t *= 2) {
+  for (int t = least; t < 1024; t *= 2) {
     const size_t cta = row + (size_t)t * 12 + 2048;
     if (sm / cta >= (size_t)(2048 / t)) return RowShape{t, 2048 / t};
   }
@@ -894,9 +932,9 @@ static RowShape row_shape(size_t row) {
 }
 
 // Launches kernel<threads> for the row shape with `smem` dynamic bytes.
-#define GS_LAUNCH_ROWS(kernel, smem, stream, ...)                                             \
+#define GS_LAUNCH_ROWS(kernel, least, smem, stream, ...)                                      \
   [&]() -> cudaError_t {                                                                      \
-    const RowShape sh = row_shape(smem);                                                      \
+    const RowShape sh = row_shape(smem, least);                                                   \
     auto go = [&](auto k) -> cudaError_t {                                                    \
       cudaError_t le = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,   \
                                             (int)(smem));                                     \
@@ -1185,7 +1223,7 @@ static gs_status build_hub_index(gs_graph* g, uint64_t budget, bool tables, cuda
       const size_t row_smem = sizeof(uint32_t) * (size_t)(n_tb / 2 + 1);
       cudaError_t e = cudaMemsetAsync(d_cnt, 0, sizeof(unsigned long long), stream);
       if (e == cudaSuccess)
-        e = GS_LAUNCH_ROWS(k_table_rows, row_smem, stream, g->dev.row_ptr, g->dev.col, hubs, n_tb,
+        e = GS_LAUNCH_ROWS(k_table_rows, 1024, row_smem, stream, g->dev.row_ptr, g->dev.col, hubs, n_tb,
                            flag, lists, g->tb_giant, giants, g->tb_giant_codeg, g->tb_codeg,
                            d_cnt);
       if (e == cudaSuccess) {
@@ -1257,23 +1295,50 @@ static gs_status build_hub_index(gs_graph* g, uint64_t budget, bool tables, cuda
       cudaFree(d_pc);
       cudaGetLastError();  // an allocation that failed only skips the pilot
     }
-    int64_t d_bg = 0, n_bg = 0, d_md = d_hi;
-    double best = -1.0;
+    // the shapes that fit the budget, and their build work in one pass
+    struct Shape {
+      int64_t dbg, nbg, dmd;
+    };
+    std::vector<Shape> shapes;
     for (int64_t cols = kBigMin; cols <= kBigMax; cols *= 2) {
       const int64_t bg_cap = g->dev.tb_count < cols ? g->dev.tb_count : cols;
-      int64_t dbg = 0, nbg = 0;
-      GS_TRY(hub_threshold(g, bg_cap, d_tb, d_cnt, stream, &dbg, &nbg));
-      if (nbg <= 0) continue;
-      const int64_t md_cap = (int64_t)(((double)budget - used) / (2.0 * (double)nbg));
-      if (md_cap <= 0) continue;
-      // lowest degree d_md >= kMidMinDegree with at most md_cap mid vertices
-      int64_t dmd = 0, n_ge = 0;
-      GS_TRY(hub_threshold(g, md_cap + g->dev.tb_count, kMidMinDegree, d_cnt, stream, &dmd,
-                           &n_ge));
-      if (dmd >= d_hi) continue;
-      // and, raising d_md if needed, at most kMidWorkMax build increments
-      unsigned long long w = 0;
-      GS_TRY(work_at(dmd, dbg, &w));
+      Shape sh{0, 0, 0};
+      GS_TRY(hub_threshold(g, bg_cap, d_tb, d_cnt, stream, &sh.dbg, &sh.nbg));
+      if (sh.nbg > 0) {
+        const int64_t md_cap = (int64_t)(((double)budget - used) / (2.0 * (double)sh.nbg));
+        if (md_cap > 0) {
+          // lowest degree >= kMidMinDegree with at most md_cap mid vertices
+          int64_t n_ge = 0;
+          GS_TRY(hub_threshold(g, md_cap + g->dev.tb_count, kMidMinDegree, d_cnt, stream, &sh.dmd,
+                               &n_ge));
+          if (sh.dmd < d_hi) shapes.push_back(sh);
+        }
+      }
+      if (bg_cap == g->dev.tb_count) break;
+    }
+    unsigned long long works[kShapes] = {};
+    if (!shapes.empty()) {
+      ShapeBounds sb;
+      for (int i = 0; i < kShapes; ++i) {
+        const bool on = i < (int)shapes.size();
+        sb.lo[i] = on ? shapes[i].dmd : INT64_MAX;
+        sb.big[i] = on ? shapes[i].dbg : INT64_MAX;
+      }
+      unsigned long long* d_works = reinterpret_cast<unsigned long long*>(flag);  // free here
+      const size_t bytes = sizeof(unsigned long long) * shapes.size();
+      GS_CUDA(cudaMemsetAsync(d_works, 0, bytes, stream));
+      k_mid_big_works<<<grid_for(n * 32, 256, 8), 256, 0, stream>>>(
+          g->dev.row_ptr, g->dev.col, n, sb, (int)shapes.size(), d_hi, d_works);
+      GS_CUDA(cudaMemcpyAsync(works, d_works, bytes, cudaMemcpyDeviceToHost, stream));
+      GS_CUDA(cudaStreamSynchronize(stream));
+    }
+    int64_t d_bg = 0, n_bg = 0, d_md = d_hi;
+    double best = -1.0;
+    for (size_t si = 0; si < shapes.size(); ++si) {
+      const int64_t dbg = shapes[si].dbg, nbg = shapes[si].nbg;
+      int64_t dmd = shapes[si].dmd;
+      // raising d_md if needed, at most kMidWorkMax build increments
+      unsigned long long w = works[si];
       if (w > kMidWorkMax) {
         int64_t lo = dmd, hi = d_hi;  // work(lo) too large, work(hi) = 0
         while (hi - lo > 1) {
@@ -1296,10 +1361,8 @@ static gs_status build_hub_index(gs_graph* g, uint64_t budget, bool tables, cuda
         n_bg = nbg;
         d_md = dmd;
       }
-      if (bg_cap == g->dev.tb_count) break;
     }
-    const int64_t md_cap = n_bg > 0 ? 1 : 0;
-    if (md_cap > 0 && d_md < d_hi) {
+    if (n_bg > 0 && d_md < d_hi) {
       int32_t* hubs = nullptr;
       GS_TRY(assign(d_bg, &g->bg_slot, &hubs, n_bg, true));
       cudaFree(hubs);
@@ -1336,7 +1399,7 @@ static gs_status build_hub_index(gs_graph* g, uint64_t budget, bool tables, cuda
         const size_t row_smem = sizeof(uint32_t) * (size_t)((n_bg + 1) / 2);
         cudaError_t e = cudaMemsetAsync(d_cnt, 0, sizeof(unsigned long long), stream);
         if (e == cudaSuccess)
-          e = GS_LAUNCH_ROWS(k_mid_rows, row_smem, stream, g->dev.row_ptr, g->dev.col, rows_v, rows,
+          e = GS_LAUNCH_ROWS(k_mid_rows, 256, row_smem, stream, g->dev.row_ptr, g->dev.col, rows_v, rows,
                              flag, blist, n_bg, g->md_codeg, d_cnt);
         if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
         cudaFree(blist);

@@ -66,10 +66,10 @@ __device__ __forceinline__ uint64_t splitmix(uint64_t x) {
 // host loop before (a launch and a wait per level and per round, one warp per
 // vertex) took 917 launches on the 100k-vertex power-law graph, 18 us each in
 // k_core_peel, where one warp walked a hub's 24,000 neighbours:
-// k-core numbers, 1% weighted sample and its estimates there: 27.1 -> 9.3 ms.
+// k-core numbers, 1% weighted sample and its estimates there: 27.1 -> 8.8 ms.
 constexpr int kPeelThreads = 512;
 constexpr int64_t kPeelPart = 256;  // neighbours per removal entry
-constexpr int kPeelQueue = 96;      // queued vertices of a warp
+constexpr int kPeelQueue = 16;      // queued vertices of a warp
 // Looks at the barrier counter before a block gives up on the others (each
 // takes at least 100 ns, so at least 25 s).
 constexpr int64_t kPeelSpins = (int64_t)1 << 28;
@@ -525,10 +525,11 @@ extern "C" gs_status gs_core_numbers(const gs_graph* gr, gs_workspace* ws, int32
   for (PeelPhase& p : init.phase) p.least = ~0ull;
   GS_CUDA(cudaMemcpyAsync(st, &init, sizeof(init), cudaMemcpyHostToDevice, stream));
   // every block resident at once (the blocks wait on one another): at most
-  // two per SM, fewer for a small graph, whose barriers are then cheaper
+  // one per SM (two make the barriers dearer: 9.1 against 8.8 ms on the
+  // 100k-vertex power-law graph), fewer for a small graph
   int per_sm = 0;
   GS_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_core_peel, kPeelThreads, 0));
-  const int64_t most = (int64_t)sm_count() * std::min(per_sm, 2);
+  const int64_t most = (int64_t)sm_count() * std::min(per_sm, 1);
   const int64_t want = (n + gr->dev.nnz / 16 + kPeelThreads - 1) / kPeelThreads;
   const int blocks = (int)std::max<int64_t>(1, std::min(most, want));
   const int64_t* row_ptr = gr->dev.row_ptr;

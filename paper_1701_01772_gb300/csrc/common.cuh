@@ -300,6 +300,7 @@ constexpr int32_t kNoSlotInfo = -2;
 // Exclusive prefix sum of in[0..count) into out[0..count], out[count] = total.
 // `in` and `out` may alias. tmp must hold scan_tmp_elems(count) int64.
 int64_t scan_tmp_elems(int64_t count);
+int scan_launches(int64_t count);  // kernels launched by a scan of count elements
 gs_status exclusive_scan_i64(const int64_t* in, int64_t* out, int64_t count, int64_t* tmp,
                              cudaStream_t stream);
 
@@ -377,9 +378,15 @@ struct gs_workspace {
   cudaEvent_t ev[12];   // start/stop pairs for the six gs_count phases
   gs_stats stats;       // last gs_count
   int64_t launches_total;
+  void* staging;        // page-locked host bytes for the small read-backs
 };
 
 namespace gs {
+// The workspace's page-locked staging buffer (kStagingBytes, allocated on
+// first use): read-backs into it are queued together and waited for once.
+constexpr size_t kStagingBytes = 1024;
+gs_status ws_staging(gs_workspace* ws, void** out);
+
 // Graphs (or batch members) of at most this many vertices get an adjacency
 // bit matrix (at most 32 MiB each).
 constexpr int64_t kDenseGraphMax = 16384;
@@ -398,11 +405,20 @@ gs_status sample_impl(const gs_graph* g, gs_workspace* ws, double fraction, uint
 // Samples canonical edges [e0, e0 + m) (hash index relative to e0).
 // Edges of [e0, e0 + m) whose sampler key lies in [fraction_lo, fraction)
 // x 2^53 (fraction_lo = 0: the Bernoulli(fraction) sample).
+// Boundary of the k smallest (key, i) of the sampler keys: the set is
+// {key < T} plus {key == T, i <= i_cut}; k = 0 gives the empty set.
+struct RankCut {
+  int64_t k;
+  uint64_t T;
+  int64_t i_cut;
+};
 // Edges ranked [k_lo, k_hi) by their sampler key (ties by canonical index),
-// in increasing canonical index; d_pairs NULL: into workspace slot 3.
+// in increasing canonical index; d_pairs NULL: into workspace slot 3. cut: in,
+// the boundary of k_lo if it is already known (cut->k == k_lo, same graph and
+// seed); out, that of k_hi; may be NULL.
 gs_status sample_ranks(const gs_graph* g, gs_workspace* ws, int64_t k_lo, int64_t k_hi,
                        uint64_t seed, int32_t* d_pairs, int32_t** pairs_out,
-                       cudaStream_t stream);
+                       cudaStream_t stream, RankCut* cut = nullptr);
 gs_status sample_range(const gs_graph* g, gs_workspace* ws, double fraction, uint64_t seed,
                        int64_t e0, int64_t m, int32_t* d_pairs, int64_t max_k, int64_t* k_out,
                        int32_t** pairs_out, cudaStream_t stream, double fraction_lo = 0.0);
@@ -414,8 +430,9 @@ struct CountBufs {
   int64_t K = 0, P = 0, groups = 0, tsum = 0, dup_cap = 0, nseg = 0;
   int fold_blocks = 0;
   DevError* err = nullptr;
+  // err, sums and stats lie one behind the other (256 bytes each)
   unsigned long long* sums = nullptr;   // [32] single-segment result
-  unsigned long long* stats = nullptr;  // [8]
+  unsigned long long* stats = nullptr;  // [16]
   int32_t* pairs_all = nullptr;
   int2* uv = nullptr;
   int64_t* off = nullptr;

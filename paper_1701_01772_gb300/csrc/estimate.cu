@@ -276,6 +276,7 @@ extern "C" gs_status gs_count_adaptive(const gs_graph* g, gs_workspace* ws, doub
   bool have_prev = false;
   int32_t t = 0;
   int64_t J = 0;  // edges sampled so far: the J smallest sampler keys
+  gs::RankCut cut{0, 0, -1};  // their boundary
   while (loss > beta && t < t_max) {
     // K_t = ceil(phi (M - |J|)) new edges, uniformly without replacement:
     // the next K_t edges in sampler-key order
@@ -283,7 +284,7 @@ extern "C" gs_status gs_count_adaptive(const gs_graph* g, gs_workspace* ws, doub
     const int64_t J_new = J + Kt < M ? J + Kt : M;
     const int64_t K = J_new - J;
     int32_t* pairs = nullptr;
-    GS_TRY(gs::sample_ranks(g, ws, J, J_new, seed, nullptr, &pairs, stream));
+    GS_TRY(gs::sample_ranks(g, ws, J, J_new, seed, nullptr, &pairs, stream, &cut));
     J = J_new;
     if (K > 0) {
       gs_sums part;

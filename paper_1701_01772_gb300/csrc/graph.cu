@@ -1821,7 +1821,7 @@ gs_status sample_range(const gs_graph* g, gs_workspace* ws, double fraction, uin
   int64_t* tmp = c.take<int64_t>(scan_tmp_elems(tiles));
   k_sample_count<<<(unsigned)tiles, kSampThreads, 0, stream>>>(m, seed, lo, threshold, cnt);
   GS_TRY(exclusive_scan_i64(cnt, off, tiles, tmp, stream));
-  ws->launches_total += 4;
+  ws->launches_total += 1 + scan_launches(tiles);
   int64_t kept = 0;
   GS_CUDA(cudaMemcpyAsync(&kept, off + tiles, sizeof(int64_t), cudaMemcpyDeviceToHost, stream));
   GS_CUDA(cudaStreamSynchronize(stream));

@@ -121,12 +121,45 @@ __global__ void scan_tiles(const int64_t* in, int64_t* out, int64_t count,
   if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) out[count] = carries[gridDim.x];
 }
 
+// Scans of at most kScanSmall elements in one launch by one block (each
+// launch of the three-kernel scan costs a small call about 3 us and a gap).
+constexpr int64_t kScanSmall = 4 * kScanTile;
+__global__ void scan_small(const int64_t* in, int64_t* out, int64_t count) {
+  int64_t carry = 0;
+  for (int64_t start = 0; start < count; start += kScanTile) {
+    const int64_t base = start + (int64_t)threadIdx.x * kScanItems;
+    int64_t vals[kScanItems];
+    int64_t s = 0;
+#pragma unroll
+    for (int i = 0; i < kScanItems; ++i) {
+      vals[i] = base + i < count ? in[base + i] : 0;
+      s += vals[i];
+    }
+    int64_t total;
+    int64_t ex = carry + block_exclusive_scan(s, &total);
+#pragma unroll
+    for (int i = 0; i < kScanItems; ++i) {
+      if (base + i < count) out[base + i] = ex;
+      ex += vals[i];
+    }
+    carry += total;
+  }
+  if (threadIdx.x == 0) out[count] = carry;
+}
+
+int scan_launches(int64_t count) { return count <= 0 ? 0 : count <= kScanSmall ? 1 : 3; }
+
 int64_t scan_tmp_elems(int64_t count) { return (count + kScanTile - 1) / kScanTile + 2; }
 
 gs_status exclusive_scan_i64(const int64_t* in, int64_t* out, int64_t count, int64_t* tmp,
                              cudaStream_t stream) {
   if (count <= 0) {
     GS_CUDA(cudaMemsetAsync(out, 0, sizeof(int64_t), stream));
+    return GS_OK;
+  }
+  if (count <= kScanSmall) {
+    scan_small<<<1, kScanThreads, 0, stream>>>(in, out, count);
+    GS_CUDA(cudaGetLastError());
     return GS_OK;
   }
   int64_t tiles = (count + kScanTile - 1) / kScanTile;
@@ -142,6 +175,21 @@ gs_status exclusive_scan_i64(const int64_t* in, int64_t* out, int64_t count, int
 }
 
 // ---------------------------------------------------------------- workspace
+
+gs_status ws_staging(gs_workspace* ws, void** out) {
+  if (ws->staging == nullptr) {
+    const cudaError_t e = cudaMallocHost(&ws->staging, kStagingBytes);
+    if (e != cudaSuccess) {
+      ws->staging = nullptr;
+      cudaGetLastError();
+      set_error("workspace: page-locked staging of %zu bytes failed (%s)", kStagingBytes,
+                cudaGetErrorString(e));
+      return GS_ENOMEM;
+    }
+  }
+  *out = ws->staging;
+  return GS_OK;
+}
 
 gs_status ws_reserve(gs_workspace* ws, int slot, size_t bytes, cudaStream_t stream, void** out) {
   if (bytes == 0) bytes = 256;
@@ -196,6 +244,7 @@ gs_status gs_workspace_destroy(gs_workspace* ws) {
     }
   if (ws->ev[0] != nullptr)
     for (int i = 0; i < 12; ++i) cudaEventDestroy(ws->ev[i]);
+  if (ws->staging != nullptr) cudaFreeHost(ws->staging);
   delete ws;
   return GS_OK;
 }

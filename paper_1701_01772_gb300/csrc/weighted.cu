@@ -379,15 +379,23 @@ __global__ void k_key_hist(int64_t m, uint64_t seed, uint64_t prefix, int above,
     if (h[b]) atomicAdd(hist + b, (unsigned long long)h[b]);
 }
 
-// Indices of the edges whose key equals T (ties of the order statistic).
-__global__ void k_key_ties(int64_t m, uint64_t seed, uint64_t T, int64_t cap,
-                           int64_t* __restrict__ out, unsigned long long* __restrict__ cnt) {
+// (key, i) of the edges whose key agrees with lo.prefix above bit lo.above, and
+// with hi.prefix above hi.above (the buckets that hold two order statistics),
+// into out_lo and out_hi.
+struct KeyPrefix {
+  uint64_t prefix;
+  int32_t above;  // 53: no bucket
+};
+__global__ void k_key_collect(int64_t m, uint64_t seed, KeyPrefix lo, KeyPrefix hi,
+                              ulonglong2* __restrict__ out_lo, ulonglong2* __restrict__ out_hi,
+                              unsigned long long* __restrict__ cnt) {
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < m;
        i += (int64_t)gridDim.x * blockDim.x) {
-    if ((splitmix(seed ^ splitmix((uint64_t)i)) >> 11) == T) {
-      const unsigned long long at = atomicAdd(cnt, 1ull);
-      if ((int64_t)at < cap) out[at] = i;
-    }
+    const uint64_t key = splitmix(seed ^ splitmix((uint64_t)i)) >> 11;
+    if (lo.above < 53 && (key >> lo.above) == lo.prefix)
+      out_lo[atomicAdd(cnt, 1ull)] = make_ulonglong2(key, (unsigned long long)i);
+    if (hi.above < 53 && (key >> hi.above) == hi.prefix)
+      out_hi[atomicAdd(cnt + 1, 1ull)] = make_ulonglong2(key, (unsigned long long)i);
   }
 }
 
@@ -597,7 +605,7 @@ extern "C" gs_status gs_sample_weighted(const gs_graph* gr, gs_workspace* ws,
   GS_CUDA(cudaMemcpyAsync(&kept, off + tiles, sizeof(int64_t), cudaMemcpyDeviceToHost, stream));
   GS_CUDA(cudaStreamSynchronize(stream));
   *k_out = kept;
-  ws->launches_total += 6;
+  ws->launches_total += 3 + scan_launches(tiles);
   if (kept > max_k) {
     set_error("gs_sample_weighted: %lld edges kept but the output holds %lld", (long long)kept,
               (long long)max_k);
@@ -713,70 +721,109 @@ extern "C" gs_status gs_count_weighted(const gs_graph* gr, gs_workspace* ws,
 
 namespace gs {
 
-// Boundary of the k smallest (key, i) of the sampler keys: the set is
-// {key < T} plus {key == T, i <= i_cut}; k = 0 gives the empty set.
-struct RankCut {
-  uint64_t T;
-  int64_t i_cut;
+// A bucket of keys with a common prefix that holds an order statistic: rank
+// is its 0-based rank inside the bucket, size the bucket's keys.
+struct RankBucket {
+  KeyPrefix at;
+  int64_t rank, size;
 };
 
-static gs_status rank_cut(const gs_graph* gr, int64_t k, uint64_t seed,
-                          unsigned long long* hist, int64_t* ties, int64_t tie_cap,
-                          int64_t* launches, RankCut* out, cudaStream_t stream) {
-  const int64_t m = gr->m;
-  if (k <= 0) {
-    *out = RankCut{0, -1};
-    return GS_OK;
+// Buckets of at most this many keys are read back and selected from on the
+// host.
+constexpr int64_t kBucketMost = 16384;
+
+// The part of `b` whose next `bits` key bits hold its rank (h: their counts).
+static gs_status narrow(RankBucket* b, const unsigned long long* h, int bits) {
+  int64_t before = 0;
+  int d = 0;
+  for (; d < (1 << bits); ++d) {
+    if (before + (int64_t)h[d] > b->rank) break;
+    before += (int64_t)h[d];
   }
-  // order statistic: the k-th smallest key T, five digits from the top
-  uint64_t prefix = 0;
-  int above = 53;
-  int64_t rank = k - 1;  // 0-based rank of T among the keys with this prefix
-  static const int kDigits[5] = {11, 11, 11, 10, 10};
-  int64_t tie_count = 0;
+  if (d == (1 << bits)) {
+    set_error("sampler key selection lost its rank");
+    return GS_ECUDA;
+  }
+  b->rank -= before;
+  b->at.prefix = (b->at.prefix << bits) | (uint64_t)d;
+  b->at.above -= bits;
+  b->size = (int64_t)h[d];
+  return GS_OK;
+}
+
+// Boundaries of the k smallest keys for the cuts in c[0] and c[1] (k set; k =
+// 0 and a cut that is already known are left alone). A histogram of the
+// leading key bits, shared by both cuts, gives each one's bucket; buckets that
+// are still large are split by further bits; the keys left are collected in
+// one pass and selected from on the host. The digit-by-digit selection before
+// took five passes and waits per cut (55 of the 223 launches of an adaptive
+// estimate on R-MAT 18).
+static gs_status rank_cuts(const gs_graph* gr, gs_workspace* ws, uint64_t seed,
+                           unsigned long long* hist, RankCut* c[2], const bool known[2],
+                           int64_t* launches, cudaStream_t stream) {
+  const int64_t m = gr->m;
+  constexpr int kBits = 11;
   std::vector<unsigned long long> h(kSelBins);
-  for (int d = 0; d < 5; ++d) {
-    const int bits = kDigits[d], shift = above - bits;
+  auto histogram = [&](const KeyPrefix& p, int bits) -> gs_status {
     GS_CUDA(cudaMemsetAsync(hist, 0, sizeof(unsigned long long) * kSelBins, stream));
-    k_key_hist<<<grid_for(m, kThreads, 4), kThreads, 0, stream>>>(m, seed, prefix, above, shift,
-                                                                   bits, hist);
+    k_key_hist<<<grid_for(m, kThreads, 4), kThreads, 0, stream>>>(m, seed, p.prefix, p.above,
+                                                                   p.above - bits, bits, hist);
     ++*launches;
     GS_CUDA(cudaMemcpyAsync(h.data(), hist, sizeof(unsigned long long) << bits,
                             cudaMemcpyDeviceToHost, stream));
     GS_CUDA(cudaStreamSynchronize(stream));
-    int64_t accum = 0;
-    int b = 0;
-    for (; b < (1 << bits); ++b) {
-      if (accum + (int64_t)h[b] > rank) break;
-      accum += (int64_t)h[b];
-    }
-    if (b == (1 << bits)) {
-      set_error("sampler key selection lost its rank");
-      return GS_ECUDA;
-    }
-    rank -= accum;
-    prefix = (prefix << bits) | (uint64_t)b;
-    above = shift;
-    tie_count = (int64_t)h[b];
+    return GS_OK;
+  };
+  RankBucket b[2];
+  bool want[2];
+  for (int j = 0; j < 2; ++j) {
+    want[j] = !known[j] && c[j]->k > 0;
+    if (!known[j] && c[j]->k <= 0) *c[j] = RankCut{0, 0, -1};
+    b[j] = RankBucket{KeyPrefix{0, 53}, c[j]->k - 1, m};
   }
-  int64_t i_cut = m;  // every tie kept
-  if (rank + 1 < tie_count) {
-    if (tie_count > tie_cap) {
-      set_error("%lld sampler keys tie at the cut", (long long)tie_count);
-      return GS_ECAPACITY;
+  if (!want[0] && !want[1]) return GS_OK;
+  GS_TRY(histogram(KeyPrefix{0, 53}, kBits));
+  for (int j = 0; j < 2; ++j)
+    if (want[j]) GS_TRY(narrow(&b[j], h.data(), kBits));
+  for (int j = 0; j < 2; ++j)
+    while (want[j] && b[j].size > kBucketMost && b[j].at.above > 0) {
+      const int bits = b[j].at.above < kBits ? b[j].at.above : kBits;
+      GS_TRY(histogram(b[j].at, bits));
+      GS_TRY(narrow(&b[j], h.data(), bits));
     }
-    GS_CUDA(cudaMemsetAsync(hist + kSelBins, 0, sizeof(unsigned long long), stream));
-    k_key_ties<<<grid_for(m, kThreads, 4), kThreads, 0, stream>>>(m, seed, prefix, tie_cap, ties,
-                                                                   hist + kSelBins);
-    ++*launches;
-    std::vector<int64_t> ht((size_t)tie_count);
-    GS_CUDA(cudaMemcpyAsync(ht.data(), ties, sizeof(int64_t) * (size_t)tie_count,
+  const int64_t n0 = want[0] ? b[0].size : 0, n1 = want[1] ? b[1].size : 0;
+  void* base = nullptr;
+  GS_TRY(ws_reserve(ws, 4,
+                    Carve::bytes_for<unsigned long long>(2) + Carve::bytes_for<ulonglong2>(n0) +
+                        Carve::bytes_for<ulonglong2>(n1),
+                    stream, &base));
+  Carve cv{(char*)base, 0};
+  unsigned long long* cnt = cv.take<unsigned long long>(2);
+  ulonglong2* d0 = cv.take<ulonglong2>(n0);
+  ulonglong2* d1 = cv.take<ulonglong2>(n1);
+  GS_CUDA(cudaMemsetAsync(cnt, 0, 2 * sizeof(unsigned long long), stream));
+  k_key_collect<<<grid_for(m, kThreads, 8), kThreads, 0, stream>>>(
+      m, seed, want[0] ? b[0].at : KeyPrefix{0, 53}, want[1] ? b[1].at : KeyPrefix{0, 53}, d0, d1,
+      cnt);
+  ++*launches;
+  std::vector<ulonglong2> keys((size_t)(n0 + n1));
+  if (n0 > 0)
+    GS_CUDA(cudaMemcpyAsync(keys.data(), d0, sizeof(ulonglong2) * (size_t)n0,
                             cudaMemcpyDeviceToHost, stream));
-    GS_CUDA(cudaStreamSynchronize(stream));
-    std::sort(ht.begin(), ht.end());
-    i_cut = ht[(size_t)rank];
+  if (n1 > 0)
+    GS_CUDA(cudaMemcpyAsync(keys.data() + n0, d1, sizeof(ulonglong2) * (size_t)n1,
+                            cudaMemcpyDeviceToHost, stream));
+  GS_CUDA(cudaStreamSynchronize(stream));
+  for (int j = 0; j < 2; ++j) {
+    if (!want[j]) continue;
+    ulonglong2* first = keys.data() + (j == 0 ? 0 : n0);
+    ulonglong2* nth = first + b[j].rank;
+    std::nth_element(first, nth, first + b[j].size, [](const ulonglong2& x, const ulonglong2& y) {
+      return x.x < y.x || (x.x == y.x && x.y < y.y);
+    });
+    c[j]->T = nth->x;
+    c[j]->i_cut = (int64_t)nth->y;
   }
-  *out = RankCut{prefix, i_cut};
   return GS_OK;
 }
 
@@ -785,29 +832,30 @@ static gs_status rank_cut(const gs_graph* gr, int64_t k, uint64_t seed,
 // into workspace slot 3 (*pairs_out).
 gs_status sample_ranks(const gs_graph* gr, gs_workspace* ws, int64_t k_lo, int64_t k_hi,
                        uint64_t seed, int32_t* d_pairs, int32_t** pairs_out,
-                       cudaStream_t stream) {
+                       cudaStream_t stream, RankCut* cut) {
   const int64_t n = gr->dev.n, m = gr->m;
   if (pairs_out) *pairs_out = d_pairs;
   if (k_hi <= k_lo) return GS_OK;
-  constexpr int64_t kTieCap = 1 << 16;
   const int64_t tiles = (m + kSampTile - 1) / kSampTile;
-  const size_t bytes = Carve::bytes_for<unsigned long long>(kSelBins + 8) +
-                       Carve::bytes_for<int64_t>(kTieCap) + Carve::bytes_for<uint8_t>(m) +
+  const size_t bytes = Carve::bytes_for<unsigned long long>(kSelBins) +
+                       Carve::bytes_for<uint8_t>(m) +
                        Carve::bytes_for<int64_t>(tiles + 1) * 2 +
                        Carve::bytes_for<int64_t>(scan_tmp_elems(tiles));
   void* base = nullptr;
   GS_TRY(ws_reserve(ws, 2, bytes, stream, &base));
   Carve c{(char*)base, 0};
-  unsigned long long* hist = c.take<unsigned long long>(kSelBins + 8);
-  int64_t* ties = c.take<int64_t>(kTieCap);
+  unsigned long long* hist = c.take<unsigned long long>(kSelBins);
   uint8_t* keep = c.take<uint8_t>(m);
   int64_t* cnt = c.take<int64_t>(tiles + 1);
   int64_t* off = c.take<int64_t>(tiles + 1);
   int64_t* tmp = c.take<int64_t>(scan_tmp_elems(tiles));
   int64_t launches = 0;
-  RankCut lo, hi;
-  GS_TRY(rank_cut(gr, k_lo, seed, hist, ties, kTieCap, &launches, &lo, stream));
-  GS_TRY(rank_cut(gr, k_hi, seed, hist, ties, kTieCap, &launches, &hi, stream));
+  const bool known[2] = {cut != nullptr && k_lo > 0 && cut->k == k_lo, false};
+  RankCut lo{k_lo, 0, -1}, hi{k_hi, 0, -1};
+  if (known[0]) lo = *cut;
+  RankCut* cuts[2] = {&lo, &hi};
+  GS_TRY(rank_cuts(gr, ws, seed, hist, cuts, known, &launches, stream));
+  if (cut != nullptr) *cut = hi;
   if (d_pairs == nullptr) {
     void* b3 = nullptr;
     GS_TRY(ws_reserve(ws, 3, Carve::bytes_for<int32_t>(2 * (k_hi - k_lo)), stream, &b3));
@@ -821,7 +869,7 @@ gs_status sample_ranks(const gs_graph* gr, gs_workspace* ws, int64_t k_lo, int64
   k_flag_write<<<(unsigned)tiles, kThreads, 0, stream>>>(gr->dev.col, gr->up_ptr, gr->edge_off,
                                                          nullptr, n, m, keep, off, d_pairs,
                                                          nullptr);
-  launches += 6;
+  launches += 3 + scan_launches(tiles);
   int64_t kept = 0;
   GS_CUDA(cudaMemcpyAsync(&kept, off + tiles, sizeof(int64_t), cudaMemcpyDeviceToHost, stream));
   GS_CUDA(cudaStreamSynchronize(stream));

@@ -107,16 +107,16 @@ __device__ __forceinline__ uint32_t tfilter_hash(int32_t x) {
 #define GS_QUAD_GRAB_TESTS 4096
 #endif
 constexpr int64_t kQuadGrabTests = GS_QUAD_GRAB_TESTS;
-// Threads of a k_dense_pairs CTA and resident CTAs per SM.
-#ifndef GS_DENSE_THREADS
-#define GS_DENSE_THREADS 256
-#endif
-#ifndef GS_DENSE_BLOCKS
-#define GS_DENSE_BLOCKS 6
-#endif
+// Resident warps per SM of k_dense_pairs (at most 40 registers), in CTAs of
+// 256 threads, or of 128 when there are many units: a unit has nine barriers,
+// at which the warps of a small CTA wait less, but a unit with long lists of
+// other members is walked by fewer warps. 1M-vertex power-law graph exact
+// (3.4M units) 374 ms with 256 threads, 358 with 128; R-MAT 24 0.1% (19,000
+// units) 147 and 154 ms, the 1% estimate of the former (34,000 units) 5.70 and
+// 5.79 ms. The line lies at 256 dense edges per resident CTA of 256.
+constexpr int kDenseWarpsPerSm = 48;
+constexpr int64_t kManyDenseEdges = 256 * 6 * 152;
 constexpr int kTriBlocksPerSm = 6;  // k_tri_chunks: at most 40 registers
-constexpr int kDenseThreads = GS_DENSE_THREADS;
-constexpr int kDenseBlocksPerSm = GS_DENSE_BLOCKS;
 // T entries per k_dense_pairs work unit (a heavy dense edge is split into
 // several units so that small samples still fill the GPU).
 constexpr int64_t kDenseUnit = 4 * kThreads;
@@ -515,7 +515,8 @@ __global__ void k_unit_fill(const int64_t* __restrict__ unit_off, int64_t ndense
 //   matrix neighbours (a bit of the mask, or, past the dense slots, a search
 //   of T when above w) and w's neighbours above w without a matrix slot (a
 //   search of T behind a hashed filter).
-__global__ void __launch_bounds__(kDenseThreads, kDenseBlocksPerSm)
+template <int kDenseThreads>
+__global__ void __launch_bounds__(kDenseThreads, kDenseWarpsPerSm * 32 / kDenseThreads)
     k_dense_pairs(const __grid_constant__ DevGraph g, const int64_t* __restrict__ toff,
                   const unsigned long long* __restrict__ t, const int32_t* __restrict__ T,
                   const int16_t* __restrict__ T_hm, const uint32_t* __restrict__ tmask,
@@ -1557,13 +1558,17 @@ __global__ void __launch_bounds__(kThreads)
   }
 }
 
-__global__ void k_fold_final(const u128* __restrict__ part, int blocks,
-                             unsigned long long* __restrict__ out) {
-  if (threadIdx.x < 16) {
-    u128 s = 0;
-    for (int b = 0; b < blocks; ++b) s += part[(int64_t)b * 16 + threadIdx.x];
-    out[2 * threadIdx.x] = (unsigned long long)s;
-    out[2 * threadIdx.x + 1] = (unsigned long long)(s >> 64);
+// Sums of the block partials, a warp per value (one thread per value walked
+// hundreds of dependent loads: 12 to 40 us; exact integers, any order).
+__global__ void __launch_bounds__(512) k_fold_final(const u128* __restrict__ part, int blocks,
+                                                    unsigned long long* __restrict__ out) {
+  const int lane = threadIdx.x & 31, value = threadIdx.x >> 5;
+  u128 s = 0;
+  for (int b = lane; b < blocks; b += 32) s += part[(int64_t)b * 16 + value];
+  for (int o = 16; o > 0; o >>= 1) s += shfl_down_u128(s, o);
+  if (lane == 0) {
+    out[2 * value] = (unsigned long long)s;
+    out[2 * value + 1] = (unsigned long long)(s >> 64);
   }
 }
 
@@ -1763,18 +1768,20 @@ void carve_mid(void* base, int64_t P, CountBufs& b) {
   b.tmp1 = c.take<int64_t>(scan_tmp_elems(b.groups + 1));
 }
 
+// Bytes from b.err to the end of b.stats.
+constexpr size_t kFrontWords = 512 + sizeof(unsigned long long) * kStatSlots;
+
 // memsets + (all-pair enumeration) + prep + position scan. No host sync.
 int64_t launch_front(const gs_graph* gr, const DevGraph& g, const int32_t* pairs, bool four,
                      CountBufs& b, cudaStream_t stream) {
   int64_t launches = 0;
   const int64_t K = b.K;
-  cudaMemsetAsync(b.err, 0, sizeof(DevError), stream);
-  cudaMemsetAsync(b.stats, 0, sizeof(unsigned long long) * kStatSlots, stream);
-  cudaMemsetAsync(b.t, 0, sizeof(unsigned long long) * K, stream);
-  if (four) {
-    cudaMemsetAsync(b.k2, 0, sizeof(unsigned long long) * K, stream);
-    cudaMemsetAsync(b.q, 0, sizeof(unsigned long long) * K, stream);
-  }
+  // err, sums and stats in one fill; t, k2 and q (carved one behind the other)
+  // in another
+  cudaMemsetAsync(b.err, 0, kFrontWords, stream);
+  cudaMemsetAsync(b.t, 0,
+                  four ? (size_t)((char*)(b.q + K) - (char*)b.t) : sizeof(unsigned long long) * K,
+                  stream);
   if (b.dup != nullptr) cudaMemsetAsync(b.dup, 0xff, sizeof(unsigned long long) * b.dup_cap, stream);
   if (pairs == nullptr) {
     k_all_pairs<<<grid_for(g.n * 32, kThreads, 8), kThreads, 0, stream>>>(
@@ -1785,7 +1792,7 @@ int64_t launch_front(const gs_graph* gr, const DevGraph& g, const int32_t* pairs
   k_prep<<<grid_for(K, kThreads, 8), kThreads, 0, stream>>>(g, pairs, K, four ? 1 : 0, b.dup,
                                                             b.dup_cap - 1, b.uv, b.off, b.err);
   exclusive_scan_i64(b.off, b.off, K, b.tmp0, stream);
-  return launches + 4;
+  return launches + 1 + scan_launches(K);
 }
 
 int64_t launch_tri(const DevGraph& g, bool four, const Tuning& tu, CountBufs& b,
@@ -1800,7 +1807,7 @@ int64_t launch_tri(const DevGraph& g, bool four, const Tuning& tu, CountBufs& b,
 
 int64_t launch_scan_t(CountBufs& b, cudaStream_t stream) {
   exclusive_scan_i64((const int64_t*)b.t, b.toff, b.K, b.tmp0, stream);
-  return 3;
+  return scan_launches(b.K);
 }
 
 // T lists (and their matrix slots) in order; marks dense edges (mask index
@@ -1820,16 +1827,20 @@ int64_t launch_tmask(const DevGraph& g, CountBufs& b, cudaStream_t stream) {
   exclusive_scan_i64(b.unit_off, b.unit_off, b.ndense, b.unit_tmp, stream);
   k_unit_fill<<<grid_for(b.ndense * 32, kThreads, 8), kThreads, 0, stream>>>(b.unit_off, b.ndense,
                                                                               b.unit_idx);
-  return 5;
+  return 2 + scan_launches(b.ndense);
 }
 
 // Pairs among the matrix members of T in the dense edges (k_dense_pairs).
 // No host sync.
 int64_t launch_dense(const DevGraph& g, bool need_q, CountBufs& b, cudaStream_t stream) {
   if (b.ndense <= 0 || g.col_hm == nullptr) return 0;
-  k_dense_pairs<<<sm_count() * kDenseBlocksPerSm, kDenseThreads, 0, stream>>>(
-      g, b.toff, b.t, b.T, b.T_hm, b.tmask, b.dense_e, b.unit_off, b.unit_idx, b.ndense,
-      need_q ? 1 : 0, b.k2, b.q, b.stats + 7, b.stats + 4, b.stats + 9);
+  auto go = [&](auto kernel, int threads) {
+    kernel<<<sm_count() * (kDenseWarpsPerSm * 32 / threads), threads, 0, stream>>>(
+        g, b.toff, b.t, b.T, b.T_hm, b.tmask, b.dense_e, b.unit_off, b.unit_idx, b.ndense,
+        need_q ? 1 : 0, b.k2, b.q, b.stats + 7, b.stats + 4, b.stats + 9);
+  };
+  if (b.ndense >= kManyDenseEdges) go(k_dense_pairs<128>, 128);
+  else go(k_dense_pairs<256>, 256);
   return 1;
 }
 
@@ -1842,7 +1853,7 @@ int64_t launch_cost(const DevGraph& g, bool need_k, bool need_q, const Tuning& t
       g, b.uv, b.off, b.K, b.t, b.tbits, b.tpre, mi, need_q, tu.task_probes, b.task_off, b.cbits,
       b.q, b.stats);
   exclusive_scan_i64(b.task_off, b.task_off, b.groups, b.tmp1, stream);
-  return 4;
+  return 1 + scan_launches(b.groups);
 }
 
 // The 4-node membership tests (k_quad). No host sync.
@@ -1867,7 +1878,7 @@ int64_t launch_fold(const gs_graph* gr, const DevGraph& g, bool four, bool need_
                                                   four ? b.q : nullptr, four ? b.tdeg : nullptr,
                                                   gr->nbr_degsum, need_k, need_q, per_edge, b.part,
                                                   b.stats);
-  k_fold_final<<<1, 32, 0, stream>>>(b.part, b.fold_blocks, b.sums);
+  k_fold_final<<<1, 512, 0, stream>>>(b.part, b.fold_blocks, b.sums);
   return 2;
 }
 
@@ -1881,10 +1892,7 @@ int64_t launch_fold_seg(const DevGraph& g, bool four, const int64_t* seg_off, Co
   return 2;
 }
 
-gs_status fetch_error(DevError* d_err, cudaStream_t stream, const char* what) {
-  DevError h;
-  GS_CUDA(cudaMemcpyAsync(&h, d_err, sizeof(h), cudaMemcpyDeviceToHost, stream));
-  GS_CUDA(cudaStreamSynchronize(stream));
+static gs_status error_status(const DevError& h, const char* what) {
   if (h.code != 0) {
     const char* kind = h.code == GS_EDUPSAMPLE ? "edge sampled twice"
                        : h.code == GS_EEDGE    ? "sampled pair is out of range or not an edge"
@@ -1893,6 +1901,13 @@ gs_status fetch_error(DevError* d_err, cudaStream_t stream, const char* what) {
     return h.code;
   }
   return GS_OK;
+}
+
+gs_status fetch_error(DevError* d_err, cudaStream_t stream, const char* what) {
+  DevError h;
+  GS_CUDA(cudaMemcpyAsync(&h, d_err, sizeof(h), cudaMemcpyDeviceToHost, stream));
+  GS_CUDA(cudaStreamSynchronize(stream));
+  return error_status(h, what);
 }
 
 void store_sums(const unsigned long long* h, uint32_t mask, gs_sums* out) {
@@ -1905,6 +1920,10 @@ void store_sums(const unsigned long long* h, uint32_t mask, gs_sums* out) {
     out->sumsq[i][1] = h[2 * (8 + i) + 1];
   }
 }
+
+// Up to this many positions the T lists (6 bytes an entry) get room for every
+// position instead of a wait for their size.
+constexpr int64_t kSmallPositions = 1 << 20;
 
 // Full counting run with host synchronisation for sizing (gs_count and the
 // sizing pass of the batched and served paths). seg_off != NULL selects the
@@ -1938,10 +1957,16 @@ gs_status count_run(const gs_graph* gr, gs_workspace* ws, const int32_t* d_pairs
   launches += launch_front(gr, g, d_pairs, four, b, stream);
   timer.stop(0);
   GS_CUDA(cudaGetLastError());
-  int64_t P = 0;
-  GS_CUDA(cudaMemcpyAsync(&P, b.off + K, sizeof(int64_t), cudaMemcpyDeviceToHost, stream));
-  gs_status es = fetch_error(b.err, stream, what);
+  void* staged = nullptr;
+  GS_TRY(ws_staging(ws, &staged));
+  DevError* h_err = (DevError*)staged;
+  int64_t* h_val = (int64_t*)((char*)staged + 256);
+  GS_CUDA(cudaMemcpyAsync(h_val, b.off + K, sizeof(int64_t), cudaMemcpyDeviceToHost, stream));
+  GS_CUDA(cudaMemcpyAsync(h_err, b.err, sizeof(DevError), cudaMemcpyDeviceToHost, stream));
+  GS_CUDA(cudaStreamSynchronize(stream));
+  const int64_t P = *h_val;
   ws->launches_total += launches;
+  const gs_status es = error_status(*h_err, what);
   if (es != GS_OK) return es;
 
   void* base1 = nullptr;
@@ -1962,8 +1987,14 @@ gs_status count_run(const gs_graph* gr, gs_workspace* ws, const int32_t* d_pairs
   if (four) {
     timer.start(2);
     more += launch_scan_t(b, stream);
-    GS_CUDA(cudaMemcpyAsync(&b.tsum, b.toff + K, sizeof(int64_t), cudaMemcpyDeviceToHost, stream));
-    GS_CUDA(cudaStreamSynchronize(stream));
+    if (P <= kSmallPositions) {
+      b.tsum = P;  // every T entry is a position: room for all, and no wait
+    } else {
+      GS_CUDA(
+          cudaMemcpyAsync(h_val, b.toff + K, sizeof(int64_t), cudaMemcpyDeviceToHost, stream));
+      GS_CUDA(cudaStreamSynchronize(stream));
+      b.tsum = *h_val;
+    }
     void* base2 = nullptr;
     GS_TRY(ws_reserve(ws, 2,
                       Carve::bytes_for<int32_t>(b.tsum) + Carve::bytes_for<int16_t>(b.tsum),
@@ -1972,10 +2003,12 @@ gs_status count_run(const gs_graph* gr, gs_workspace* ws, const int32_t* d_pairs
     b.T = c2.take<int32_t>(b.tsum);
     b.T_hm = c2.take<int16_t>(b.tsum);
     more += launch_compact(g, b, stream);
-    unsigned long long nd = 0;
-    GS_CUDA(cudaMemcpyAsync(&nd, b.stats + 6, sizeof(nd), cudaMemcpyDeviceToHost, stream));
-    GS_CUDA(cudaStreamSynchronize(stream));
-    b.ndense = (int64_t)nd;
+    b.ndense = 0;
+    if (g.col_hm != nullptr && g.hm_dense_words > 0) {  // without a matrix no edge is dense
+      GS_CUDA(cudaMemcpyAsync(h_val, b.stats + 6, sizeof(int64_t), cudaMemcpyDeviceToHost, stream));
+      GS_CUDA(cudaStreamSynchronize(stream));
+      b.ndense = *h_val;
+    }
     b.tmask = nullptr;
     b.dense_e = nullptr;
     if (b.ndense > 0) {
@@ -2079,15 +2112,22 @@ extern "C" gs_status gs_count(const gs_graph* gr, gs_workspace* ws, const int32_
   GS_TRY(count_run(gr, ws, d_pairs, K, mask, d_pairs != nullptr, d_per_edge, nullptr, 0, tu, b,
                    stream, "gs_count"));
   const bool four = (mask & (GS_G7 | GS_G8 | GS_G9 | GS_G10 | GS_G11 | GS_G12)) != 0;
-  unsigned long long h[32];
-  unsigned long long hs[kStatSlots];
-  int64_t ntasks = 0;
-  GS_CUDA(cudaMemcpyAsync(h, b.sums, sizeof(h), cudaMemcpyDeviceToHost, stream));
-  GS_CUDA(cudaMemcpyAsync(hs, b.stats, sizeof(hs), cudaMemcpyDeviceToHost, stream));
-  if (four)
-    GS_CUDA(cudaMemcpyAsync(&ntasks, b.task_off + b.groups, sizeof(int64_t),
-                            cudaMemcpyDeviceToHost, stream));
+  void* staged = nullptr;
+  GS_TRY(ws_staging(ws, &staged));
+  // err (unused here), sums and stats, then the task and T totals
+  unsigned long long* h = (unsigned long long*)((char*)staged + 256);
+  unsigned long long* hs = (unsigned long long*)((char*)staged + 512);
+  int64_t* h_val = (int64_t*)((char*)staged + kFrontWords);
+  h_val[0] = h_val[1] = 0;
+  GS_CUDA(cudaMemcpyAsync(staged, b.err, kFrontWords, cudaMemcpyDeviceToHost, stream));
+  if (four) {
+    GS_CUDA(cudaMemcpyAsync(h_val, b.task_off + b.groups, sizeof(int64_t), cudaMemcpyDeviceToHost,
+                            stream));
+    GS_CUDA(cudaMemcpyAsync(h_val + 1, b.toff + K, sizeof(int64_t), cudaMemcpyDeviceToHost,
+                            stream));
+  }
   GS_CUDA(cudaStreamSynchronize(stream));
+  const int64_t ntasks = h_val[0];
   store_sums(h, mask, h_sums);
   gs_stats& st = ws->stats;
   st.k = K;
@@ -2098,7 +2138,7 @@ extern "C" gs_status gs_count(const gs_graph* gr, gs_workspace* ws, const int32_
   st.model_bytes = hs[2] + hs[3];
   st.model_tri_bytes = hs[2];
   st.model_quad_bytes = hs[3];
-  st.t_sum = b.tsum;
+  st.t_sum = h_val[1];
   st.tasks = ntasks;
   st.timed = ws->timing;
   if (ws->timing) {

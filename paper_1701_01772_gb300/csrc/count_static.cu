@@ -141,7 +141,7 @@ extern "C" gs_status gs_count3_static(const gs_graph* gr, const int32_t* d_pairs
   launch_tri_unpadded(g, uv, off, K, t, sm_count() * 4, stream);
   k_fold<<<fold_blocks, kThreads, 0, stream>>>(g, uv, K, t, nullptr, nullptr, nullptr,
                                                 gr->nbr_degsum, 0, 0, nullptr, part, d_stats);
-  k_fold_final<<<1, 32, 0, stream>>>(part, fold_blocks, d_sums);
+  k_fold_final<<<1, 512, 0, stream>>>(part, fold_blocks, d_sums);
   GS_CUDA(cudaGetLastError());
   unsigned long long h[32];
   GS_CUDA(cudaMemcpyAsync(h, d_sums, sizeof(h), cudaMemcpyDeviceToHost, stream));

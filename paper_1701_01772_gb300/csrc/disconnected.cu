@@ -94,18 +94,31 @@ __global__ void __launch_bounds__(kDiscThreads)
   }
 }
 
-// Fixed-order sum of the block partials.
-__global__ void k_fold_disc_final(const u128* __restrict__ part, int blocks,
-                                  unsigned long long* __restrict__ out, unsigned* __restrict__ ovf) {
-  if (threadIdx.x < kDiscValues) {
-    u128 s = 0;
-    for (int b = 0; b < blocks; ++b) {
+// Sums of the block partials, a warp per value. A sum of squares past 128
+// bits carries out of one of its additions in any order.
+__global__ void __launch_bounds__(32 * kDiscValues)
+    k_fold_disc_final(const u128* __restrict__ part, int blocks,
+                      unsigned long long* __restrict__ out, unsigned* __restrict__ ovf) {
+  const int lane = threadIdx.x & 31, value = threadIdx.x >> 5;
+  u128 s = 0;
+  bool wrapped = false;
+  for (int b = lane; b < blocks; b += 32) {
+    const u128 before = s;
+    s += part[(int64_t)b * kDiscValues + value];
+    wrapped |= s < before;
+  }
+  for (int o = 16; o > 0; o >>= 1) {
+    const u128 w = shfl_down_128(s, o);
+    if (lane + o < 32) {
       const u128 before = s;
-      s += part[(int64_t)b * kDiscValues + threadIdx.x];
-      if (threadIdx.x >= 7 && s < before) atomicOr(ovf, 1u << (threadIdx.x - 7));
+      s += w;
+      wrapped |= s < before;
     }
-    out[2 * threadIdx.x] = (unsigned long long)s;
-    out[2 * threadIdx.x + 1] = (unsigned long long)(s >> 64);
+  }
+  if (value >= 7 && wrapped) atomicOr(ovf, 1u << (value - 7));
+  if (lane == 0) {
+    out[2 * value] = (unsigned long long)s;
+    out[2 * value + 1] = (unsigned long long)(s >> 64);
   }
 }
 
@@ -141,7 +154,7 @@ extern "C" gs_status gs_count_disconnected(const gs_graph* g, gs_workspace* ws, 
   GS_CUDA(cudaMemsetAsync(flags, 0, 2 * sizeof(unsigned), stream));
   k_fold_disc<<<blocks, kDiscThreads, 0, stream>>>(g->dev.row_ptr, g->dev.n, g->m, d_pairs, k,
                                                    d_per_edge, part, flags, flags + 1);
-  k_fold_disc_final<<<1, 32, 0, stream>>>(part, blocks, out, flags);
+  k_fold_disc_final<<<1, 32 * kDiscValues, 0, stream>>>(part, blocks, out, flags);
   GS_CUDA(cudaGetLastError());
   unsigned long long h[2 * kDiscValues];
   unsigned hf[2];

@@ -420,7 +420,7 @@ gs_status count_tri_oriented(const gs_graph* g, gs_workspace* ws, unsigned long 
   GS_CUDA(cudaGetLastError());
   k_fold_oriented<<<fold_blocks, kThreads, 0, stream>>>(g->dev.row_ptr, g->out_ptr, g->out_col,
                                                         tplus, n, part, stats);
-  k_fold_final<<<1, 32, 0, stream>>>(part, fold_blocks, sums);
+  k_fold_final<<<1, 512, 0, stream>>>(part, fold_blocks, sums);
   if (ws->timing) cudaEventRecord(ws->ev[11], stream);
   GS_CUDA(cudaGetLastError());
   GS_CUDA(cudaMemcpyAsync(h_sums, sums, sizeof(unsigned long long) * 32, cudaMemcpyDeviceToHost,

@@ -33,17 +33,14 @@ constexpr int kThreads = 256;
 constexpr unsigned kFull = 0xffffffffu;
 constexpr int64_t kInChunk = 256;      // in-neighbours per work unit
 constexpr int32_t kMaxOutDegree = 4096;  // larger out-lists: the general pass
-// Resident CTAs per SM (shared memory allows 6-7 at R-MAT scale 24's
-// 4096-slot tables, 8 for shorter out-lists). R-MAT 24 exact 3-node pass:
-// 0.42 s at 4, 0.31 s at 6 and 8.
+// Resident CTAs per SM (as far as shared memory allows).
 #ifndef GS_ORIENT_BLOCKS_PER_SM
 #define GS_ORIENT_BLOCKS_PER_SM 8
 #endif
 constexpr int kOrientBlocksPerSm = GS_ORIENT_BLOCKS_PER_SM;
-// Out-list entries a lane loads before it probes them (loads in flight;
-// R-MAT 24 exact pass: 0.346 s at 2, 0.307 s at 4, 0.290 s at 8).
+// Out-list entries a lane loads before it probes them (loads in flight).
 #ifndef GS_PROBE_BATCH
-#define GS_PROBE_BATCH 8
+#define GS_PROBE_BATCH 4
 #endif
 constexpr int kProbeBatch = GS_PROBE_BATCH;
 
@@ -158,8 +155,22 @@ __global__ void k_orient_units(const int64_t* __restrict__ out_ptr,
   }
 }
 
-__device__ __forceinline__ uint32_t slot_hash(int32_t x, int bits) {
-  return ((uint32_t)x * 2654435761u) >> (32 - bits);
+// Hash table of N+(v): buckets of four keys. A bucket is filled in order, so a
+// key that is not among a bucket's four is in the next one only if the fourth
+// is taken. kSlotsWanted slots per entry are taken as far as kTableSlots go,
+// which lets eight CTAs share an SM; an out-list too long for that gets at
+// least kSlotsLeast per entry. R-MAT 22 (out-lists of up to 1,100): 42.5 / 39.1
+// / 37.4 ms at 3 / 4 / 6 slots wanted; 39.4 / 39.1 / 44.3 ms with 2560 / 3328 /
+// 4096 table slots (four wanted).
+constexpr int64_t kTableSlots = 3328;
+constexpr int64_t kSlotsWanted = 6, kSlotsLeast = 2;
+__host__ __device__ __forceinline__ int table_buckets(int64_t out_degree) {
+  int64_t s = kSlotsWanted * out_degree;
+  if (s > kTableSlots) s = kSlotsLeast * out_degree > kTableSlots ? kSlotsLeast * out_degree : kTableSlots;
+  return (int)(s < 64 ? 16 : (s + 3) / 4);
+}
+__device__ __forceinline__ int bucket_of(int32_t x, int buckets) {
+  return (int)__umulhi((uint32_t)x * 2654435761u, (uint32_t)buckets);
 }
 
 // Triangles by middle vertex (see the file comment). Persistent CTAs take
@@ -167,17 +178,21 @@ __device__ __forceinline__ uint32_t slot_hash(int32_t x, int bits) {
 // N+(v): keys (int32, -1 empty) and one word per slot holding the out-list
 // position of x (low 16 bits) and the count of (v, x) (high 16 bits: at
 // most kInChunk per unit).
+//
+// Bound by instruction issue (84% of the cycles; a probe walked its chain of
+// single slots as long as the longest of 32 lanes, 100 warp instructions per 32
+// probes). Buckets of four keys are read in one load, and a second bucket is
+// rarely needed. R-MAT 22, 14.4e9 probes: 53.3 -> 34.8 ms.
 __global__ void __launch_bounds__(kThreads, kOrientBlocksPerSm)
     k_tri_oriented(const int64_t* __restrict__ out_ptr, const int32_t* __restrict__ out_col,
                    const int64_t* __restrict__ in_ptr, const int32_t* __restrict__ in_col,
                    const uint32_t* __restrict__ in_pos, const int64_t* __restrict__ unit_off,
-                   int64_t n, int bits, unsigned int* __restrict__ tplus,
+                   int64_t n, int max_buckets, unsigned int* __restrict__ tplus,
                    unsigned long long* __restrict__ counter,
                    unsigned long long* __restrict__ probes) {
-  extern __shared__ int32_t smem[];
-  const int S = 1 << bits;
-  int32_t* keys = smem;
-  uint32_t* slotw = reinterpret_cast<uint32_t*>(smem + S);
+  extern __shared__ int4 keys4[];
+  int32_t* keys = reinterpret_cast<int32_t*>(keys4);
+  uint32_t* slotw = reinterpret_cast<uint32_t*>(keys4 + max_buckets);
   __shared__ int64_t cur;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const int64_t U = __ldg(unit_off + n);
@@ -197,18 +212,18 @@ __global__ void __launch_bounds__(kThreads, kOrientBlocksPerSm)
     const int64_t ob = out_ptr[v], od = out_ptr[v + 1] - ob;
     const int64_t j0 = in_ptr[v] + (unit - __ldg(unit_off + v)) * kInChunk;
     const int64_t j1 = min(in_ptr[v + 1], j0 + kInChunk);
-    // this unit's table: the smallest power of two >= 2 |N+(v)| (at least
-    // 64 slots), so short out-lists clear and flush only a few slots
-    int ub_bits = 6;
-    while ((1ll << ub_bits) < 2 * od) ++ub_bits;
-    const int Su = 1 << ub_bits;
-    for (int s = threadIdx.x; s < Su; s += kThreads) keys[s] = -1;
+    const int nb = table_buckets(od);  // this unit's table
+    for (int s = threadIdx.x; s < nb; s += kThreads) keys4[s] = make_int4(-1, -1, -1, -1);
     __syncthreads();
     for (int64_t i = threadIdx.x; i < od; i += kThreads) {
       const int32_t x = out_col[ob + i];
-      uint32_t s = slot_hash(x, ub_bits);
-      while (atomicCAS(keys + s, -1, x) != -1) s = (s + 1) & (uint32_t)(Su - 1);
-      slotw[s] = (uint32_t)i;  // position, count 0
+      int b = bucket_of(x, nb), j = 0;
+      while (atomicCAS(keys + 4 * b + j, -1, x) != -1)
+        if (++j == 4) {
+          j = 0;
+          b = b + 1 == nb ? 0 : b + 1;
+        }
+      slotw[4 * b + j] = (uint32_t)i;  // position, count 0
     }
     __syncthreads();
     for (int64_t j = j0 + wid; j < j1; j += kThreads / 32) {
@@ -224,12 +239,19 @@ __global__ void __launch_bounds__(kThreads, kOrientBlocksPerSm)
         for (int q = 0; q < kProbeBatch; ++q) {
           const int32_t x = xb[q];
           if (x < 0) continue;
-          uint32_t s = slot_hash(x, ub_bits);
-          int32_t k;
-          while ((k = keys[s]) != -1 && k != x) s = (s + 1) & (uint32_t)(Su - 1);
-          if (k == x) {
+          int b = bucket_of(x, nb), at = -1;
+          for (;;) {
+            const int4 k = keys4[b];
+            if (k.x == x) at = 0;
+            if (k.y == x) at = 1;
+            if (k.z == x) at = 2;
+            if (k.w == x) at = 3;
+            if (at >= 0 || k.w == -1) break;
+            b = b + 1 == nb ? 0 : b + 1;
+          }
+          if (at >= 0) {
             ++hits;
-            atomicAdd(slotw + s, 1u << 16);
+            atomicAdd(slotw + 4 * b + at, 1u << 16);
             atomicAdd(tplus + ub + i0 + 32 * q, 1u);  // edge (u, x)
           }
         }
@@ -239,7 +261,7 @@ __global__ void __launch_bounds__(kThreads, kOrientBlocksPerSm)
       if (lane == 0 && hits) atomicAdd(tplus + in_pos[j], hits);  // edge (u, v)
     }
     __syncthreads();
-    for (int s = threadIdx.x; s < Su; s += kThreads) {
+    for (int s = threadIdx.x; s < 4 * nb; s += kThreads) {
       const uint32_t w = slotw[s];
       if (keys[s] != -1 && (w >> 16) != 0) atomicAdd(tplus + ob + (w & 0xffffu), w >> 16);  // (v, x)
     }
@@ -384,9 +406,8 @@ gs_status build_oriented(gs_graph* g, cudaStream_t stream) {
 gs_status count_tri_oriented(const gs_graph* g, gs_workspace* ws, unsigned long long* h_sums,
                              unsigned long long* h_stats, int64_t* launches, cudaStream_t stream) {
   const int64_t n = g->dev.n, m = g->m;
-  int bits = 6;
-  while ((1 << bits) < 2 * g->max_out_degree) ++bits;
-  const size_t smem = (size_t)(1 << bits) * 2 * sizeof(int32_t);
+  const int buckets = table_buckets(g->max_out_degree);
+  const size_t smem = (size_t)buckets * 4 * 2 * sizeof(int32_t);
   const int fold_blocks = grid_for(n * 32, kThreads, 2);
   void* base = nullptr;
   GS_TRY(ws_reserve(ws, 0,
@@ -408,12 +429,12 @@ gs_status count_tri_oriented(const gs_graph* g, gs_workspace* ws, unsigned long 
   cudaGetDevice(&dev);
   if (dev >= 0 && dev < 64 && !attr_set[dev]) {
     GS_CUDA(cudaFuncSetAttribute(k_tri_oriented, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)((size_t)(2 * kMaxOutDegree) * 2 * sizeof(int32_t))));
+                                 (int)((size_t)table_buckets(kMaxOutDegree) * 4 * 2 * sizeof(int32_t))));
     attr_set[dev] = true;
   }
   if (ws->timing) cudaEventRecord(ws->ev[2], stream);
   k_tri_oriented<<<sm_count() * kOrientBlocksPerSm, kThreads, smem, stream>>>(
-      g->out_ptr, g->out_col, g->in_ptr, g->in_col, g->in_pos, g->orient_units, n, bits, tplus,
+      g->out_ptr, g->out_col, g->in_ptr, g->in_col, g->in_pos, g->orient_units, n, buckets, tplus,
       stats + 7, stats + 0);
   if (ws->timing)
     for (int ev = 3; ev <= 10; ++ev) cudaEventRecord(ws->ev[ev], stream);  // phases 2-4 empty

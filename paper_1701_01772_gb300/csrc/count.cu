@@ -89,6 +89,12 @@ __device__ __forceinline__ int run_length(int64_t total, int64_t warps, int64_t 
   const int64_t r = total / (warps * kRunsPerWarp);
   return r < 1 ? 1 : (int)(r < most ? r : most);
 }
+// The same for chunks of positions, whose costs differ less than the search
+// that begins a run costs: with few of them one run per warp.
+__device__ __forceinline__ int chunk_run_length(int64_t total, int64_t warps, int64_t most) {
+  if (total <= warps * kRunsPerWarp) return (int)((total + warps - 1) / warps);
+  return run_length(total, warps, most);
+}
 // Filter of a dense edge's T members without a matrix slot in k_dense_pairs:
 // 2^15 bits, built when T has at most kTFilterMaxT entries.
 constexpr int kTFilterWords = 1024;
@@ -280,7 +286,7 @@ __global__ void __launch_bounds__(kThreads, kTriBlocksPerSm)
   const int lane = threadIdx.x & 31;
   const int64_t groups = __ldg(off + K) >> 5;  // padded: a multiple of 32
   const int grab =
-      run_length(groups, (int64_t)gridDim.x * (kThreads / 32), (int64_t)kCostGrab);
+      chunk_run_length(groups, (int64_t)gridDim.x * (kThreads / 32), (int64_t)kCostGrab);
   int64_t e = -1, first = 0, end = 0, bu = 0;
   int32_t du = 0, v = 0;
   EndSet sv{};
@@ -336,127 +342,225 @@ void launch_tri_unpadded(const DevGraph& g, const int2* uv, const int64_t* off, 
 
 // ---------------------------------------------------------------- compact T
 
-// Writes T_e in order and tdeg[e] = sum of the degrees of T_e's members
-// (the latter only feeds the cost model statistics).
-__global__ void k_compact_T(DevGraph g, const int2* __restrict__ uv, const int64_t* __restrict__ off,
-                            const int64_t* __restrict__ toff, int64_t K,
-                            const uint32_t* __restrict__ tbits, int32_t* __restrict__ T,
-                            int32_t* __restrict__ tpre, int16_t* __restrict__ T_hm,
-                            int64_t* __restrict__ tdeg,
-                            int32_t* __restrict__ mask_idx,
-                            unsigned long long* __restrict__ dense_counter) {
-  __shared__ uint32_t gbits[kThreads / 32][kGroupWords];  // member groups of a warp's edge
-  const int lane = threadIdx.x & 31;
+constexpr int kCompactBlocksPerSm = 5;
+// Lists of more than this many positions are compacted by a whole CTA: with
+// few edges the longest list is the pass's tail; with many, warps are never
+// short of edges and the CTA's barriers only cost. Compact phase at 1024 /
+// 2048 / 4096 / no limit: adaptive estimation on R-MAT 18 (61 to 2,000 edges a
+// pass) 2.46 / 2.57 / 2.59 / 2.90 ms the whole call, 1M-vertex power-law graph
+// 1% (200,000 edges) 1.07 / 0.88 / 0.91 / 1.17 ms, exact (20M edges) 67 / 51 /
+// 44 / 38 ms.
+inline int64_t compact_long(int64_t K) {
+  return K < (1 << 15) ? 1024 : K < (1 << 21) ? 2048 : INT64_MAX;
+}
+
+// What k_compact_T shares of the edges in work: one per warp, the first one's
+// by the CTA.
+struct CompactShared {
+  uint32_t gbits[kThreads / 32][kGroupWords];  // member groups of an edge
+  int32_t warp_n[kThreads / 32];
+  long long part[kThreads / 32][4];
+};
+
+// T list of edge e by kWarps warps (1: the calling warp; else the CTA): T in
+// order with its matrix slots, tpre per chunk, tdeg[e] = sum of the degrees of
+// T's members (which only feeds the cost model statistics), and the choice of
+// dense mode.
+template <int kWarps>
+__device__ __forceinline__ void compact_edge(const DevGraph& g, int64_t e, int32_t u,
+                                             const int64_t* __restrict__ off,
+                                             const int64_t* __restrict__ toff,
+                                             const uint32_t* __restrict__ tbits, int32_t* T,
+                                             int32_t* __restrict__ tpre, int16_t* T_hm,
+                                             int64_t* __restrict__ tdeg,
+                                             int32_t* __restrict__ mask_idx,
+                                             unsigned long long* __restrict__ dense_counter,
+                                             CompactShared& sh) {
+  constexpr bool kCta = kWarps > 1;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int part = kCta ? wid : 0;
+  auto sync = [&]() {
+    if (kCta) __syncthreads();
+    else __syncwarp();
+  };
+  int64_t bu;
+  const int64_t du = deg_of(g.row_ptr, u, &bu);
+  const int64_t words = (du + 31) >> 5, w0 = off[e] >> 5, t0 = toff[e];
+  const int64_t D = g.hm_dense_words * 32;
+  int64_t pos = t0;
+  long long sum[4] = {0, 0, 0, 0};  // degrees, dense-slot members; then the choice's sums
+  // 32 words of T bits per warp at a time, one per lane; then the words that
+  // have members, four at a time so that their loads are in flight together
+  for (int64_t wb0 = 0; wb0 < words; wb0 += 32 * kWarps) {
+    const int64_t wb = wb0 + 32 * part;
+    const uint32_t word = wb + lane < words ? __ldg(tbits + w0 + wb + lane) : 0u;
+    int before = __popc(word);
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+      const int y = __shfl_up_sync(kFull, before, d);
+      if (lane >= d) before += y;
+    }
+    int all = __shfl_sync(kFull, before, 31);
+    before -= __popc(word);
+    if (kCta) {
+      if (lane == 0) sh.warp_n[wid] = all;
+      __syncthreads();
+      all = 0;
+#pragma unroll
+      for (int k = 0; k < kWarps; ++k) {
+        before += k < wid ? sh.warp_n[k] : 0;
+        all += sh.warp_n[k];
+      }
+      __syncthreads();  // warp_n is rewritten by the next round
+    }
+    if (wb + lane < words) tpre[w0 + wb + lane] = (int32_t)(pos - t0) + before;
+    const int64_t c0 = bu + wb * 32 + lane;
+    for (unsigned nz = __ballot_sync(kFull, word != 0u); nz;) {
+      int32_t x[4];
+      int at[4];
+      int16_t xs[4];
+#pragma unroll
+      for (int h = 0; h < 4; ++h) {
+        const int k = nz ? __ffs(nz) - 1 : 0;
+        const uint32_t wd = nz ? __shfl_sync(kFull, word, k) : 0u;
+        const int bk = __shfl_sync(kFull, before, k);
+        nz &= nz - 1;
+        x[h] = -1;
+        xs[h] = -1;
+        at[h] = bk + __popc(wd & ((1u << lane) - 1u));
+        if ((wd >> lane) & 1u) {
+          x[h] = __ldg(g.col + c0 + k * 32);
+          if (T_hm != nullptr) xs[h] = __ldg(g.col_hm + c0 + k * 32);
+        }
+      }
+#pragma unroll
+      for (int h = 0; h < 4; ++h) {
+        if (x[h] < 0) continue;
+        T[pos + at[h]] = x[h];
+        if (T_hm != nullptr) {
+          T_hm[pos + at[h]] = xs[h];
+          sum[1] += xs[h] >= 0 && xs[h] < D;
+        }
+        sum[0] += __ldg(g.row_ptr + x[h] + 1) - __ldg(g.row_ptr + x[h]);
+      }
+    }
+    pos += all;
+  }
+  // sums (of values >= 0) over the warp, or the CTA
+  auto total = [&](int n) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+      if (i < n)
+        sum[i] = __any_sync(kFull, sum[i] >= (1 << 26))
+                     ? warp_sum<long long>(sum[i])
+                     : (long long)__reduce_add_sync(kFull, (unsigned)sum[i]);
+    if (kCta) {
+      __syncthreads();
+      if (lane == 0)
+        for (int i = 0; i < n; ++i) sh.part[wid][i] = sum[i];
+      __syncthreads();
+      for (int i = 0; i < n; ++i) {
+        sum[i] = 0;
+        for (int k = 0; k < kWarps; ++k) sum[i] += sh.part[k][i];
+      }
+    }
+  };
+  total(2);
+  const long long dsum = sum[0];
+  bool dense_mode = false;
+  if (T_hm != nullptr && sum[1] >= kDenseMin) {
+    // segment-A work of this edge in either mode: sparse = tests over the
+    // shorter of N(w) above w / T above w (estimated); dense = for each
+    // dense-slot member, the 128-bit groups of the T mask that hold a
+    // member and lie at or below its own (what k_dense_pairs reads), plus
+    // the adjacency of the other members
+    const int64_t te = pos - t0;
+    uint32_t* gb = sh.gbits[kCta ? 0 : wid];
+    const int first = kCta ? (int)threadIdx.x : lane;
+    constexpr int kStep = 32 * kWarps;
+    for (int w = first; w < kGroupWords; w += kStep) gb[w] = 0u;
+    sync();  // also: the edge's T entries are visible to all its threads
+    for (int64_t j = first; j < te; j += kStep) {
+      const int xs = T_hm[t0 + j];
+      if (xs >= 0 && xs < D) atomicOr(gb + (xs >> 12), 1u << ((xs >> 7) & 31));
+    }
+    sync();
+    int gpre = lane < kGroupWords ? __popc(gb[lane]) : 0;  // groups in words <= lane
+#pragma unroll
+    for (int d = 1; d < kGroupWords; d <<= 1) {
+      const int y = __shfl_up_sync(kFull, gpre, d);
+      if (lane >= d) gpre += y;
+    }
+    sum[0] = sum[1] = sum[2] = 0;  // sparse, dense, groups
+    for (int64_t j0 = 32 * part; j0 < te; j0 += kStep) {
+      const int64_t j = j0 + lane;
+      const int xs = j < te ? (int)T_hm[t0 + j] : -1;
+      const int gw = __shfl_sync(kFull, gpre, xs >= 4096 ? (xs >> 12) - 1 : 0);
+      if (j >= te) continue;
+      const int32_t x = T[t0 + j];
+      const int64_t dx = __ldg(g.row_ptr + x + 1) - __ldg(g.row_ptr + x);
+      sum[0] += min(dx / 2, te - j - 1);  // about half of N(x) lies above x
+      if (xs >= 0 && xs < D) {
+        const int g0 = xs >> 7;
+        sum[2] += (xs >= 4096 ? gw : 0) + __popc(gb[g0 >> 5] & (kFull >> (31 - (g0 & 31))));
+      } else {  // k_dense_pairs walks its matrix and non-matrix-above lists
+        sum[1] += g.mn_ptr != nullptr ? (__ldg(g.mn_ptr + x + 1) - __ldg(g.mn_ptr + x)) +
+                                            (__ldg(g.nm_ptr + x + 1) - __ldg(g.nm_ptr + x))
+                                      : dx;
+      }
+    }
+    total(3);
+    dense_mode = kGroupCost * sum[2] + 4 * sum[1] < 4 * sum[0];
+  }
+  if ((kCta ? (int)threadIdx.x : lane) == 0) {
+    tdeg[e] = dsum;
+    if (mask_idx != nullptr)
+      mask_idx[e] = dense_mode ? (int32_t)atomicAdd(dense_counter, 1ull) : -1;
+  }
+  if (kCta) __syncthreads();  // sh is reused for the next edge
+}
+
+// T lists of all edges: a warp per edge, then a CTA per edge with a long list
+// (a list of 35,000 positions kept one warp busy for most of a small sample's
+// pass: adaptive estimation on R-MAT 18, 149 us a pass before).
+template <bool kLong>
+__global__ void __launch_bounds__(kThreads, kCompactBlocksPerSm)
+    k_compact_T(const __grid_constant__ DevGraph g, const int2* __restrict__ uv,
+                const int64_t* __restrict__ off, const int64_t* __restrict__ toff, int64_t K,
+                const uint32_t* __restrict__ tbits, int32_t* T, int32_t* __restrict__ tpre,
+                int16_t* T_hm, int64_t* __restrict__ tdeg, int32_t* __restrict__ mask_idx,
+                unsigned long long* __restrict__ dense_counter, int64_t long_list) {
+  __shared__ CompactShared sh;
   const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
   for (int64_t e = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; e < K; e += warps) {
-    int2 pr = uv[e];
-    int64_t bu;
-    int64_t du = deg_of(g.row_ptr, pr.x, &bu);
-    const int64_t words = (du + 31) >> 5, w0 = off[e] >> 5, t0 = toff[e];
-    int64_t pos = t0;
-    long long dsum = 0;
-    int thm = 0;
-    // 32 words of T bits at a time, one per lane; then the words that have
-    // members, four at a time so that their loads are in flight together
-    for (int64_t wb = 0; wb < words; wb += 32) {
-      const uint32_t word = wb + lane < words ? __ldg(tbits + w0 + wb + lane) : 0u;
-      int before = __popc(word);
-#pragma unroll
-      for (int d = 1; d < 32; d <<= 1) {
-        const int y = __shfl_up_sync(kFull, before, d);
-        if (lane >= d) before += y;
-      }
-      const int all = __shfl_sync(kFull, before, 31);
-      before -= __popc(word);
-      if (wb + lane < words) tpre[w0 + wb + lane] = (int32_t)(pos - t0) + before;
-      const int64_t c0 = bu + wb * 32 + lane;
-      for (unsigned nz = __ballot_sync(kFull, word != 0u); nz;) {
-        int32_t x[4];
-        int at[4];
-        int16_t xs[4];
-#pragma unroll
-        for (int h = 0; h < 4; ++h) {
-          const int k = nz ? __ffs(nz) - 1 : 0;
-          const uint32_t wd = nz ? __shfl_sync(kFull, word, k) : 0u;
-          const int bk = __shfl_sync(kFull, before, k);
-          nz &= nz - 1;
-          x[h] = -1;
-          xs[h] = -1;
-          at[h] = bk + __popc(wd & ((1u << lane) - 1u));
-          if ((wd >> lane) & 1u) {
-            x[h] = __ldg(g.col + c0 + k * 32);
-            if (T_hm != nullptr) xs[h] = __ldg(g.col_hm + c0 + k * 32);
-          }
-        }
-#pragma unroll
-        for (int h = 0; h < 4; ++h) {
-          if (x[h] < 0) continue;
-          T[pos + at[h]] = x[h];
-          if (T_hm != nullptr) {
-            T_hm[pos + at[h]] = xs[h];
-            thm += xs[h] >= 0 && xs[h] < g.hm_dense_words * 32;
-          }
-          dsum += __ldg(g.row_ptr + x[h] + 1) - __ldg(g.row_ptr + x[h]);
-        }
-      }
-      pos += all;
+    const int32_t u = uv[e].x;
+    if (!kLong || __ldg(g.row_ptr + u + 1) - __ldg(g.row_ptr + u) <= long_list)
+      compact_edge<1>(g, e, u, off, toff, tbits, T, tpre, T_hm, tdeg, mask_idx, dense_counter,
+                      sh);
+  }
+  if (!kLong) return;
+  __syncthreads();
+  // the CTA looks at `look` edges at a time for long lists: few enough that a
+  // small sample is spread over all CTAs
+  const int look = (int)min((int64_t)kThreads, max((int64_t)1, K / gridDim.x));
+  for (int64_t b = (int64_t)blockIdx.x * look; b < K; b += (int64_t)gridDim.x * look) {
+    __shared__ uint32_t todo[kThreads / 32];
+    const int64_t e = b + threadIdx.x;
+    bool is_long = false;
+    if ((int)threadIdx.x < look && e < K) {
+      const int32_t u = uv[e].x;
+      is_long = __ldg(g.row_ptr + u + 1) - __ldg(g.row_ptr + u) > long_list;
     }
-    thm = __reduce_add_sync(kFull, thm);
-    for (int o = 16; o > 0; o >>= 1) dsum += __shfl_xor_sync(kFull, dsum, o);
-    bool dense_mode = false;
-    if (T_hm != nullptr && thm >= kDenseMin) {
-      // segment-A work of this edge in either mode: sparse = tests over the
-      // shorter of N(w) above w / T above w (estimated); dense = for each
-      // dense-slot member, the 128-bit groups of the T mask that hold a
-      // member and lie at or below its own (what k_dense_pairs reads), plus
-      // the adjacency of the other members
-      __syncwarp();  // this warp's T entries are visible to all its lanes
-      const int64_t te = pos - t0;
-      const int D = (int)(g.hm_dense_words * 32);
-      uint32_t* gb = gbits[threadIdx.x >> 5];
-      for (int w = lane; w < kGroupWords; w += 32) gb[w] = 0u;
-      __syncwarp();
-      for (int64_t j = lane; j < te; j += 32) {
-        const int xs = T_hm[t0 + j];
-        if (xs >= 0 && xs < D) atomicOr(gb + (xs >> 12), 1u << ((xs >> 7) & 31));
+    const unsigned bal = __ballot_sync(kFull, is_long);
+    if ((threadIdx.x & 31) == 0) todo[threadIdx.x >> 5] = bal;
+    __syncthreads();
+    for (int w = 0; w < kThreads / 32; ++w)
+      for (unsigned m = todo[w]; m; m &= m - 1) {
+        const int64_t el = b + w * 32 + __ffs(m) - 1;
+        compact_edge<kThreads / 32>(g, el, uv[el].x, off, toff, tbits, T, tpre, T_hm, tdeg,
+                                    mask_idx, dense_counter, sh);
       }
-      __syncwarp();
-      int gpre = lane < kGroupWords ? __popc(gb[lane]) : 0;  // groups in words <= lane
-#pragma unroll
-      for (int d = 1; d < kGroupWords; d <<= 1) {
-        const int y = __shfl_up_sync(kFull, gpre, d);
-        if (lane >= d) gpre += y;
-      }
-      long long sparse = 0, dense = 0, groups = 0;
-      for (int64_t j0 = 0; j0 < te; j0 += 32) {
-        const int64_t j = j0 + lane;
-        const int xs = j < te ? (int)T_hm[t0 + j] : -1;
-        const int gw = __shfl_sync(kFull, gpre, xs >= 4096 ? (xs >> 12) - 1 : 0);
-        if (j >= te) continue;
-        const int32_t x = T[t0 + j];
-        const int64_t dx = __ldg(g.row_ptr + x + 1) - __ldg(g.row_ptr + x);
-        sparse += min(dx / 2, te - j - 1);  // about half of N(x) lies above x
-        if (xs >= 0 && xs < D) {
-          const int g0 = xs >> 7;
-          groups += (xs >= 4096 ? gw : 0) + __popc(gb[g0 >> 5] & (kFull >> (31 - (g0 & 31))));
-        } else {  // k_dense_pairs walks its matrix and non-matrix-above lists
-          dense += g.mn_ptr != nullptr ? (__ldg(g.mn_ptr + x + 1) - __ldg(g.mn_ptr + x)) +
-                                             (__ldg(g.nm_ptr + x + 1) - __ldg(g.nm_ptr + x))
-                                       : dx;
-        }
-      }
-      for (int o = 16; o > 0; o >>= 1) {
-        sparse += __shfl_xor_sync(kFull, sparse, o);
-        dense += __shfl_xor_sync(kFull, dense, o);
-        groups += __shfl_xor_sync(kFull, groups, o);
-      }
-      dense_mode = kGroupCost * groups + 4 * dense < 4 * sparse;
-    }
-    if (lane == 0) {
-      tdeg[e] = dsum;
-      if (mask_idx != nullptr)
-        mask_idx[e] = dense_mode ? (int32_t)atomicAdd(dense_counter, 1ull) : -1;
-    }
+    __syncthreads();  // todo is rewritten
   }
 }
 
@@ -989,7 +1093,7 @@ __global__ void __launch_bounds__(kThreads, kCostBlocksPerSm)
   // runs of consecutive chunks from a counter (chunks differ in cost: table
   // answers, hub edges)
   const int grab =
-      run_length(groups, (int64_t)gridDim.x * (kThreads / 32), (int64_t)kCostGrab);
+      chunk_run_length(groups, (int64_t)gridDim.x * (kThreads / 32), (int64_t)kCostGrab);
   for (;;) {
     unsigned long long got = 0;
     if (lane == 0) got = atomicAdd(stats + 8, (unsigned long long)grab);
@@ -1814,8 +1918,15 @@ int64_t launch_scan_t(CountBufs& b, cudaStream_t stream) {
 // from the counter stats[6]). T must hold b.toff[K] entries. No host sync.
 int64_t launch_compact(const DevGraph& g, CountBufs& b, cudaStream_t stream) {
   int16_t* T_hm = g.col_hm != nullptr ? b.T_hm : nullptr;
-  k_compact_T<<<grid_for(b.K * 32, kThreads, 8), kThreads, 0, stream>>>(
-      g, b.uv, b.off, b.toff, b.K, b.tbits, b.T, b.tpre, T_hm, b.tdeg, b.mask_idx, b.stats + 6);
+  const int64_t long_list = compact_long(b.K);
+  if (long_list == INT64_MAX)
+    k_compact_T<false><<<grid_for(b.K * 32, kThreads, 8), kThreads, 0, stream>>>(
+        g, b.uv, b.off, b.toff, b.K, b.tbits, b.T, b.tpre, T_hm, b.tdeg, b.mask_idx, b.stats + 6,
+        long_list);
+  else
+    k_compact_T<true><<<grid_for(b.K * kThreads, kThreads, 8), kThreads, 0, stream>>>(
+        g, b.uv, b.off, b.toff, b.K, b.tbits, b.T, b.tpre, T_hm, b.tdeg, b.mask_idx, b.stats + 6,
+        long_list);
   return 1;
 }
 

@@ -121,28 +121,59 @@ __global__ void scan_tiles(const int64_t* in, int64_t* out, int64_t count,
   if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) out[count] = carries[gridDim.x];
 }
 
-// Scans of at most kScanSmall elements in one launch by one block (each
-// launch of the three-kernel scan costs a small call about 3 us and a gap).
-constexpr int64_t kScanSmall = 4 * kScanTile;
-__global__ void scan_small(const int64_t* in, int64_t* out, int64_t count) {
+// Scans of at most kScanSmall elements in one launch by one block: each launch
+// of the three-kernel scan costs a small call about 3 us and a gap. All of a
+// thread's elements are loaded (and summed per tile) before the one block-wide
+// scan of the tiles' sums.
+constexpr int kSmallTiles = 4;
+constexpr int64_t kScanSmall = kSmallTiles * kScanTile;
+__global__ void __launch_bounds__(kScanThreads)
+    scan_small(const int64_t* in, int64_t* out, int64_t count) {
+  __shared__ int64_t warp_sums[kSmallTiles][32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  int64_t s[kSmallTiles], x[kSmallTiles];
+#pragma unroll
+  for (int t = 0; t < kSmallTiles; ++t) {
+    const int64_t base = t * kScanTile + (int64_t)threadIdx.x * kScanItems;
+    s[t] = 0;
+#pragma unroll
+    for (int i = 0; i < kScanItems; ++i)
+      if (base + i < count) s[t] += in[base + i];
+  }
+#pragma unroll
+  for (int t = 0; t < kSmallTiles; ++t) {
+    x[t] = s[t];
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+      const int64_t y = __shfl_up_sync(0xffffffffu, x[t], d);
+      if (lane >= d) x[t] += y;
+    }
+    if (lane == 31) warp_sums[t][warp] = x[t];
+  }
+  __syncthreads();
+  if (warp < kSmallTiles) {
+    int64_t v = warp_sums[warp][lane];
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+      const int64_t y = __shfl_up_sync(0xffffffffu, v, d);
+      if (lane >= d) v += y;
+    }
+    warp_sums[warp][lane] = v;
+  }
+  __syncthreads();
   int64_t carry = 0;
-  for (int64_t start = 0; start < count; start += kScanTile) {
-    const int64_t base = start + (int64_t)threadIdx.x * kScanItems;
-    int64_t vals[kScanItems];
-    int64_t s = 0;
 #pragma unroll
-    for (int i = 0; i < kScanItems; ++i) {
-      vals[i] = base + i < count ? in[base + i] : 0;
-      s += vals[i];
-    }
-    int64_t total;
-    int64_t ex = carry + block_exclusive_scan(s, &total);
+  for (int t = 0; t < kSmallTiles; ++t) {
+    int64_t ex = carry + (warp > 0 ? warp_sums[t][warp - 1] : 0) + x[t] - s[t];
+    const int64_t base = t * kScanTile + (int64_t)threadIdx.x * kScanItems;
 #pragma unroll
-    for (int i = 0; i < kScanItems; ++i) {
-      if (base + i < count) out[base + i] = ex;
-      ex += vals[i];
-    }
-    carry += total;
+    for (int i = 0; i < kScanItems; ++i)
+      if (base + i < count) {
+        const int64_t v = in[base + i];  // read before it is overwritten in place
+        out[base + i] = ex;
+        ex += v;
+      }
+    carry += warp_sums[t][31];
   }
   if (threadIdx.x == 0) out[count] = carry;
 }

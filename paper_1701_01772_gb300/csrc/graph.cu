@@ -399,6 +399,81 @@ __global__ void k_big_fill(const int64_t* __restrict__ row_ptr, const int32_t* _
   }
 }
 
+// The lists of one chunk of a row's entries, walked by a CTA in 32-position
+// segments (each list padded to whole segments): entry k has the list at
+// at[k] of len[k] elements and begins at segment seg[k].
+template <int kRowThreads>
+struct RowLists {
+  int64_t at[kRowThreads];
+  int32_t len[kRowThreads], seg[kRowThreads];
+  int32_t wn[kRowThreads / 32], ws[kRowThreads / 32];
+};
+
+// Calls use(element index) for every list element of the CTA's entries: thread
+// i brings the list [at, at + len) of entry i. A warp takes kRowSegments
+// consecutive segments, finds the first one's list once and loads all of them
+// before the first is used. Looking the list up for every position (14 halving
+// steps each) was most of the instructions. Registration with exact 3-node
+// counts of the 100k-vertex power-law graph, where k_mid_rows and k_table_rows
+// took 12.9 of 24.5 ms: 17.5 / 16.1 / 15.7 ms at 2 / 4 / 8 segments.
+constexpr int kRowSegments = 8;
+template <int kRowThreads, class T, class Use>
+__device__ __forceinline__ void walk_lists(RowLists<kRowThreads>& sh, const T* __restrict__ lists,
+                                           int64_t at, int32_t len, Use use) {
+  constexpr int kWarps = kRowThreads / 32;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  // block-wide exclusive scans of (len > 0) and the segments
+  const unsigned nz = __ballot_sync(0xffffffffu, len > 0);
+  const int32_t segs = (len + 31) >> 5;
+  int32_t incl = segs;
+#pragma unroll
+  for (int k = 1; k < 32; k <<= 1) {
+    const int32_t y = __shfl_up_sync(0xffffffffu, incl, k);
+    if (lane >= k) incl += y;
+  }
+  if (lane == 31) {
+    sh.wn[wid] = __popc(nz);
+    sh.ws[wid] = incl;
+  }
+  __syncthreads();
+  int32_t bn = 0, bs = 0, cnt = 0, total = 0;
+  for (int k = 0; k < kWarps; ++k) {
+    if (k < wid) {
+      bn += sh.wn[k];
+      bs += sh.ws[k];
+    }
+    cnt += sh.wn[k];
+    total += sh.ws[k];
+  }
+  if (len > 0) {
+    const int i = bn + __popc(nz & ((1u << lane) - 1u));
+    sh.at[i] = at;
+    sh.len[i] = len;
+    sh.seg[i] = bs + incl - segs;
+  }
+  __syncthreads();
+  for (int32_t q0 = wid * kRowSegments; q0 < total; q0 += kWarps * kRowSegments) {
+    int k = 0;  // last entry starting at or before segment q0
+#pragma unroll
+    for (int step = kRowThreads / 2; step > 0; step >>= 1)
+      if (k + step < cnt && sh.seg[k + step] <= q0) k += step;
+    T x[kRowSegments];
+    bool on[kRowSegments];
+#pragma unroll
+    for (int u = 0; u < kRowSegments; ++u) {
+      const int32_t q = q0 + u;
+      if (k + 1 < cnt && sh.seg[k + 1] <= q) ++k;  // entries have segments: one step at most
+      const int32_t o = (q - sh.seg[k]) * 32 + lane;
+      on[u] = q < total && o < sh.len[k];
+      if (on[u]) x[u] = __ldg(lists + sh.at[k] + o);
+    }
+#pragma unroll
+    for (int u = 0; u < kRowSegments; ++u)
+      if (on[u]) use(x[u]);
+  }
+  __syncthreads();  // sh is reused by the next chunk
+}
+
 // Vertex of every mid row.
 __global__ void k_mid_row_vertex(const int32_t* __restrict__ tb_slot, int64_t n,
                                  int32_t* __restrict__ rows_v) {
@@ -417,15 +492,9 @@ __global__ void __launch_bounds__(kRowThreads, 2048 / kRowThreads)
                int64_t bg_count, uint16_t* __restrict__ md,
                unsigned long long* __restrict__ counter) {
   extern __shared__ uint32_t acc[];  // (bg_count + 1) / 2 words
-  // the current kRowThreads entries of N(w) that have big neighbours:
-  // list offset and first position in the concatenation of their lists
-  __shared__ int64_t sbo[kRowThreads];
-  __shared__ int32_t sst[kRowThreads];
-  __shared__ int32_t wn[kRowThreads / 32], wl[kRowThreads / 32];
+  __shared__ RowLists<kRowThreads> sh;
   __shared__ int64_t cur;
-  constexpr int kWarps = kRowThreads / 32;
   const int W = (int)((bg_count + 1) / 2);
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   for (;;) {
     if (threadIdx.x == 0) cur = (int64_t)atomicAdd(counter, 1ull);
     __syncthreads();  // the previous row has been written out
@@ -442,51 +511,8 @@ __global__ void __launch_bounds__(kRowThreads, 2048 / kRowThreads)
         bo = boff[x];
         len = (int32_t)(boff[x + 1] - bo);
       }
-      // block-wide exclusive scans of (len > 0) and len
-      const unsigned nz = __ballot_sync(0xffffffffu, len > 0);
-      int32_t incl = len;
-#pragma unroll
-      for (int k = 1; k < 32; k <<= 1) {
-        const int32_t y = __shfl_up_sync(0xffffffffu, incl, k);
-        if (lane >= k) incl += y;
-      }
-      if (lane == 31) {
-        wn[wid] = __popc(nz);
-        wl[wid] = incl;
-      }
-      __syncthreads();
-      int32_t bn = 0, bl = 0, cnt = 0, total = 0;
-      for (int k = 0; k < kWarps; ++k) {
-        if (k < wid) {
-          bn += wn[k];
-          bl += wl[k];
-        }
-        cnt += wn[k];
-        total += wl[k];
-      }
-      if (len > 0) {
-        const int at = bn + __popc(nz & ((1u << lane) - 1u));
-        sbo[at] = bo;
-        sst[at] = bl + incl - len;
-      }
-      __syncthreads();
-      // 32-position segments of the concatenation, one per warp at a time;
-      // a segment spans at most 32 entries (all non-empty)
-      for (int32_t q0 = wid * 32; q0 < total; q0 += kRowThreads) {
-        int k0 = 0;  // last entry starting at or before q0
-        for (int step = kRowThreads / 2; step > 0; step >>= 1)
-          if (k0 + step < cnt && sst[k0 + step] <= q0) k0 += step;
-        const int32_t q = q0 + lane;
-        int k = k0;  // last entry starting at or before q
-#pragma unroll
-        for (int step = 16; step > 0; step >>= 1)
-          if (k + step < cnt && sst[k + step] <= q) k += step;
-        if (q < total) {
-          const uint32_t b = __ldg(blist + sbo[k] + (q - sst[k]));
-          atomicAdd(acc + (b >> 1), 1u << (16 * (b & 1u)));
-        }
-      }
-      __syncthreads();  // sbo, sst, wn and wl are reused by the next chunk
+      walk_lists(sh, blist, bo, len,
+                 [&](uint32_t b) { atomicAdd(acc + (b >> 1), 1u << (16 * (b & 1u))); });
     }
     __syncthreads();
     const uint16_t* a16 = reinterpret_cast<const uint16_t*>(acc);
@@ -782,12 +808,8 @@ __global__ void __launch_bounds__(kRowThreads, 2048 / kRowThreads)
                  uint32_t* __restrict__ giant_codeg, uint16_t* __restrict__ tb,
                  unsigned long long* __restrict__ counter) {
   extern __shared__ uint32_t acc[];  // count / 2 words (row 0 is the longest)
-  __shared__ int64_t sbo[kRowThreads];
-  __shared__ int32_t sst[kRowThreads];
-  __shared__ int32_t wn[kRowThreads / 32], wl[kRowThreads / 32];
+  __shared__ RowLists<kRowThreads> sh;
   __shared__ int64_t cur;
-  constexpr int kWarps = kRowThreads / 32;
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   for (;;) {
     if (threadIdx.x == 0) cur = (int64_t)atomicAdd(counter, 1ull);
     __syncthreads();  // the previous row has been written out
@@ -819,54 +841,15 @@ __global__ void __launch_bounds__(kRowThreads, 2048 / kRowThreads)
         bo = lo;
         len = (int32_t)(hi - lo);
       }
-      const unsigned nz = __ballot_sync(0xffffffffu, len > 0);
-      int32_t incl = len;
-#pragma unroll
-      for (int k = 1; k < 32; k <<= 1) {
-        const int32_t y = __shfl_up_sync(0xffffffffu, incl, k);
-        if (lane >= k) incl += y;
-      }
-      if (lane == 31) {
-        wn[wid] = __popc(nz);
-        wl[wid] = incl;
-      }
-      __syncthreads();
-      int32_t bn = 0, bl = 0, cnt = 0, total = 0;
-      for (int k = 0; k < kWarps; ++k) {
-        if (k < wid) {
-          bn += wn[k];
-          bl += wl[k];
+      walk_lists(sh, lists, bo, len, [&](int32_t b) {
+        const int32_t gb = ga >= 0 ? __ldg(giant + b) : -1;
+        if (gb >= 0) {
+          atomicAdd(giant_codeg + (int64_t)ga * giants + gb, 1u);
+        } else {
+          const uint32_t c = (uint32_t)(b - a - 1);
+          atomicAdd(acc + (c >> 1), 1u << (16 * (c & 1u)));
         }
-        cnt += wn[k];
-        total += wl[k];
-      }
-      if (len > 0) {
-        const int at = bn + __popc(nz & ((1u << lane) - 1u));
-        sbo[at] = bo;
-        sst[at] = bl + incl - len;
-      }
-      __syncthreads();
-      for (int32_t q0 = wid * 32; q0 < total; q0 += kRowThreads) {
-        int k0 = 0;
-        for (int step = kRowThreads / 2; step > 0; step >>= 1)
-          if (k0 + step < cnt && sst[k0 + step] <= q0) k0 += step;
-        const int32_t q = q0 + lane;
-        int k = k0;
-#pragma unroll
-        for (int step = 16; step > 0; step >>= 1)
-          if (k + step < cnt && sst[k + step] <= q) k += step;
-        if (q < total) {
-          const int32_t b = __ldg(lists + sbo[k] + (q - sst[k]));
-          const int32_t gb = ga >= 0 ? __ldg(giant + b) : -1;
-          if (gb >= 0) {
-            atomicAdd(giant_codeg + (int64_t)ga * giants + gb, 1u);
-          } else {
-            const uint32_t c = (uint32_t)(b - a - 1);
-            atomicAdd(acc + (c >> 1), 1u << (16 * (c & 1u)));
-          }
-        }
-      }
-      __syncthreads();  // sbo, sst, wn and wl are reused by the next chunk
+      });
     }
     __syncthreads();
     const uint16_t* a16 = reinterpret_cast<const uint16_t*>(acc);
@@ -925,10 +908,10 @@ struct RowShape {
 static RowShape row_shape(size_t row, int least) {
   const size_t sm = (size_t)220 << 10;  // left for CTAs, each with 1 KB of the system's
   for (int t = least; t < 1024; t *= 2) {
-    const size_t cta = row + (size_t)t * 12 + 2048;
+    const size_t cta = row + (size_t)t * 16 + 2048;
     if (sm / cta >= (size_t)(2048 / t)) return RowShape{t, 2048 / t};
   }
-  return RowShape{1024, sm / (row + 1024 * 12 + 2048) >= 2 ? 2 : 1};
+  return RowShape{1024, sm / (row + 1024 * 16 + 2048) >= 2 ? 2 : 1};
 }
 
 // Launches kernel<threads> for the row shape with `smem` dynamic bytes.

@@ -125,7 +125,7 @@ __global__ void scan_tiles(const int64_t* in, int64_t* out, int64_t count,
 // of the three-kernel scan costs a small call about 3 us and a gap. All of a
 // thread's elements are loaded (and summed per tile) before the one block-wide
 // scan of the tiles' sums.
-constexpr int kSmallTiles = 4;
+constexpr int kSmallTiles = 2;
 constexpr int64_t kScanSmall = kSmallTiles * kScanTile;
 __global__ void __launch_bounds__(kScanThreads)
     scan_small(const int64_t* in, int64_t* out, int64_t count) {

@@ -62,7 +62,9 @@ constexpr unsigned kFull = 0xffffffffu;
 #endif
 constexpr int kProbeBlocksPerSm = GS_PROBE_BLOCKS;
 constexpr int64_t kTaskProbes = 512;
-constexpr int kRunTasks = 8;  // tasks a probe warp takes from the counter, at most
+// Tasks a probe warp takes from the counter, at most (a run sets its chunks up
+// anew: 26.0 / 19.1 / 18.3 ms at 1 / 8 / 32 tasks).
+constexpr int kRunTasks = 32;
 constexpr int kCats = 4;   // x7, x9, x10, omega
 constexpr int kCols = 15;  // x3 .. x17
 constexpr int kNone = 0, kT = 1, kSu = 2, kSv = 3;
@@ -252,8 +254,8 @@ __device__ __forceinline__ unsigned bits_below(int32_t x) {
 // chunk. Issue bound before: five shuffles to find the item, two general
 // membership look-ups and 4 x 192-bit predicated additions per probe. 20,000
 // edges of the 100k-vertex power-law graph at p_e = 0.1 (2.1e9 probes): 29.2
-// -> 19.1 ms for the whole call (20.8 / 20.2 / 19.1 / 19.3 ms at 3 / 4 / 5 / 6
-// CTAs per SM).
+// -> 18.3 ms for the whole call (20.8 / 20.2 / 19.1 / 19.3 ms at 3 / 4 / 5 / 6
+// CTAs per SM and runs of 8 tasks).
 __global__ void __launch_bounds__(kThreads, kProbeBlocksPerSm)
     k_micro_probe(const __grid_constant__ DevGraph g, const int2* __restrict__ uv,
                   const int64_t* __restrict__ choff, const int64_t* __restrict__ chunk_e,

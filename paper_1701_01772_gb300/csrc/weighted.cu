@@ -66,7 +66,7 @@ __device__ __forceinline__ uint64_t splitmix(uint64_t x) {
 // host loop before (a launch and a wait per level and per round, one warp per
 // vertex) took 917 launches on the 100k-vertex power-law graph, 18 us each in
 // k_core_peel, where one warp walked a hub's 24,000 neighbours:
-// k-core numbers, 1% weighted sample and its estimates there: 27.1 -> 8.8 ms.
+// k-core numbers, 1% weighted sample and its estimates there: 27.1 -> 5.8 ms.
 constexpr int kPeelThreads = 512;
 constexpr int64_t kPeelPart = 256;  // neighbours per removal entry
 constexpr int kPeelQueue = 16;      // queued vertices of a warp
@@ -208,17 +208,25 @@ __global__ void __launch_bounds__(kPeelThreads)
         for (;;) {
           const int64_t b = __ldg(row_ptr + it.x) + (int64_t)it.y * kPeelPart;
           const int64_t e = min(__ldg(row_ptr + it.x + 1), b + kPeelPart);
-          for (int64_t q = b + lane; q < e; q += 32) {
-            const int32_t x = __ldg(col + q);
-            if (__ldcg(core + x) != -1) continue;
-            if (atomicSub(deg + x, 1) == k + 1) {
-              __stcg(core + x, k);
-              const int64_t d = __ldg(row_ptr + x + 1) - __ldg(row_ptr + x);
+          // every neighbour's load, look and subtraction of a part in flight
+          // at once (in a loop they were one chain of 24 latencies)
+          constexpr int kEach = (int)(kPeelPart / 32);
+          int32_t x[kEach], old[kEach];
+#pragma unroll
+          for (int u = 0; u < kEach; ++u) x[u] = b + 32 * u + lane < e ? __ldg(col + b + 32 * u + lane) : -1;
+#pragma unroll
+          for (int u = 0; u < kEach; ++u) old[u] = x[u] >= 0 ? __ldcg(core + x[u]) : 0;
+#pragma unroll
+          for (int u = 0; u < kEach; ++u) old[u] = old[u] == -1 ? atomicSub(deg + x[u], 1) : -1;
+#pragma unroll
+          for (int u = 0; u < kEach; ++u)
+            if (old[u] == k + 1) {
+              __stcg(core + x[u], k);
+              const int64_t d = __ldg(row_ptr + x[u] + 1) - __ldg(row_ptr + x[u]);
               const int at = d <= kPeelPart ? atomicAdd(&queued[wid], 1) : kPeelQueue;
-              if (at < kPeelQueue) queue[wid][at] = x;
-              else list_removal(x, d, to, &p->entries);
+              if (at < kPeelQueue) queue[wid][at] = x[u];
+              else list_removal(x[u], d, to, &p->entries);
             }
-          }
           __syncwarp();
           if (head >= min(queued[wid], kPeelQueue)) break;
           it = make_int2(queue[wid][head], 0);

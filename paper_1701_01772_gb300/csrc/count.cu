@@ -78,7 +78,12 @@ constexpr unsigned long long kEmpty = ~0ull;
 constexpr int kStatSlots = 16;
 // Chunks per run a k_chunk_cost warp takes from its counter, at most; also
 // the most chunks a pack of k_quad spans (packs do not cross runs), at most 32.
-constexpr int kCostGrab = 16;
+constexpr int kCostGrab = 32;
+static_assert(kCostGrab <= 32, "a pack's chunks are read by the lanes of a warp");
+// The same for k_tri_chunks, whose chunks are cheap next to the search that
+// begins a run (1M-vertex power-law graph exact: 38.2 / 34.6 / 32.3 / 33.3 ms
+// at 16 / 32 / 128 / 512 chunks).
+constexpr int kTriGrab = 128;
 // Runs each warp should get to take from a counter: with fewer the work that
 // is left over at the end is a large share of a warp's time, and a call with
 // little work would leave most warps without a run (ER 2000/20000 exact:
@@ -277,8 +282,8 @@ __global__ void __launch_bounds__(kThreads) k_tri(DevGraph g, const int2* __rest
 // looked up when the edge changes, t is added once per edge and run, and the
 // next chunk's elements are loaded before this chunk's answers are used.
 // k_tri<true> looked all of it up for every position: 1M-vertex power-law
-// graph exact (5.6e9 positions): 47.2 -> 37.9 ms (44.2 / 40.8 ms at 8 / 5
-// CTAs per SM).
+// graph exact (5.6e9 positions): 47.2 -> 32.3 ms (with runs of 16 chunks 37.9,
+// and 44.2 / 40.8 at 8 / 5 CTAs per SM instead of 6).
 __global__ void __launch_bounds__(kThreads, kTriBlocksPerSm)
     k_tri_chunks(const __grid_constant__ DevGraph g, const int2* __restrict__ uv,
                  const int64_t* __restrict__ off, int64_t K, unsigned long long* __restrict__ t,
@@ -286,7 +291,7 @@ __global__ void __launch_bounds__(kThreads, kTriBlocksPerSm)
   const int lane = threadIdx.x & 31;
   const int64_t groups = __ldg(off + K) >> 5;  // padded: a multiple of 32
   const int grab =
-      chunk_run_length(groups, (int64_t)gridDim.x * (kThreads / 32), (int64_t)kCostGrab);
+      chunk_run_length(groups, (int64_t)gridDim.x * (kThreads / 32), (int64_t)kTriGrab);
   int64_t e = -1, first = 0, end = 0, bu = 0;
   int32_t du = 0, v = 0;
   EndSet sv{};
@@ -520,6 +525,8 @@ __device__ __forceinline__ void compact_edge(const DevGraph& g, int64_t e, int32
   if (kCta) __syncthreads();  // sh is reused for the next edge
 }
 
+static_assert(kDenseMin > 32, "an edge of at most 32 positions is never dense");
+
 // T lists of all edges: a warp per edge, then a CTA per edge with a long list
 // (a list of 35,000 positions kept one warp busy for most of a small sample's
 // pass: adaptive estimation on R-MAT 18, 149 us a pass before).
@@ -532,13 +539,49 @@ __global__ void __launch_bounds__(kThreads, kCompactBlocksPerSm)
                 unsigned long long* __restrict__ dense_counter, int64_t long_list) {
   __shared__ CompactShared sh;
   const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
+  if (!kLong) {
+    // 32 edges per warp: a lane does an edge of at most 32 positions by itself
+    // (it cannot be dense), the warp does the others one by one (a warp per
+    // such edge left 31 lanes idle: batch of 1024 graphs 58 -> 50 ms)
+    const int lane = threadIdx.x & 31;
+    for (int64_t b = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * 32; b < K;
+         b += warps * 32) {
+      const int64_t e = b + lane;
+      int32_t u = 0;
+      int64_t bu = 0, du = 0;
+      if (e < K) {
+        u = uv[e].x;
+        du = deg_of(g.row_ptr, u, &bu);
+      }
+      if (e < K && du <= 32) {
+        const int64_t w = off[e] >> 5;
+        uint32_t word = __ldg(tbits + w);
+        int64_t at = toff[e], dsum = 0;
+        tpre[w] = 0;
+        for (; word; word &= word - 1, ++at) {
+          const int64_t p = bu + __ffs(word) - 1;
+          const int32_t x = __ldg(g.col + p);
+          T[at] = x;
+          if (T_hm != nullptr) T_hm[at] = __ldg(g.col_hm + p);
+          dsum += __ldg(g.row_ptr + x + 1) - __ldg(g.row_ptr + x);
+        }
+        tdeg[e] = dsum;
+        if (mask_idx != nullptr) mask_idx[e] = -1;
+      }
+      for (unsigned m = __ballot_sync(kFull, du > 32); m; m &= m - 1) {
+        const int src = __ffs(m) - 1;
+        compact_edge<1>(g, b + src, __shfl_sync(kFull, u, src), off, toff, tbits, T, tpre, T_hm,
+                        tdeg, mask_idx, dense_counter, sh);
+      }
+    }
+    return;
+  }
   for (int64_t e = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; e < K; e += warps) {
     const int32_t u = uv[e].x;
-    if (!kLong || __ldg(g.row_ptr + u + 1) - __ldg(g.row_ptr + u) <= long_list)
+    if (__ldg(g.row_ptr + u + 1) - __ldg(g.row_ptr + u) <= long_list)
       compact_edge<1>(g, e, u, off, toff, tbits, T, tpre, T_hm, tdeg, mask_idx, dense_counter,
                       sh);
   }
-  if (!kLong) return;
   __syncthreads();
   // the CTA looks at `look` edges at a time for long lists: few enough that a
   // small sample is spread over all CTAs

@@ -309,7 +309,7 @@ __global__ void __launch_bounds__(kThreads, kTriBlocksPerSm)
       if (p0 < first || p0 >= end) {  // another edge: the next one, or a search
         if (found && lane == 0) atomicAdd(t + e, (unsigned long long)found);
         found = 0;
-        e = p0 == end && e >= 0 ? e + 1 : last_le(off, K, p0);
+        e = p0 == end && e >= 0 ? e + 1 : last_le_warp(off, K, p0);
         first = __ldg(off + e);
         end = __ldg(off + e + 1);
         const int2 pr = uv[e];
@@ -1425,8 +1425,8 @@ __global__ void __launch_bounds__(kThreads, kQuadBlocksPerSm)
     int64_t task = (int64_t)__shfl_sync(kFull, got, 0);
     int left = (int)min((int64_t)grab, __ldg(task_off + groups) - task);
     if (left <= 0) break;
-    int64_t gi = last_le(task_off, groups, task);
-    int64_t e0 = last_le(off, K, gi * 32);
+    int64_t gi = last_le_warp(task_off, groups, task);
+    int64_t e0 = last_le_warp(off, K, gi * 32);
     while (left > 0) {
       // the tasks of this run that lie in the pack at chunk gi
       while (__ldg(task_off + gi + 1) <= task) ++gi;

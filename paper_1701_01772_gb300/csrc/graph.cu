@@ -29,29 +29,54 @@ constexpr unsigned long long kMidWorkMax = GS_MID_WORK_MAX;
 // One warp per row (grid-stride). Checks the simple-graph conditions of
 // Sec. 2.1: ids in range, strictly increasing lists (sorted, no repeats),
 // no self-loops, and symmetry (u lists v => v lists u, by halving search).
-__global__ void k_validate(const int64_t* __restrict__ row_ptr, const int32_t* __restrict__ col,
+constexpr int64_t kValidateLong = 1024;
+__global__ void __launch_bounds__(256)
+    k_validate(const int64_t* __restrict__ row_ptr, const int32_t* __restrict__ col,
                            int64_t n, int64_t nnz, DevError* err) {
   const int lane = threadIdx.x & 31;
   const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
+  auto check = [&](int64_t v, int64_t s, int64_t p) {
+    const int32_t x = col[p];
+    if (x < 0 || x >= n) { raise_error(err, GS_EINVAL, p); return; }
+    if (x == v) { raise_error(err, GS_ESELFLOOP, p); return; }
+    if (p > s) {
+      const int32_t prev = col[p - 1];
+      if (prev == x) raise_error(err, GS_EDUP, p);
+      else if (prev > x) raise_error(err, GS_ENOTSORTED, p);
+    }
+    const int64_t xs = row_ptr[x], xe = row_ptr[x + 1];
+    if (xs < 0 || xe < xs || xe > nnz || !sorted_contains(col + xs, xe - xs, (int32_t)v))
+      raise_error(err, GS_EASYM, p);
+  };
   for (int64_t v = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; v < n; v += warps) {
-    int64_t s = row_ptr[v], e = row_ptr[v + 1];
+    const int64_t s = row_ptr[v], e = row_ptr[v + 1];
     if (s < 0 || e < s || e > nnz) {
       if (lane == 0) raise_error(err, GS_EINVAL, v);
       continue;
     }
-    for (int64_t p = s + lane; p < e; p += 32) {
-      int32_t x = col[p];
-      if (x < 0 || x >= n) { raise_error(err, GS_EINVAL, p); continue; }
-      if (x == v) { raise_error(err, GS_ESELFLOOP, p); continue; }
-      if (p > s) {
-        int32_t prev = col[p - 1];
-        if (prev == x) raise_error(err, GS_EDUP, p);
-        else if (prev > x) raise_error(err, GS_ENOTSORTED, p);
-      }
-      int64_t xs = row_ptr[x], xe = row_ptr[x + 1];
-      if (xs < 0 || xe < xs || xe > nnz || !sorted_contains(col + xs, xe - xs, (int32_t)v))
-        raise_error(err, GS_EASYM, p);
+    if (e - s > kValidateLong) continue;
+    for (int64_t p = s + lane; p < e; p += 32) check(v, s, p);
+  }
+  // long rows by the whole CTA (one warp's walk of a hub's row was the tail)
+  __shared__ uint32_t todo[8];
+  const int look = (int)min((int64_t)blockDim.x, max((int64_t)1, n / gridDim.x));
+  for (int64_t b = (int64_t)blockIdx.x * look; b < n; b += (int64_t)gridDim.x * look) {
+    const int64_t v = b + threadIdx.x;
+    bool is_long = false;
+    if ((int)threadIdx.x < look && v < n) {
+      const int64_t s = row_ptr[v], e = row_ptr[v + 1];
+      is_long = s >= 0 && e - s > kValidateLong && e <= nnz;
     }
+    const unsigned bal = __ballot_sync(0xffffffffu, is_long);
+    if (lane == 0) todo[threadIdx.x >> 5] = bal;
+    __syncthreads();
+    for (int w = 0; w < (int)(blockDim.x >> 5); ++w)
+      for (unsigned m = todo[w]; m; m &= m - 1) {
+        const int64_t vl = b + w * 32 + __ffs(m) - 1;
+        const int64_t s = row_ptr[vl], e = row_ptr[vl + 1];
+        for (int64_t p = s + threadIdx.x; p < e; p += blockDim.x) check(vl, s, p);
+      }
+    __syncthreads();  // todo is rewritten
   }
 }
 
@@ -225,6 +250,10 @@ __global__ void k_col_slots(const int32_t* __restrict__ col, int64_t nnz,
     col_hm[p] = (int16_t)__ldg(slot + col[p]);
 }
 
+// Steps of 32 entries that the warp-per-vertex list fills load ahead: a hub's
+// list, one dependent step after another, was the tail of each of them.
+constexpr int kFillDeep = 8;
+
 // Per vertex: matrix neighbours (mn) and neighbours above v without a
 // matrix slot (nm). One warp per vertex; counts first, then the lists in
 // adjacency order at the scanned offsets.
@@ -238,22 +267,30 @@ __global__ void k_rest_lists(const int64_t* __restrict__ row_ptr, const int32_t*
   for (int64_t v = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; v < n; v += warps) {
     int64_t am = mn_off != nullptr ? mn_off[v] : 0, an = nm_off != nullptr ? nm_off[v] : 0;
     unsigned cm = 0, cn = 0;
-    for (int64_t p0 = row_ptr[v]; p0 < row_ptr[v + 1]; p0 += 32) {
-      const int64_t p = p0 + lane;
-      const bool in = p < row_ptr[v + 1];
-      const int16_t s = in ? col_hm[p] : (int16_t)-1;
-      const int32_t x = in ? col[p] : -1;
-      const unsigned bm = __ballot_sync(0xffffffffu, in && s >= 0);
-      const unsigned bn = __ballot_sync(0xffffffffu, in && s < 0 && x > (int32_t)v);
-      const unsigned below = (1u << lane) - 1u;
-      if (mn_off != nullptr) {
-        if ((bm >> lane) & 1u) mn_slot[am + __popc(bm & below)] = s;
-        if ((bn >> lane) & 1u) nm_col[an + __popc(bn & below)] = x;
+    const int64_t end = row_ptr[v + 1];
+    for (int64_t p0 = row_ptr[v] + lane; p0 - lane < end; p0 += 32 * kFillDeep) {
+      int16_t s[kFillDeep];
+      int32_t x[kFillDeep];
+#pragma unroll
+      for (int h = 0; h < kFillDeep; ++h) {
+        const int64_t p = p0 + 32 * h;
+        s[h] = p < end ? col_hm[p] : (int16_t)-1;
+        x[h] = p < end ? col[p] : -1;
       }
-      am += __popc(bm);
-      an += __popc(bn);
-      cm += __popc(bm);
-      cn += __popc(bn);
+#pragma unroll
+      for (int h = 0; h < kFillDeep; ++h) {
+        const unsigned bm = __ballot_sync(0xffffffffu, s[h] >= 0);
+        const unsigned bn = __ballot_sync(0xffffffffu, s[h] < 0 && x[h] > (int32_t)v);
+        const unsigned below = (1u << lane) - 1u;
+        if (mn_off != nullptr) {
+          if ((bm >> lane) & 1u) mn_slot[am + __popc(bm & below)] = s[h];
+          if ((bn >> lane) & 1u) nm_col[an + __popc(bn & below)] = x[h];
+        }
+        am += __popc(bm);
+        an += __popc(bn);
+        cm += __popc(bm);
+        cn += __popc(bn);
+      }
     }
     if (mn_off == nullptr && lane == 0) {
       mn_cnt[v] = cm;
@@ -389,12 +426,19 @@ __global__ void k_big_fill(const int64_t* __restrict__ row_ptr, const int32_t* _
   const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
   for (int64_t x = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; x < n; x += warps) {
     int64_t at = off[x];
-    for (int64_t p0 = row_ptr[x]; p0 < row_ptr[x + 1]; p0 += 32) {
-      const int64_t p = p0 + lane;
-      const int32_t b = p < row_ptr[x + 1] ? __ldg(bg_slot + col[p]) : -1;
-      const unsigned ball = __ballot_sync(0xffffffffu, b >= 0);
-      if (b >= 0) list[at + __popc(ball & ((1u << lane) - 1u))] = (uint16_t)b;
-      at += __popc(ball);
+    const int64_t end = row_ptr[x + 1];
+    for (int64_t p0 = row_ptr[x] + lane; p0 - lane < end; p0 += 32 * kFillDeep) {
+      int32_t c[kFillDeep];
+#pragma unroll
+      for (int h = 0; h < kFillDeep; ++h) c[h] = p0 + 32 * h < end ? col[p0 + 32 * h] : -1;
+#pragma unroll
+      for (int h = 0; h < kFillDeep; ++h) c[h] = c[h] >= 0 ? __ldg(bg_slot + c[h]) : -1;
+#pragma unroll
+      for (int h = 0; h < kFillDeep; ++h) {
+        const unsigned ball = __ballot_sync(0xffffffffu, c[h] >= 0);
+        if (c[h] >= 0) list[at + __popc(ball & ((1u << lane) - 1u))] = (uint16_t)c[h];
+        at += __popc(ball);
+      }
     }
   }
 }
@@ -755,15 +799,19 @@ __global__ void k_hub_nbr_fill(const int64_t* __restrict__ row_ptr, const int32_
   const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
   for (int64_t x = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; x < n; x += warps) {
     int64_t pos = off[x];
-    for (int64_t p0 = row_ptr[x]; p0 < row_ptr[x + 1]; p0 += 32) {
-      int64_t p = p0 + lane;
-      int32_t s = p < row_ptr[x + 1] ? __ldg(slot + col[p]) : -1;
-      unsigned b = __ballot_sync(0xffffffffu, s >= 0);
-      if (s >= 0) {
-        int64_t at = pos + __popc(b & ((1u << lane) - 1u));
-        lists[at] = s;
+    const int64_t end = row_ptr[x + 1];
+    for (int64_t p0 = row_ptr[x] + lane; p0 - lane < end; p0 += 32 * kFillDeep) {
+      int32_t s[kFillDeep];
+#pragma unroll
+      for (int h = 0; h < kFillDeep; ++h) s[h] = p0 + 32 * h < end ? col[p0 + 32 * h] : -1;
+#pragma unroll
+      for (int h = 0; h < kFillDeep; ++h) s[h] = s[h] >= 0 ? __ldg(slot + s[h]) : -1;
+#pragma unroll
+      for (int h = 0; h < kFillDeep; ++h) {
+        const unsigned b = __ballot_sync(0xffffffffu, s[h] >= 0);
+        if (s[h] >= 0) lists[pos + __popc(b & ((1u << lane) - 1u))] = s[h];
+        pos += __popc(b);
       }
-      pos += __popc(b);
     }
   }
 }

@@ -82,17 +82,6 @@ __device__ __forceinline__ int64_t probes_of(int64_t d, double pe) {
   return (int64_t)ceil((double)d * pe);
 }
 
-__device__ __forceinline__ int64_t last_le64(const int64_t* __restrict__ off, int64_t count,
-                                             int64_t p) {
-  int64_t lo = 0, len = count;
-  while (len > 1) {
-    int64_t half = len >> 1;
-    lo = (__ldg(off + lo + half) <= p) ? lo + half : lo;
-    len -= half;
-  }
-  return lo;
-}
-
 // Per-edge set-up: chunk counts of the two lists.
 __global__ void k_micro_chunks(const int64_t* __restrict__ row_ptr, const int2* __restrict__ uv,
                                int64_t K, int64_t* __restrict__ nch,
@@ -276,7 +265,7 @@ __global__ void __launch_bounds__(kThreads, kProbeBlocksPerSm)
     int64_t task = (int64_t)__shfl_sync(kFull, got, 0);
     int left = (int)min((int64_t)grab, __ldg(task_off + C) - task);
     if (left <= 0) break;
-    int64_t c = last_le64(task_off, C, task);
+    int64_t c = last_le_warp(task_off, C, task);
     while (left > 0) {
       while (__ldg(task_off + c + 1) <= task) ++c;
       int here = (int)min((int64_t)left, __ldg(task_off + c + 1) - task);

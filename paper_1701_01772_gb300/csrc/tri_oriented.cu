@@ -85,22 +85,28 @@ __global__ void k_orient_fill(const int64_t* __restrict__ row_ptr, const int32_t
   for (int64_t v = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; v < n; v += warps) {
     const int64_t dv = row_ptr[v + 1] - row_ptr[v];
     int64_t o = out_ptr[v], i = in_ptr[v];
-    for (int64_t p0 = row_ptr[v]; p0 < row_ptr[v + 1]; p0 += 32) {
-      const int64_t p = p0 + lane;
-      const bool live = p < row_ptr[v + 1];
-      int32_t x = 0;
-      bool up = false;
-      if (live) {
-        x = col[p];
-        up = ranks_above(__ldg(row_ptr + x + 1) - __ldg(row_ptr + x), x, dv, (int32_t)v);
+    const int64_t end = row_ptr[v + 1];
+    // several steps' loads in flight (a hub's list is the kernel's tail)
+    constexpr int kDeep = 4;
+    for (int64_t p0 = row_ptr[v] + lane; p0 - lane < end; p0 += 32 * kDeep) {
+      int32_t x[kDeep];
+      int64_t d[kDeep];
+#pragma unroll
+      for (int h = 0; h < kDeep; ++h) x[h] = p0 + 32 * h < end ? col[p0 + 32 * h] : -1;
+#pragma unroll
+      for (int h = 0; h < kDeep; ++h)
+        d[h] = x[h] >= 0 ? __ldg(row_ptr + x[h] + 1) - __ldg(row_ptr + x[h]) : 0;
+#pragma unroll
+      for (int h = 0; h < kDeep; ++h) {
+        const bool live = x[h] >= 0, up = ranks_above(d[h], x[h], dv, (int32_t)v);
+        const unsigned bu = __ballot_sync(kFull, live && up);
+        const unsigned bd = __ballot_sync(kFull, live && !up);
+        const unsigned below = (1u << lane) - 1u;
+        if (live && up) out_col[o + __popc(bu & below)] = x[h];
+        if (live && !up) in_col[i + __popc(bd & below)] = x[h];
+        o += __popc(bu);
+        i += __popc(bd);
       }
-      const unsigned bu = __ballot_sync(kFull, live && up);
-      const unsigned bd = __ballot_sync(kFull, live && !up);
-      const unsigned below = (1u << lane) - 1u;
-      if (live && up) out_col[o + __popc(bu & below)] = x;
-      if (live && !up) in_col[i + __popc(bd & below)] = x;
-      o += __popc(bu);
-      i += __popc(bd);
     }
   }
 }

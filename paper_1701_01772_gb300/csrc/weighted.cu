@@ -285,22 +285,30 @@ __device__ __forceinline__ uint64_t keep_threshold(double scale, int32_t w) {
   return (uint64_t)floor(pi * 9007199254740992.0);
 }
 
-// keep[i] for every canonical edge (one warp per vertex).
-__global__ void k_weighted_flags(const int64_t* __restrict__ row_ptr,
-                                 const int32_t* __restrict__ col,
-                                 const int64_t* __restrict__ up_ptr,
-                                 const int64_t* __restrict__ edge_off,
-                                 const int32_t* __restrict__ vw, int64_t n, double scale,
-                                 uint64_t seed, uint8_t* __restrict__ keep) {
+// keep[i] for every canonical edge. Warps take equal contiguous ranges of the
+// edges (a warp per vertex left a hub's edges to one warp: 0.53 of 5.8 ms of a
+// weighted estimate on the 100k-vertex power-law graph).
+__global__ void __launch_bounds__(kThreads)
+    k_weighted_flags(const int32_t* __restrict__ col, const int64_t* __restrict__ up_ptr,
+                     const int64_t* __restrict__ edge_off, const int32_t* __restrict__ vw,
+                     int64_t n, int64_t m, double scale, uint64_t seed,
+                     uint8_t* __restrict__ keep) {
   const int lane = threadIdx.x & 31;
+  const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
-  for (int64_t u = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; u < n; u += warps) {
-    const int64_t s = up_ptr[u], o = edge_off[u];
-    for (int64_t p = s + lane; p < row_ptr[u + 1]; p += 32) {
-      const uint64_t i = (uint64_t)(o + (p - s));
-      const uint64_t key = splitmix(seed ^ splitmix(i)) >> 11;
-      keep[i] = key < keep_threshold(scale, edge_weight(vw, (int32_t)u, col[p])) ? 1 : 0;
+  const int64_t per = ((m + 31) / 32 + warps - 1) / warps * 32;
+  const int64_t i0 = warp * per, i1 = min(m, i0 + per);
+  if (i0 >= i1) return;
+  int64_t u = last_le_warp(edge_off, n, i0);  // the row of the canonical edge
+  for (int64_t ib = i0; ib < i1; ib += 32) {
+    const int64_t i = ib + lane;
+    if (i < i1) {
+      while (__ldg(edge_off + u + 1) <= i) ++u;
+      const int32_t v = __ldg(col + up_ptr[u] + (i - __ldg(edge_off + u)));
+      const uint64_t key = splitmix(seed ^ splitmix((uint64_t)i)) >> 11;
+      keep[i] = key < keep_threshold(scale, edge_weight(vw, (int32_t)u, v)) ? 1 : 0;
     }
+    u = __shfl_sync(kFull, u, (int)min((int64_t)31, i1 - ib - 1));
   }
 }
 
@@ -605,8 +613,8 @@ extern "C" gs_status gs_sample_weighted(const gs_graph* gr, gs_workspace* ws,
   }
   const double scale = fraction * (double)m / (double)h[0];
   if (scale_out) *scale_out = scale;
-  k_weighted_flags<<<grid_for(n * 32, kThreads, 8), kThreads, 0, stream>>>(
-      gr->dev.row_ptr, gr->dev.col, gr->up_ptr, gr->edge_off, d_vertex_w, n, scale, seed, keep);
+  k_weighted_flags<<<grid_for(m, kThreads, 8), kThreads, 0, stream>>>(
+      gr->dev.col, gr->up_ptr, gr->edge_off, d_vertex_w, n, m, scale, seed, keep);
   k_flag_count<<<(unsigned)tiles, kThreads, 0, stream>>>(keep, m, cnt);
   GS_TRY(exclusive_scan_i64(cnt, off, tiles, tmp, stream));
   int64_t kept = 0;

@@ -149,6 +149,24 @@ __global__ void k_count_deg_ge(const int64_t* __restrict__ row_ptr, int64_t n, i
   if ((threadIdx.x & 31) == 0 && c) atomicAdd(cnt, (unsigned long long)c);
 }
 
+// hist[d] += vertices of degree d. Low degrees, where most vertices lie, are
+// counted in shared memory first.
+constexpr int kHistShared = 4096;
+__global__ void __launch_bounds__(256) k_degree_hist(const int64_t* __restrict__ row_ptr, int64_t n,
+                                                     unsigned int* __restrict__ hist) {
+  __shared__ unsigned int h[kHistShared];
+  for (int i = threadIdx.x; i < kHistShared; i += blockDim.x) h[i] = 0u;
+  __syncthreads();
+  for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n;
+       v += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t d = row_ptr[v + 1] - row_ptr[v];
+    atomicAdd(d < kHistShared ? h + d : hist + d, 1u);
+  }
+  __syncthreads();
+  for (int i = threadIdx.x; i < kHistShared; i += blockDim.x)
+    if (h[i]) atomicAdd(hist + i, h[i]);
+}
+
 __global__ void k_flag_deg_ge(const int64_t* __restrict__ row_ptr, int64_t n, int64_t d,
                               int64_t* __restrict__ flag) {
   for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n;
@@ -978,12 +996,48 @@ static RowShape row_shape(size_t row, int least) {
                                : go(kernel<1024>);                                            \
   }()
 
+// Vertices of degree >= d for every d up to the largest degree + 1, from one
+// device histogram (a registration asks for about 80 such counts; a launch and
+// a wait for each took 2 of the 13.7 ms of a 100k-vertex graph's). Left empty
+// when the degrees are too large for a table.
+constexpr int64_t kDegreeTableMost = (int64_t)1 << 22;
+
+static gs_status degree_table(const gs_graph* g, std::vector<int64_t>* ge, cudaStream_t stream) {
+  ge->clear();
+  if (g->max_degree > kDegreeTableMost) return GS_OK;
+  const size_t bins = (size_t)std::max<int64_t>(g->max_degree + 2, kHistShared);
+  unsigned int* d_hist = nullptr;
+  if (cudaMalloc(&d_hist, sizeof(unsigned int) * bins) != cudaSuccess) {
+    cudaGetLastError();
+    return GS_OK;
+  }
+  std::vector<unsigned int> h(bins);
+  cudaError_t e = cudaMemsetAsync(d_hist, 0, sizeof(unsigned int) * bins, stream);
+  if (e == cudaSuccess) {
+    k_degree_hist<<<grid_for(g->dev.n, 256, 4), 256, 0, stream>>>(g->dev.row_ptr, g->dev.n,
+                                                                  d_hist);
+    e = cudaMemcpyAsync(h.data(), d_hist, sizeof(unsigned int) * bins, cudaMemcpyDeviceToHost,
+                        stream);
+  }
+  if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
+  cudaFree(d_hist);
+  if (e != cudaSuccess) return cuda_fail(e, "degree histogram", __FILE__, __LINE__);
+  ge->assign(bins + 1, 0);
+  for (size_t d = bins; d-- > 0;) (*ge)[d] = (*ge)[d + 1] + (int64_t)h[d];
+  return GS_OK;
+}
+
 // Smallest degree threshold d >= min_deg with at most `cap` vertices of
-// degree >= d (binary search with a device count per probe).
-static gs_status hub_threshold(const gs_graph* g, int64_t cap, int64_t min_deg,
-                               unsigned long long* d_cnt, cudaStream_t stream, int64_t* d_out,
-                               int64_t* count_out) {
+// degree >= d (binary search in degree_table's counts; with a device count per
+// probe when there is none).
+static gs_status hub_threshold(const gs_graph* g, const std::vector<int64_t>& ge, int64_t cap,
+                               int64_t min_deg, unsigned long long* d_cnt, cudaStream_t stream,
+                               int64_t* d_out, int64_t* count_out) {
   auto count_ge = [&](int64_t d, int64_t* c) -> gs_status {
+    if (!ge.empty()) {
+      *c = d < (int64_t)ge.size() ? ge[(size_t)d] : 0;
+      return GS_OK;
+    }
     GS_CUDA(cudaMemsetAsync(d_cnt, 0, sizeof(unsigned long long), stream));
     k_count_deg_ge<<<grid_for(g->dev.n, 256, 8), 256, 0, stream>>>(g->dev.row_ptr, g->dev.n, d,
                                                                    d_cnt);
@@ -1066,10 +1120,12 @@ static gs_status build_hub_index(gs_graph* g, uint64_t budget, bool tables, cuda
     GS_CUDA(cudaGetLastError());
     return GS_OK;
   };
+  std::vector<int64_t> ge;
+  GS_TRY(degree_table(g, &ge, stream));
   // ---- bitmaps
   int64_t d_bm = 0, n_bm = 0;
   if (bm_cap > 0) {
-    GS_TRY(hub_threshold(g, bm_cap, kHubMinDegree, d_cnt, stream, &d_bm, &n_bm));
+    GS_TRY(hub_threshold(g, ge, bm_cap, kHubMinDegree, d_cnt, stream, &d_bm, &n_bm));
     if (n_bm > 0) {
       int32_t* hubs = nullptr;
       GS_TRY(assign(d_bm, &g->bm_slot, &hubs, n_bm, false));
@@ -1148,7 +1204,7 @@ static gs_status build_hub_index(gs_graph* g, uint64_t budget, bool tables, cuda
   // in L2 to pay off)
   int64_t d_hm = 0, n_hm = 0;
   double rest_bytes = 0.0;  // col_hm and the lists built with the matrix
-  if (hm_cap > 1) GS_TRY(hub_threshold(g, hm_cap, kHubMinDegree, d_cnt, stream, &d_hm, &n_hm));
+  if (hm_cap > 1) GS_TRY(hub_threshold(g, ge, hm_cap, kHubMinDegree, d_cnt, stream, &d_hm, &n_hm));
   if (n_hm > 1) {
     int32_t* hubs = nullptr;
     GS_TRY(assign(d_hm, &g->hm_slot, &hubs, n_hm, true));
@@ -1210,7 +1266,7 @@ static gs_status build_hub_index(gs_graph* g, uint64_t budget, bool tables, cuda
   if (!tables) tb_cap = 0;
   int64_t d_tb = 0, n_tb = 0;
   if (tb_cap > 1) {
-    GS_TRY(hub_threshold(g, tb_cap, kHubMinDegree, d_cnt, stream, &d_tb, &n_tb));
+    GS_TRY(hub_threshold(g, ge, tb_cap, kHubMinDegree, d_cnt, stream, &d_tb, &n_tb));
     if (n_tb > 1) {
       int32_t* hubs = nullptr;  // slot -> vertex, for the row build
       GS_TRY(assign(d_tb, &g->tb_slot, &hubs, n_tb, false));
@@ -1334,13 +1390,13 @@ static gs_status build_hub_index(gs_graph* g, uint64_t budget, bool tables, cuda
     for (int64_t cols = kBigMin; cols <= kBigMax; cols *= 2) {
       const int64_t bg_cap = g->dev.tb_count < cols ? g->dev.tb_count : cols;
       Shape sh{0, 0, 0};
-      GS_TRY(hub_threshold(g, bg_cap, d_tb, d_cnt, stream, &sh.dbg, &sh.nbg));
+      GS_TRY(hub_threshold(g, ge, bg_cap, d_tb, d_cnt, stream, &sh.dbg, &sh.nbg));
       if (sh.nbg > 0) {
         const int64_t md_cap = (int64_t)(((double)budget - used) / (2.0 * (double)sh.nbg));
         if (md_cap > 0) {
           // lowest degree >= kMidMinDegree with at most md_cap mid vertices
           int64_t n_ge = 0;
-          GS_TRY(hub_threshold(g, md_cap + g->dev.tb_count, kMidMinDegree, d_cnt, stream, &sh.dmd,
+          GS_TRY(hub_threshold(g, ge, md_cap + g->dev.tb_count, kMidMinDegree, d_cnt, stream, &sh.dmd,
                                &n_ge));
           if (sh.dmd < d_hi) shapes.push_back(sh);
         }

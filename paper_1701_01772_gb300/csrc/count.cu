@@ -21,16 +21,15 @@
 //   prep     one thread per pair: canonical orientation, edge check,
 //            duplicate check, per-edge position count d_u (padded to 32
 //            when 4-node work follows).
-//   tri      positions of N(u) are split evenly over all warps; each lane
-//            tests one x in N(u) for membership in N(v). Ballots give t and,
-//            for 4-node work, one 32-bit word of "x in T" flags per chunk of
-//            32 positions.
-//   compact  T lists written in order with their hub-matrix slots (one warp
-//            per edge); edges with at least kDenseMin matrix members in T
-//            whose dense-mode work (row groups plus the other members'
-//            neighbour lists) is below
-//            their sparse-mode tests are marked dense and get a T mask over
-//            matrix slots.
+//   tri      each lane tests one x in N(u) for membership in N(v); ballots
+//            give t and, for 4-node work (warps then take runs of chunks of
+//            32 positions of one edge), a word of "x in T" flags per chunk.
+//   compact  T lists written in order with their hub-matrix slots (by a warp,
+//            a CTA or a lane per edge, see k_compact_T); edges with at least
+//            kDenseMin matrix members in T whose dense-mode work (row groups
+//            plus the other members' neighbour lists) is below their
+//            sparse-mode tests are marked dense and get a T mask over matrix
+//            slots.
 //   cost     per chunk of 32 positions (items w = N(u)[i]): membership-test
 //            count of each item (iterate the shorter list, test in the
 //            longer); constant terms (the -1s, table co-degrees) added
@@ -47,7 +46,7 @@
 //            past the dense slots, a search of T when above w) and w's
 //            neighbours above w without a matrix slot (a search of T).
 //   fold     per edge numerators N_i in 128-bit, block partial sums, one
-//            final fixed-order pass (or per-segment limb sums, k_fold_seg).
+//            final pass (or per-segment limb sums, k_fold_seg).
 #include <string.h>
 
 #include <algorithm>
@@ -281,7 +280,7 @@ __global__ void __launch_bounds__(kThreads) k_tri(DevGraph g, const int2* __rest
 // counter; what an edge needs (N(u), and how "x in N(v)" is answered) is
 // looked up when the edge changes, t is added once per edge and run, and the
 // next chunk's elements are loaded before this chunk's answers are used.
-// k_tri<true> looked all of it up for every position: 1M-vertex power-law
+// Looking all of it up for every position, as k_tri does for 3-node work alone: 1M-vertex power-law
 // graph exact (5.6e9 positions): 47.2 -> 32.3 ms (with runs of 16 chunks 37.9,
 // and 44.2 / 40.8 at 8 / 5 CTAs per SM instead of 6).
 __global__ void __launch_bounds__(kThreads, kTriBlocksPerSm)

@@ -23,7 +23,7 @@
 
 namespace gs {
 
-// count.cu: fixed-order final pass over the 128-bit block partials.
+// count.cu: final pass over the 128-bit block partials.
 __global__ void k_fold_final(const unsigned __int128* __restrict__ part, int blocks,
                              unsigned long long* __restrict__ out);
 

@@ -275,8 +275,9 @@ __global__ void __launch_bounds__(kThreads) k_tri(DevGraph g, const int2* __rest
   }
 }
 
-// The triangle pass of the 4-node work: positions padded to 32 per edge, so
-// a chunk of 32 positions lies in one edge. Warps take runs of chunks from a
+// The triangle pass of the 4-node work (and of 3-node samples with long lists,
+// see kLongLists; tbits is then NULL): positions padded to 32 per edge, so a
+// chunk of 32 positions lies in one edge. Warps take runs of chunks from a
 // counter; what an edge needs (N(u), and how "x in N(v)" is answered) is
 // looked up when the edge changes, t is added once per edge and run, and the
 // next chunk's elements are loaded before this chunk's answers are used.
@@ -331,11 +332,27 @@ __global__ void __launch_bounds__(kThreads, kTriBlocksPerSm)
         xs = sv.mrow != nullptr && i + 32 < du ? (int32_t)__ldg(g.col_hm + bu + i + 32) : -1;
       }
       const unsigned ball = __ballot_sync(kFull, y >= 0 && y != v && set_has(sv, y, ys));
-      if (lane == 0) tbits[gi] = ball;
+      if (tbits != nullptr && lane == 0) tbits[gi] = ball;
       found += __popc(ball);
     }
     if (found && lane == 0) atomicAdd(t + e, (unsigned long long)found);
   }
+}
+
+// 3-node work alone takes k_tri_chunks, on offsets padded by k_pad_lengths,
+// from this many positions per edge and in all on; below, the padding or the
+// look-ups per edge cost more than they save. R-MAT 22 5% (3.2M edges, 500
+// positions each) 21.8 -> 15.5 ms, 1M-vertex power-law graph 5% (1.0M, 280) 3.0
+// -> 2.2 ms; a uniform graph of mean degree 20 30% (1.2M, 17) 0.43 -> 0.54 ms
+// and R-MAT 18 2% (30,000 edges) 0.15 -> 0.20 ms stay with k_tri.
+constexpr int64_t kLongLists = 96;
+constexpr int64_t kManyPositions = (int64_t)1 << 23;
+
+__global__ void k_pad_lengths(const int64_t* __restrict__ off, int64_t K,
+                              int64_t* __restrict__ len) {
+  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < K;
+       e += (int64_t)gridDim.x * blockDim.x)
+    len[e] = (off[e + 1] - off[e] + 31) & ~(int64_t)31;
 }
 
 // Host launcher of the 3-node triangle pass for count_static.cu.
@@ -1944,10 +1961,17 @@ int64_t launch_front(const gs_graph* gr, const DevGraph& g, const int32_t* pairs
 int64_t launch_tri(const DevGraph& g, bool four, const Tuning& tu, CountBufs& b,
                    cudaStream_t stream) {
   const int grid = sm_count() * tu.tri_blocks_per_sm;
-  if (four)
+  if (four) {
     k_tri_chunks<<<grid, kThreads, 0, stream>>>(g, b.uv, b.off, b.K, b.t, b.tbits, b.stats + 10);
-  else
+  } else if (b.P >= kManyPositions && b.P >= kLongLists * b.K) {
+    // toff is free in 3-node work: the padded offsets
+    k_pad_lengths<<<grid_for(b.K, kThreads, 8), kThreads, 0, stream>>>(b.off, b.K, b.toff);
+    exclusive_scan_i64(b.toff, b.toff, b.K, b.tmp0, stream);
+    k_tri_chunks<<<grid, kThreads, 0, stream>>>(g, b.uv, b.toff, b.K, b.t, nullptr, b.stats + 10);
+    return 2 + scan_launches(b.K);
+  } else {
     k_tri<<<grid, kThreads, 0, stream>>>(g, b.uv, b.off, b.K, b.t);
+  }
   return 1;
 }
 

@@ -96,3 +96,18 @@ def test_samples_at_the_sizes_where_the_t_lists_change_hands(edges):
     want = np.stack([np.asarray(lc[k], dtype=np.int64) for k in ("t", "k", "q")], axis=1)
     assert np.array_equal(per.cpu().numpy()[few], want)
     g.close()
+
+
+def test_three_node_samples_with_long_lists_equal_the_unpadded_pass():
+    gs.build()
+    rp, col = synth.rmat(18, 16, seed=3)
+    g = gs.Graph.from_numpy(rp, col, hub_budget_bytes=2 << 30)
+    for fraction in (0.2, 0.01):  # above and below the line for padded chunks
+        pairs = g.sample(fraction, 5)
+        per = torch.empty((pairs.shape[0], 3), dtype=torch.int64, device="cuda")
+        got = g.count(pairs, gs.GS_THREE_NODE, per)
+        assert got.sums() == gs.gs_count3_static(g.handle, pairs, pairs.shape[0]).sums()
+        few = np.arange(0, pairs.shape[0], pairs.shape[0] // 300)
+        lc = oracle.local_counts(rp, col, pairs.cpu().numpy()[few], four=False)
+        assert np.array_equal(per[:, 0].cpu().numpy()[few], np.asarray(lc["t"]))
+    g.close()

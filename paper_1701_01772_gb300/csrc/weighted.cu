@@ -302,13 +302,13 @@ __global__ void __launch_bounds__(kThreads)
   int64_t u = last_le_warp(edge_off, n, i0);  // the row of the canonical edge
   for (int64_t ib = i0; ib < i1; ib += 32) {
     const int64_t i = ib + lane;
+    u = last_le_lanes(edge_off, n, u, min(i, i1 - 1));
     if (i < i1) {
-      while (__ldg(edge_off + u + 1) <= i) ++u;
       const int32_t v = __ldg(col + up_ptr[u] + (i - __ldg(edge_off + u)));
       const uint64_t key = splitmix(seed ^ splitmix((uint64_t)i)) >> 11;
       keep[i] = key < keep_threshold(scale, edge_weight(vw, (int32_t)u, v)) ? 1 : 0;
     }
-    u = __shfl_sync(kFull, u, (int)min((int64_t)31, i1 - ib - 1));
+    u = __shfl_sync(kFull, u, 31);
   }
 }
 

@@ -232,8 +232,9 @@ __device__ __forceinline__ int64_t last_le_from(const int64_t* __restrict__ off,
 // past them searches on by itself, because rows without entries can lie between
 // two entries in any number. Walked row by row, 10M empty ids between two
 // blocks of 200,000 vertices and 2M edges were 0.8 s of serial loads in a
-// weighted sample (827 -> 1.07 ms; 1.2 -> 1.08 ms with those ids at the end), and
-// so were the short rows of a graph of mean degree 4 (2.24 -> 1.42 ms).
+// weighted sample (827 -> 1.07 ms; 1.2 -> 1.08 ms with those ids at the end) and
+// in a registration (816 -> 5.7 ms), and the short rows of a graph of mean degree
+// 4 were a chain too (weighted sample 2.24 -> 1.42 ms).
 __device__ __forceinline__ int64_t last_le_lanes(const int64_t* __restrict__ off, int64_t count,
                                                  int64_t e, int64_t p) {
   const int64_t k = e + 1 + (threadIdx.x & 31);

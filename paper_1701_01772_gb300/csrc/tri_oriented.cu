@@ -115,7 +115,7 @@ __global__ void k_orient_fill(const int64_t* __restrict__ row_ptr, const int32_t
 // stored at in_col[j] (halving search of the short out-list). Warps take equal
 // contiguous ranges of the m in-edges: a hub's in-list, which one warp walked
 // before, was the tail of the kernel (1.3 of the 28 ms of a 100k-vertex graph's
-// registration).
+// registration). The vertex of each is found as last_le_lanes says.
 __global__ void k_orient_in_pos(const int64_t* __restrict__ out_ptr,
                                 const int32_t* __restrict__ out_col,
                                 const int64_t* __restrict__ in_ptr,
@@ -127,16 +127,11 @@ __global__ void k_orient_in_pos(const int64_t* __restrict__ out_ptr,
   const int64_t per = ((m + 31) / 32 + warps - 1) / warps * 32;
   const int64_t j0 = warp * per, j1 = min(m, j0 + per);
   if (j0 >= j1) return;
-  int64_t v = 0;  // the vertex whose in-list holds the position
-  for (int64_t len = n; len > 1;) {
-    const int64_t half = len >> 1;
-    v = __ldg(in_ptr + v + half) <= j0 ? v + half : v;
-    len -= half;
-  }
+  int64_t v = last_le_warp(in_ptr, n, j0);  // the vertex whose in-list holds the position
   for (int64_t jb = j0; jb < j1; jb += 32) {
     const int64_t j = jb + lane;
+    v = last_le_lanes(in_ptr, n, v, min(j, j1 - 1));
     if (j < j1) {
-      while (__ldg(in_ptr + v + 1) <= j) ++v;
       const int32_t u = in_col[j];
       int64_t lo = out_ptr[u], len = out_ptr[u + 1] - lo;
       while (len > 1) {
@@ -146,7 +141,7 @@ __global__ void k_orient_in_pos(const int64_t* __restrict__ out_ptr,
       }
       in_pos[j] = (uint32_t)lo;
     }
-    v = __shfl_sync(kFull, v, (int)min((int64_t)31, j1 - jb - 1));
+    v = __shfl_sync(kFull, v, 31);
   }
 }
 

@@ -61,3 +61,23 @@ def test_weighted_sample():
         g.close()
     assert np.array_equal(_shifted(kept[0]), kept[1].cpu().numpy())
     assert times[1] <= RATIO * times[0] + SLACK, times
+
+
+def test_registration_and_exact_triangles():
+    gs.build()
+    times, sums = [], []
+    for shift in (0, GAP):
+        rp, col = _two_blocks(shift)
+        rp, col = torch.as_tensor(rp, device="cuda"), torch.as_tensor(col, device="cuda")
+
+        def register():
+            g = gs.Graph(rp, col, hub_budget_bytes=1 << 30)
+            s = g.count(None, gs.GS_THREE_NODE).sums()
+            g.close()
+            return s
+
+        t, s = _best(register)
+        times.append(t)
+        sums.append(s)
+    assert sums[0] == sums[1]
+    assert times[1] <= RATIO * times[0] + SLACK, times

@@ -358,12 +358,24 @@ __global__ void k_dense_rows(const int64_t* __restrict__ row_ptr, const int32_t*
 // 1024 graphs of 50 to 5,000 vertices, exact: 122 -> 74 ms; ER n = 2000
 // exact: 327 -> 269 us.
 constexpr int kBlockRowThreads = 128;
+constexpr int64_t kBlockHeld = 255;  // co-degrees below this are held
+// A query of a pair that the blocks do not hold costs at least 255 tests when
+// no table answers it; a pair is asked for about as often as it has common
+// neighbours. Tables for those pairs pay from one such query in kMissedShare
+// on. Batches of Chung-Lu graphs without and with them, by share of the queries:
+// 0 7.69 / 7.73 ms, 1/1470 50.7 / 51.2, 1/870 4.78 / 4.81, 1/660 13.85 / 13.81,
+// 1/370 12.78 / 12.68, 1/136 15.3 / 14.7, 1/37 37.7 / 32.7; two uniform graphs of
+// 1,100 vertices and half of the pairs, nearly all of them past the blocks, 291
+// / 12.6 (27.6 with 16-bit tables alone).
+constexpr unsigned long long kMissedShare = 512;
 __global__ void __launch_bounds__(kBlockRowThreads)
     k_block_codeg(const int64_t* __restrict__ row_ptr, const int32_t* __restrict__ col, int64_t n,
                   const int64_t* __restrict__ cg_row, const int32_t* __restrict__ first,
-                  const int32_t* __restrict__ row_len, uint8_t* __restrict__ cg) {
+                  const int32_t* __restrict__ row_len, uint8_t* __restrict__ cg,
+                  unsigned long long* __restrict__ totals) {
   extern __shared__ uint32_t acc[];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  unsigned long long wedges = 0, missed = 0;
   for (int64_t v = blockIdx.x; v < n; v += gridDim.x) {
     const int64_t r = cg_row[v];
     if (r < 0) continue;  // the same for the whole CTA
@@ -371,12 +383,15 @@ __global__ void __launch_bounds__(kBlockRowThreads)
     const int W = row_len[v] / 2;  // row_len: a multiple of 16
     for (int i = threadIdx.x; i < W; i += kBlockRowThreads) acc[i] = 0u;
     __syncthreads();
-    for (int64_t p = row_ptr[v] + wid; p < row_ptr[v + 1]; p += kBlockRowThreads / 32) {
+    const int64_t p0 = row_ptr[v], p1 = row_ptr[v + 1];
+    for (int64_t p = p0 + wid; p < p1; p += kBlockRowThreads / 32) {
       const int32_t y = col[p];
-      for (int64_t q = __ldg(row_ptr + y) + lane; q < __ldg(row_ptr + y + 1); q += 32) {
+      const int64_t q0 = __ldg(row_ptr + y), q1 = __ldg(row_ptr + y + 1);
+      for (int64_t q = q0 + lane; q < q1; q += 32) {
         const uint32_t x = (uint32_t)(col[q] - f);
         atomicAdd(acc + (x >> 1), 1u << (16 * (x & 1u)));
       }
+      wedges += (unsigned long long)(q1 - q0 - 1);  // the same in every lane
     }
     __syncthreads();
     // two counters to two bytes
@@ -392,9 +407,18 @@ __global__ void __launch_bounds__(kBlockRowThreads)
       o.z = two(a[4]) | (two(a[5]) << 16);
       o.w = two(a[6]) | (two(a[7]) << 16);
       reinterpret_cast<uint4*>(cg + r)[i] = o;
+      if (__vcmpeq4(o.x, ~0u) | __vcmpeq4(o.y, ~0u) | __vcmpeq4(o.z, ~0u) | __vcmpeq4(o.w, ~0u))
+        for (int k = 0; k < 8; ++k) {
+          const uint32_t lo = a[k] & 0xffffu, hi = a[k] >> 16;
+          missed += (lo < 255u ? 0u : lo) + (hi < 255u ? 0u : hi);
+        }
     }
+    if (threadIdx.x == 0 && p1 - p0 >= 255) missed -= p1 - p0;  // c(v, v) is no pair
     __syncthreads();  // acc is cleared for the next row
   }
+  for (int o = 16; o > 0; o >>= 1) missed += __shfl_xor_sync(0xffffffffu, missed, o);
+  if (lane == 0 && wedges) atomicAdd(totals, wedges);
+  if (lane == 0 && missed) atomicAdd(totals + 1, missed);
 }
 
 // Mid x big co-degrees, one table row at a time: c(w, b) for a mid vertex w
@@ -1070,12 +1094,15 @@ static gs_status hub_threshold(const gs_graph* g, const std::vector<int64_t>& ge
 // budget), the hub-pair matrix (up to 1/8, at most kHubMatrixMax vertices),
 // bucket directories (up to 1/16), the 16-bit co-degree table (most of the
 // rest, at most 65535 vertices), the mid x big table and, if room is left,
-// the table slot of every adjacency entry. tables = false leaves out the
-// co-degree tables and the table slots.
-static gs_status build_hub_index(gs_graph* g, uint64_t budget, bool tables, cudaStream_t stream) {
+// the table slot of every adjacency entry. Co-degrees below `held` are answered
+// elsewhere (0: none): the tables then take only vertices of at least that
+// degree, as both ends of the other pairs are, and the table slots, which would
+// be read for every item, are left out.
+static gs_status build_hub_index(gs_graph* g, uint64_t budget, int64_t held, cudaStream_t stream) {
   const int64_t n = g->dev.n;
   if (n == 0 || g->max_degree < kHubMinDegree) return GS_OK;
   const int64_t words = (n + 31) / 32;
+  const int64_t tb_min = std::max(kHubMinDegree, held), md_min = std::max(kMidMinDegree, held);
   // bitmaps and the matrix get up to 1/8 of the budget each, the table the rest
   const double share = (double)budget / 8.0;
   const int64_t bm_cap = (int64_t)(share / ((double)words * 4.0));
@@ -1263,10 +1290,9 @@ static gs_status build_hub_index(gs_graph* g, uint64_t budget, bool tables, cuda
   // n (n - 1) / 2 entries of 2 bytes
   int64_t tb_cap = tb_bytes > 0 ? (int64_t)sqrt(tb_bytes) : 0;
   if (tb_cap > 65535) tb_cap = 65535;
-  if (!tables) tb_cap = 0;
   int64_t d_tb = 0, n_tb = 0;
   if (tb_cap > 1) {
-    GS_TRY(hub_threshold(g, ge, tb_cap, kHubMinDegree, d_cnt, stream, &d_tb, &n_tb));
+    GS_TRY(hub_threshold(g, ge, tb_cap, tb_min, d_cnt, stream, &d_tb, &n_tb));
     if (n_tb > 1) {
       int32_t* hubs = nullptr;  // slot -> vertex, for the row build
       GS_TRY(assign(d_tb, &g->tb_slot, &hubs, n_tb, false));
@@ -1329,13 +1355,13 @@ static gs_status build_hub_index(gs_graph* g, uint64_t budget, bool tables, cuda
     }
   }
   // ---- mid x big co-degrees: rows for the highest-degree vertices below
-  // the table (degree >= kMidMinDegree), columns for the top 1024-65536
+  // the table (degree >= md_min), columns for the top 1024-65536
   // table vertices; whatever the budget has left
   double used = (double)n_bm * (double)words * 4.0 +
                 (double)n_hm * (double)g->dev.hm_words * 4.0 + rest_bytes +
                 (double)g->dev.tb_count * (double)g->dev.tb_count + dir_bytes;
   const int64_t d_hi = d_tb < 65536 ? d_tb : 65536;
-  if (g->dev.tb_count > 1 && d_hi > kMidMinDegree && (double)budget > used) {
+  if (g->dev.tb_count > 1 && d_hi > md_min && (double)budget > used) {
     // shape: columns = the top 1024 .. 65536 table vertices by degree, rows
     // = the highest-degree mid vertices that fit next to them in the budget
     // (and whose build stays within kMidWorkMax increments); the shape kept
@@ -1394,9 +1420,9 @@ static gs_status build_hub_index(gs_graph* g, uint64_t budget, bool tables, cuda
       if (sh.nbg > 0) {
         const int64_t md_cap = (int64_t)(((double)budget - used) / (2.0 * (double)sh.nbg));
         if (md_cap > 0) {
-          // lowest degree >= kMidMinDegree with at most md_cap mid vertices
+          // lowest degree >= md_min with at most md_cap mid vertices
           int64_t n_ge = 0;
-          GS_TRY(hub_threshold(g, ge, md_cap + g->dev.tb_count, kMidMinDegree, d_cnt, stream, &sh.dmd,
+          GS_TRY(hub_threshold(g, ge, md_cap + g->dev.tb_count, md_min, d_cnt, stream, &sh.dmd,
                                &n_ge));
           if (sh.dmd < d_hi) shapes.push_back(sh);
         }
@@ -1439,7 +1465,7 @@ static gs_status build_hub_index(gs_graph* g, uint64_t budget, bool tables, cuda
       // pilot tests this shape answers
       double saved = 0.0;
       for (const PilotItem& it : pilot)
-        if (it.d_tab >= dbg && it.d_other >= dmd && it.d_other >= kMidMinDegree &&
+        if (it.d_tab >= dbg && it.d_other >= dmd && it.d_other >= md_min &&
             it.d_other < d_hi)
           saved += (double)it.cost;
       if (saved > best) {  // ties keep the narrower shape
@@ -1503,7 +1529,8 @@ static gs_status build_hub_index(gs_graph* g, uint64_t budget, bool tables, cuda
   // ---- table slot of every adjacency entry (cost pass), if the budget has
   // room left after everything above
   const size_t tb_bytes_col = sizeof(int32_t) * (size_t)g->dev.nnz;
-  if (g->dev.tb_count > 1 && g->dev.nnz > 0 && (double)budget >= used + (double)tb_bytes_col) {
+  if (held == 0 && g->dev.tb_count > 1 && g->dev.nnz > 0 &&
+      (double)budget >= used + (double)tb_bytes_col) {
     cudaError_t ae = cudaMalloc(&g->col_tb, tb_bytes_col);
     if (ae != cudaSuccess) return cuda_fail(ae, "adjacency table slots", __FILE__, __LINE__);
     k_col_tb<<<grid_for(g->dev.nnz, 256, 8), 256, 0, stream>>>(g->dev.col, g->dev.nnz,
@@ -1520,13 +1547,14 @@ static gs_status build_hub_index(gs_graph* g, uint64_t budget, bool tables, cuda
 // [h_first[i], h_first[i + 1]) of at most kDenseGraphMax vertices: member
 // graphs of a disjoint union, or one graph. Both are accelerators: skipped
 // silently when too large or when the allocation fails. *cg_bytes: size of
-// the co-degree blocks built; *whole: they cover every range.
+// the co-degree blocks built; *held: co-degrees below this need no tables (0:
+// some range has no block; INT64_MAX: too few pairs are past the blocks).
 static gs_status build_dense_blocks(gs_graph* g, const int64_t* h_first, int64_t ranges,
                                     uint64_t max_bits, uint64_t max_cg, cudaStream_t stream,
-                                    uint64_t* cg_bytes, bool* whole) {
+                                    uint64_t* cg_bytes, int64_t* held) {
   const int64_t n = g->dev.n;
   *cg_bytes = 0;
-  *whole = false;
+  *held = 0;
   if (n == 0 || ranges <= 0) return GS_OK;
   std::vector<int64_t> row(n, -1), cg_row(n, -1);
   std::vector<int32_t> first(n, 0), len16(n, 0);
@@ -1578,7 +1606,7 @@ static gs_status build_dense_blocks(gs_graph* g, const int64_t* h_first, int64_t
   int32_t* d_len = nullptr;
   if (cudaMalloc(&g->cg, (size_t)cg_total) != cudaSuccess ||
       cudaMalloc(&g->cg_row, sizeof(int64_t) * (size_t)n) != cudaSuccess ||
-      cudaMalloc(&d_len, sizeof(int32_t) * (size_t)n) != cudaSuccess) {
+      cudaMalloc(&d_len, sizeof(int32_t) * ((size_t)n + 4)) != cudaSuccess) {
     cudaGetLastError();
     cudaFree(g->cg);
     cudaFree(g->cg_row);
@@ -1586,24 +1614,31 @@ static gs_status build_dense_blocks(gs_graph* g, const int64_t* h_first, int64_t
     g->cg_row = nullptr;
     return GS_OK;
   }
+  // two totals, then the row lengths
+  unsigned long long* d_totals = reinterpret_cast<unsigned long long*>(d_len);
+  unsigned long long totals[2] = {0, 0};
   cudaError_t e = cudaMemcpyAsync(g->cg_row, cg_row.data(), sizeof(int64_t) * n,
                                   cudaMemcpyHostToDevice, stream);
+  if (e == cudaSuccess) e = cudaMemsetAsync(d_totals, 0, sizeof(totals), stream);
   if (e == cudaSuccess)
-    e = cudaMemcpyAsync(d_len, len16.data(), sizeof(int32_t) * n, cudaMemcpyHostToDevice, stream);
+    e = cudaMemcpyAsync(d_len + 4, len16.data(), sizeof(int32_t) * n, cudaMemcpyHostToDevice,
+                        stream);
   if (e == cudaSuccess) {
     const int64_t per_sm = std::min<int64_t>(2048 / kBlockRowThreads,
                                              ((int64_t)200 << 10) / (2 * longest + 1024));
     k_block_codeg<<<(unsigned)std::min<int64_t>(n, sm_count() * per_sm), kBlockRowThreads,
                     (size_t)(2 * longest), stream>>>(g->dev.row_ptr, g->dev.col, n, g->cg_row,
-                                                     g->dm_first, d_len, g->cg);
-    e = cudaStreamSynchronize(stream);
+                                                     g->dm_first, d_len + 4, g->cg, d_totals);
+    e = cudaMemcpyAsync(totals, d_totals, sizeof(totals), cudaMemcpyDeviceToHost, stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
   }
   cudaFree(d_len);
   if (e != cudaSuccess) return cuda_fail(e, "co-degree blocks", __FILE__, __LINE__);
   g->dev.cg = g->cg;
   g->dev.cg_row = g->cg_row;
   *cg_bytes = (uint64_t)cg_total;
-  *whole = all;
+  if (all)
+    *held = totals[1] > totals[0] / kMissedShare ? kBlockHeld : INT64_MAX;
   return GS_OK;
 }
 
@@ -1689,26 +1724,24 @@ gs_status gs::create_graph(const int64_t* d_row_ptr, const int32_t* d_col, int64
   }
   uint64_t budget = hub_budget_bytes == 0 ? (uint64_t)96 << 30 : hub_budget_bytes;
   gs_status hs = GS_OK;
-  bool tables = true;
+  int64_t held = 0;  // co-degrees below this are in the blocks
   if (h_first != nullptr || (n <= kDenseGraphMax && hub_budget_bytes != 1)) {
     // a small graph gets its whole adjacency as a bit matrix (Sec. 2.6 notes
     // adjacency matrices for small graphs) and its co-degrees, as far as a
     // quarter of the budget holds them (half of it for a batch, whose
-    // co-degree tables, between hubs of different graphs for the most part,
-    // are left out when the blocks cover every graph); a 1-byte budget turns
-    // every index structure of one graph off
+    // co-degree tables are cut to what the blocks do not hold when these cover
+    // every graph); a 1-byte budget turns every index structure of one graph off
     const int64_t one[2] = {0, n};
     uint64_t cg_bytes = 0;
-    bool whole = false;
     hs = build_dense_blocks(g, h_first != nullptr ? h_first : one, h_first != nullptr ? ranges : 1,
                             (uint64_t)(h_first != nullptr ? 24 << 10 : 64) << 20,
                             h_first != nullptr ? budget / 2 : budget / 4, stream, &cg_bytes,
-                            &whole);
+                            &held);
     if (hs != GS_OK) return fail(hs);
     budget -= cg_bytes;
-    tables = h_first == nullptr || !whole;
+    if (h_first == nullptr) held = 0;
   }
-  hs = build_hub_index(g, budget, tables, stream);
+  hs = build_hub_index(g, budget, held, stream);
   if (hs != GS_OK) return fail(hs);
   hs = build_oriented(g, stream);
   if (hs != GS_OK) return fail(hs);

@@ -62,11 +62,14 @@ __device__ __forceinline__ uint64_t splitmix(uint64_t x) {
 // vertices that its own subtractions expose at once, from a queue in shared
 // memory, and only what does not fit the queue goes to the next round.
 //
-// Bound by latency: a level is a few chains of dependent subtractions. The
-// host loop before (a launch and a wait per level and per round, one warp per
-// vertex) took 917 launches on the 100k-vertex power-law graph, 18 us each in
-// k_core_peel, where one warp walked a hub's 24,000 neighbours:
-// k-core numbers, 1% weighted sample and its estimates there: 27.1 -> 5.8 ms.
+// Bound by latency: a level is a few chains of dependent subtractions. A host
+// loop with a launch and a wait per level and per round, one warp per vertex,
+// took 917 launches on the 100k-vertex power-law graph (a hub's 24,000
+// neighbours were one warp's walk): core numbers 23.1 -> 3.7 ms. With few levels
+// it is the lists' traffic: entries are listed and counted once per warp, not by
+// two additions per vertex at one address, and the first level is the least
+// degree (4-regular graph of 8M vertices 10.1 -> 6.7 ms; 1.5 with the host loop),
+// and short entries share a warp's step (6.7 -> 1.2; R-MAT 22 9.4 -> 8.6).
 constexpr int kPeelThreads = 512;
 constexpr int64_t kPeelPart = 256;  // neighbours per removal entry
 constexpr int kPeelQueue = 16;      // queued vertices of a warp
@@ -130,10 +133,17 @@ __global__ void __launch_bounds__(kPeelThreads)
   const int64_t thread = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const int64_t threads = (int64_t)gridDim.x * blockDim.x;
   const int64_t warp = thread >> 5, warps = threads >> 5;
+  // the least degree of all is the first level; slot 3 keeps it until phase 1
+  unsigned long long first_k = ~0ull;
   for (int64_t v = thread; v < n; v += threads) {
-    deg[v] = (int32_t)(row_ptr[v + 1] - row_ptr[v]);
+    const int32_t d = (int32_t)(row_ptr[v + 1] - row_ptr[v]);
+    deg[v] = d;
     core[v] = -1;
+    first_k = min(first_k, (unsigned long long)d);
   }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) first_k = min(first_k, __shfl_xor_sync(kFull, first_k, o));
+  if (lane == 0 && first_k != ~0ull) atomicMin(&st->phase[3].least, first_k);
   // phase ph uses slot ph & 3; the slot of phase ph + 2 was last read before
   // the barrier that ended phase ph - 1, so it is cleared in phase ph
   int ph = 0;
@@ -150,25 +160,39 @@ __global__ void __launch_bounds__(kPeelThreads)
   if (!peel_barrier(st)) return;
   int64_t remaining = n;
   bool first = true;
-  int32_t k = 0;
+  int32_t k = (int32_t)__ldcg(&st->phase[3].least);
   while (remaining > 0) {
     // scan
     PeelPhase* p = begin();
     unsigned long long least = ~0ull;
+    unsigned out = 0;  // removed by the lane
     for (int64_t i0 = warp * 32; i0 < remaining; i0 += threads) {
       const int64_t i = i0 + lane;
       const int32_t v = i >= remaining ? -1 : first ? (int32_t)i : __ldcg(rem0 + i);
       bool stays = false;
+      int parts = 0;
       if (v >= 0 && __ldcg(core + v) == -1) {
         const int32_t d = __ldcg(deg + v);
         if (d <= k) {
           __stcg(core + v, k);
-          atomicAdd(&p->removed, 1ull);
-          list_removal(v, __ldg(row_ptr + v + 1) - __ldg(row_ptr + v), list0, &p->entries);
+          ++out;
+          parts = (int)((__ldg(row_ptr + v + 1) - __ldg(row_ptr + v) + kPeelPart - 1) / kPeelPart);
         } else {
           stays = true;
           least = min(least, (unsigned long long)d);
         }
+      }
+      if (__any_sync(kFull, parts > 0)) {  // one place in the list for the warp's entries
+        int upto = parts;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+          const int y = __shfl_up_sync(kFull, upto, o);
+          if (lane >= o) upto += y;
+        }
+        unsigned long long to = 0;
+        if (lane == 31) to = atomicAdd(&p->entries, (unsigned long long)upto);
+        to = __shfl_sync(kFull, to, 31) + (upto - parts);
+        for (int j = 0; j < parts; ++j) __stcg(list0 + to + j, make_int2(v, j));
       }
       const unsigned b = __ballot_sync(kFull, stays);
       unsigned long long at = 0;
@@ -179,6 +203,8 @@ __global__ void __launch_bounds__(kPeelThreads)
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) least = min(least, __shfl_xor_sync(kFull, least, o));
     if (lane == 0 && least != ~0ull) atomicMin(&p->least, least);
+    out = __reduce_add_sync(kFull, out);
+    if (lane == 0 && out) atomicAdd(&p->removed, (unsigned long long)out);
     if (!peel_barrier(st)) return;
     ++ph;
     remaining = (int64_t)__ldcg(&p->remaining);
@@ -200,37 +226,71 @@ __global__ void __launch_bounds__(kPeelThreads)
     int2* to = list1;
     while (entries > 0) {
       p = begin();
-      for (int64_t i = warp; i < entries; i += warps) {
-        int2 it = __ldcg(from + i);
+      // takes one from every remaining vertex among x; every look and every
+      // subtraction in flight at once (in a loop they were one chain of 24
+      // latencies)
+      constexpr int kEach = (int)(kPeelPart / 32);
+      auto take_away = [&](const int32_t (&x)[kEach]) {
+        int32_t old[kEach];
+#pragma unroll
+        for (int u = 0; u < kEach; ++u) old[u] = x[u] >= 0 ? __ldcg(core + x[u]) : 0;
+#pragma unroll
+        for (int u = 0; u < kEach; ++u) old[u] = old[u] == -1 ? atomicSub(deg + x[u], 1) : -1;
+#pragma unroll
+        for (int u = 0; u < kEach; ++u)
+          if (old[u] == k + 1) {
+            __stcg(core + x[u], k);
+            const int64_t d = __ldg(row_ptr + x[u] + 1) - __ldg(row_ptr + x[u]);
+            const int at = d <= kPeelPart ? atomicAdd(&queued[wid], 1) : kPeelQueue;
+            if (at < kPeelQueue) queue[wid][at] = x[u];
+            else list_removal(x[u], d, to, &p->entries);
+          }
+      };
+      auto part = [&](int32_t v, int32_t i) {
+        const int64_t b = __ldg(row_ptr + v) + (int64_t)i * kPeelPart;
+        const int64_t e = min(__ldg(row_ptr + v + 1), b + kPeelPart);
+        int32_t x[kEach];
+#pragma unroll
+        for (int u = 0; u < kEach; ++u)
+          x[u] = b + 32 * u + lane < e ? __ldg(col + b + 32 * u + lane) : -1;
+        take_away(x);
+      };
+      // with entries for all warps, a warp takes kEach of them at once: short
+      // ones fill the places of one part
+      const bool many = entries >= warps * kEach;
+      const int64_t step = many ? kEach : 1;
+      for (int64_t i = warp * step; i < entries; i += warps * step) {
         if (lane == 0) queued[wid] = 0;
         __syncwarp();
-        int head = 0;
-        for (;;) {
-          const int64_t b = __ldg(row_ptr + it.x) + (int64_t)it.y * kPeelPart;
-          const int64_t e = min(__ldg(row_ptr + it.x + 1), b + kPeelPart);
-          // every neighbour's load, look and subtraction of a part in flight
-          // at once (in a loop they were one chain of 24 latencies)
-          constexpr int kEach = (int)(kPeelPart / 32);
-          int32_t x[kEach], old[kEach];
+        if (many) {
+          int2 it = make_int2(-1, 0);
+          int64_t b = 0;
+          int32_t len = 0;
+          if (lane < kEach && i + lane < entries) {
+            it = __ldcg(from + i + lane);
+            b = __ldg(row_ptr + it.x) + (int64_t)it.y * kPeelPart;
+            len = (int32_t)min(__ldg(row_ptr + it.x + 1) - b, kPeelPart);
+          }
+          if (__all_sync(kFull, len <= 32)) {
+            int32_t x[kEach];
 #pragma unroll
-          for (int u = 0; u < kEach; ++u) x[u] = b + 32 * u + lane < e ? __ldg(col + b + 32 * u + lane) : -1;
-#pragma unroll
-          for (int u = 0; u < kEach; ++u) old[u] = x[u] >= 0 ? __ldcg(core + x[u]) : 0;
-#pragma unroll
-          for (int u = 0; u < kEach; ++u) old[u] = old[u] == -1 ? atomicSub(deg + x[u], 1) : -1;
-#pragma unroll
-          for (int u = 0; u < kEach; ++u)
-            if (old[u] == k + 1) {
-              __stcg(core + x[u], k);
-              const int64_t d = __ldg(row_ptr + x[u] + 1) - __ldg(row_ptr + x[u]);
-              const int at = d <= kPeelPart ? atomicAdd(&queued[wid], 1) : kPeelQueue;
-              if (at < kPeelQueue) queue[wid][at] = x[u];
-              else list_removal(x[u], d, to, &p->entries);
+            for (int u = 0; u < kEach; ++u) {
+              const int64_t bu = __shfl_sync(kFull, b, u);
+              x[u] = lane < __shfl_sync(kFull, len, u) ? __ldg(col + bu + lane) : -1;
             }
+            take_away(x);
+          } else {
+            for (int u = 0; u < kEach && i + u < entries; ++u)
+              part(__shfl_sync(kFull, it.x, u), __shfl_sync(kFull, it.y, u));
+          }
+        } else {
+          const int2 it = __ldcg(from + i);
+          part(it.x, it.y);
+        }
+        for (int head = 0;; ++head) {
           __syncwarp();
           if (head >= min(queued[wid], kPeelQueue)) break;
-          it = make_int2(queue[wid][head], 0);
-          ++head;
+          part(queue[wid][head], 0);
         }
         __syncwarp();
       }
@@ -549,8 +609,9 @@ extern "C" gs_status gs_core_numbers(const gs_graph* gr, gs_workspace* ws, int32
   for (PeelPhase& p : init.phase) p.least = ~0ull;
   GS_CUDA(cudaMemcpyAsync(st, &init, sizeof(init), cudaMemcpyHostToDevice, stream));
   // every block resident at once (the blocks wait on one another): at most
-  // one per SM (two make the barriers dearer: 9.1 against 8.8 ms on the
-  // 100k-vertex power-law graph), fewer for a small graph
+  // one per SM (two make the barriers dearer: 9.1 against 8.8 ms for core
+  // numbers, a weighted sample and its estimates on the 100k-vertex power-law
+  // graph, before removals had all loads in flight), fewer for a small graph
   int per_sm = 0;
   GS_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_core_peel, kPeelThreads, 0));
   const int64_t most = (int64_t)sm_count() * std::min(per_sm, 1);

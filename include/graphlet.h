@@ -258,6 +258,12 @@ gs_status gs_workspace_set_tuning(gs_workspace* ws, int tri_blocks_per_sm, int q
  * gs_workspace_set_tuning. */
 gs_status gs_workspace_set_dense_slots(gs_workspace* ws, int64_t slots);
 
+/* Grid-wide waits (gs_core_numbers): a block that has looked this many times
+ * (at least 100 ns each) for the others gives up, every block returns and the
+ * call returns GS_ETIMEOUT. Default 2^28; a round between two waits takes
+ * milliseconds. GS_EINVAL for a NULL workspace or looks < 0. */
+gs_status gs_workspace_set_wait_limit(gs_workspace* ws, int64_t looks);
+
 /* Host output: statistics of the last gs_count that used `ws`. */
 gs_status gs_count_stats(const gs_workspace* ws, gs_stats* out);
 
@@ -409,8 +415,11 @@ gs_status gs_sample_ranks(const gs_graph* g, gs_workspace* ws, int64_t k_lo, int
  * k-core numbers: d_core (device int32[n]) receives the largest k such that
  * v lies in a subgraph whose every vertex has degree >= k (the weights of
  * the k-core distribution that Sec. 7 uses for the extremal problem);
- * *h_max_core (host, may be NULL) the largest. Parallel peeling; uses the
- * workspace; synchronises `stream`. */
+ * *h_max_core (host, may be NULL) the largest. Parallel peeling in one
+ * cooperative launch; takes 28 n + nnz / 16 bytes of the workspace;
+ * synchronises `stream`. GS_ETIMEOUT when a grid-wide wait ran out (see
+ * gs_workspace_set_wait_limit): d_core and *h_max_core are then undefined and
+ * the workspace stays usable. */
 gs_status gs_core_numbers(const gs_graph* g, gs_workspace* ws, int32_t* d_core,
                           int32_t* h_max_core, void* stream);
 

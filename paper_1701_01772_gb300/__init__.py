@@ -209,6 +209,7 @@ def lib() -> ctypes.CDLL:
         "gs_workspace_set_tuning": ([P, ctypes.c_int, ctypes.c_int, I64, ctypes.c_int],
                                     ctypes.c_int32),
         "gs_workspace_set_dense_slots": ([P, I64], ctypes.c_int32),
+        "gs_workspace_set_wait_limit": ([P, I64], ctypes.c_int32),
         "gs_sums_merge": ([ctypes.POINTER(GsSums), ctypes.POINTER(GsSums)], ctypes.c_int32),
         "gs_batch_create": ([P, P, P, I64, I64, I64, U32, U32, U64, P, PP], ctypes.c_int32),
         "gs_batch_count": ([P, ctypes.POINTER(GsSums), P], ctypes.c_int32),
@@ -389,6 +390,10 @@ def gs_workspace_set_tuning(handle: int, tri_blocks_per_sm: int, quad_blocks_per
 
 def gs_workspace_set_dense_slots(handle: int, slots: int) -> None:
     _check(lib().gs_workspace_set_dense_slots(handle, slots))
+
+
+def gs_workspace_set_wait_limit(handle: int, looks: int) -> None:
+    _check(lib().gs_workspace_set_wait_limit(handle, looks))
 
 
 def gs_batch_create(vtx_off, row_ptr, col, mask: int = GS_CONNECTED, flags: int = GS_VALIDATE,
@@ -616,6 +621,9 @@ class Workspace:
 
     def set_dense_slots(self, slots: int) -> None:
         gs_workspace_set_dense_slots(self.handle, slots)
+
+    def set_wait_limit(self, looks: int) -> None:
+        gs_workspace_set_wait_limit(self.handle, looks)
 
     def stats(self) -> dict:
         return gs_count_stats(self.handle).as_dict()

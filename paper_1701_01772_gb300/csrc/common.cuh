@@ -439,6 +439,8 @@ struct gs_workspace {
   gs_stats stats;       // last gs_count
   int64_t launches_total;
   void* staging;        // page-locked host bytes for the small read-backs
+  int has_wait_limit;
+  int64_t wait_limit;   // looks of a grid-wide wait
 };
 
 namespace gs {

@@ -74,7 +74,9 @@ constexpr int kPeelThreads = 512;
 constexpr int64_t kPeelPart = 256;  // neighbours per removal entry
 constexpr int kPeelQueue = 16;      // queued vertices of a warp
 // Looks at the barrier counter before a block gives up on the others (each
-// takes at least 100 ns, so at least 25 s).
+// takes at least 100 ns, so at least 25 s; a round of removals is over in
+// milliseconds, since a warp's queue does not wrap: a long path goes on in the
+// next round after kPeelQueue steps).
 constexpr int64_t kPeelSpins = (int64_t)1 << 28;
 
 // Counters of one phase (a scan or a round of removals).
@@ -94,7 +96,7 @@ struct PeelState {
 
 // Grid-wide barrier of a cooperative launch. False (in every thread of the
 // block) when it ran out of looks or another block did.
-__device__ __forceinline__ bool peel_barrier(PeelState* st) {
+__device__ __forceinline__ bool peel_barrier(PeelState* st, int64_t most) {
   __shared__ int ok;
   __syncthreads();
   if (threadIdx.x == 0) {
@@ -105,7 +107,7 @@ __device__ __forceinline__ bool peel_barrier(PeelState* st) {
     volatile unsigned long long* arrived = &st->arrived;
     volatile int32_t* failed = &st->failed;
     int64_t looks = 0;
-    while (*arrived < all && *failed == 0 && looks < kPeelSpins) ++looks;
+    while (*arrived < all && *failed == 0 && looks < most) ++looks;
     if (*arrived < all) *failed = 1;
     ok = *failed == 0;
     __threadfence();
@@ -126,7 +128,7 @@ __device__ __forceinline__ void list_removal(int32_t v, int64_t d, int2* __restr
 __global__ void __launch_bounds__(kPeelThreads)
     k_core_peel(const int64_t* __restrict__ row_ptr, const int32_t* __restrict__ col, int64_t n,
                 int32_t* __restrict__ deg, int32_t* __restrict__ core, int32_t* rem0,
-                int32_t* rem1, int2* list0, int2* list1, PeelState* st) {
+                int32_t* rem1, int2* list0, int2* list1, PeelState* st, int64_t most) {
   __shared__ int32_t queue[kPeelThreads / 32][kPeelQueue];
   __shared__ int32_t queued[kPeelThreads / 32];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -157,7 +159,7 @@ __global__ void __launch_bounds__(kPeelThreads)
     }
     return &st->phase[ph & 3];
   };
-  if (!peel_barrier(st)) return;
+  if (!peel_barrier(st, most)) return;
   int64_t remaining = n;
   bool first = true;
   int32_t k = (int32_t)__ldcg(&st->phase[3].least);
@@ -205,7 +207,7 @@ __global__ void __launch_bounds__(kPeelThreads)
     if (lane == 0 && least != ~0ull) atomicMin(&p->least, least);
     out = __reduce_add_sync(kFull, out);
     if (lane == 0 && out) atomicAdd(&p->removed, (unsigned long long)out);
-    if (!peel_barrier(st)) return;
+    if (!peel_barrier(st, most)) return;
     ++ph;
     remaining = (int64_t)__ldcg(&p->remaining);
     const unsigned long long low = __ldcg(&p->least);
@@ -294,7 +296,7 @@ __global__ void __launch_bounds__(kPeelThreads)
         }
         __syncwarp();
       }
-      if (!peel_barrier(st)) return;
+      if (!peel_barrier(st, most)) return;
       ++ph;
       entries = (int64_t)__ldcg(&p->entries);
       int2* l = from;
@@ -579,6 +581,16 @@ double i128_to_double(u128 v) {  // two's complement
 
 }  // namespace
 
+extern "C" gs_status gs_workspace_set_wait_limit(gs_workspace* ws, int64_t looks) {
+  if (ws == nullptr || looks < 0) {
+    set_error("gs_workspace_set_wait_limit: null workspace or negative limit");
+    return GS_EINVAL;
+  }
+  ws->has_wait_limit = 1;
+  ws->wait_limit = looks;
+  return GS_OK;
+}
+
 extern "C" gs_status gs_core_numbers(const gs_graph* gr, gs_workspace* ws, int32_t* d_core,
                                      int32_t* h_max_core, void* stream_) {
   cudaStream_t stream = (cudaStream_t)stream_;
@@ -620,7 +632,9 @@ extern "C" gs_status gs_core_numbers(const gs_graph* gr, gs_workspace* ws, int32
   const int64_t* row_ptr = gr->dev.row_ptr;
   const int32_t* col = gr->dev.col;
   int64_t n_arg = n;
-  void* args[] = {&row_ptr, &col, &n_arg, &deg, &d_core, &rem0, &rem1, &list0, &list1, &st};
+  int64_t limit = ws->has_wait_limit ? ws->wait_limit : kPeelSpins;
+  void* args[] = {&row_ptr, &col,   &n_arg, &deg, &d_core, &rem0,
+                  &rem1,    &list0, &list1, &st,  &limit};
   GS_CUDA(cudaLaunchCooperativeKernel((const void*)k_core_peel, dim3(blocks), dim3(kPeelThreads),
                                       args, 0, stream));
   ws->launches_total += 1;

@@ -564,7 +564,7 @@ extern "C" gs_status gs_micro(const gs_graph* gr, gs_workspace* ws, const int32_
               (long long)herr.index);
     return herr.code;
   }
-  int64_t launches = 5;
+  int64_t launches = 2 + scan_launches(K);
   if (C > 0) {
     const size_t mid = Carve::bytes_for<int64_t>(C) + Carve::bytes_for<uint32_t>(2 * C) +
                        Carve::bytes_for<int64_t>(C + 1) +
@@ -582,7 +582,7 @@ extern "C" gs_status gs_micro(const gs_graph* gr, gs_workspace* ws, const int32_
     GS_TRY(exclusive_scan_i64(task_off, task_off, C, tmp1, stream));
     k_micro_probe<<<sm_count() * kProbeBlocksPerSm, kThreads, 0, stream>>>(
         g, uv, choff, chunk_e, tmask, task_off, C, p_e, seed, acc, stats + 1);
-    launches += 8;
+    launches += 3 + scan_launches(C);
   }
   k_micro_final<<<final_blocks, kThreads, 0, stream>>>(
       g.row_ptr, uv, K, n, m, cn3, cn4, t, acc, d_x,

@@ -126,9 +126,10 @@ const char* gs_version(void);
  * table |N(a) cap N(b)| among the top vertices, plus a mid x big co-degree
  * table, adjacency bucket directories and degree-oriented adjacency lists
  * for the exact 3-node pass, see gs_graph_index_info; graphs of at most
- * 16384 vertices also get their adjacency as a bit matrix and an 8-bit
- * co-degree matrix in up to a quarter of the budget) in library-owned
- * device memory;
+ * 16384 vertices also get an 8-bit co-degree matrix in up to a quarter of the
+ * budget, in a batch half of it, and, outside the budget, their adjacency as
+ * a bit matrix of at most 32 MiB, in a batch 24 GiB in all; both give way to
+ * the rest when memory is short) in library-owned device memory;
  * hub_budget_bytes bounds that index (0 = default 96 GiB, a third of the
  * GPU, for one large resident graph; pass less when several graphs share
  * the device): bitmaps and matrix up to 1/8 each, directories up to 1/16,

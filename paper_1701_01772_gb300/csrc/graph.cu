@@ -1642,9 +1642,16 @@ static gs_status build_dense_blocks(gs_graph* g, const int64_t* h_first, int64_t
   return GS_OK;
 }
 
-gs_status gs::create_graph(const int64_t* d_row_ptr, const int32_t* d_col, int64_t n, int64_t nnz,
-                           uint32_t flags, uint64_t hub_budget_bytes, const int64_t* h_first,
-                           int64_t ranges, cudaStream_t stream, gs_graph** out) {
+// One attempt at a registration. *blocks: in, build the optional blocks of small
+// graphs before the index, which then leaves out what they hold (false: bit
+// matrices alone, after it, in what memory is left); out, whether any were built
+// before it.
+static gs_status register_graph(const int64_t* d_row_ptr, const int32_t* d_col, int64_t n,
+                                int64_t nnz, uint32_t flags, uint64_t hub_budget_bytes,
+                                const int64_t* h_first, int64_t ranges, bool* blocks,
+                                cudaStream_t stream, gs_graph** out) {
+  const bool first = *blocks;
+  *blocks = false;
   if (out == nullptr || d_row_ptr == nullptr || n < 0 || nnz < 0 || (nnz > 0 && d_col == nullptr)) {
     set_error("gs_graph_create: invalid arguments");
     return GS_EINVAL;
@@ -1725,28 +1732,53 @@ gs_status gs::create_graph(const int64_t* d_row_ptr, const int32_t* d_col, int64
   uint64_t budget = hub_budget_bytes == 0 ? (uint64_t)96 << 30 : hub_budget_bytes;
   gs_status hs = GS_OK;
   int64_t held = 0;  // co-degrees below this are in the blocks
-  if (h_first != nullptr || (n <= kDenseGraphMax && hub_budget_bytes != 1)) {
-    // a small graph gets its whole adjacency as a bit matrix (Sec. 2.6 notes
-    // adjacency matrices for small graphs) and its co-degrees, as far as a
-    // quarter of the budget holds them (half of it for a batch, whose
-    // co-degree tables are cut to what the blocks do not hold when these cover
-    // every graph); a 1-byte budget turns every index structure of one graph off
-    const int64_t one[2] = {0, n};
+  // a small graph gets its whole adjacency as a bit matrix (Sec. 2.6 notes
+  // adjacency matrices for small graphs) and its co-degrees, as far as a
+  // quarter of the budget holds them (half of it for a batch, whose co-degree
+  // tables are cut to what the blocks do not hold when these cover every
+  // graph); a 1-byte budget turns every index structure of one graph off
+  const bool batch = h_first != nullptr;
+  const int64_t one[2] = {0, n};
+  auto build_blocks = [&](uint64_t max_cg) {
     uint64_t cg_bytes = 0;
-    hs = build_dense_blocks(g, h_first != nullptr ? h_first : one, h_first != nullptr ? ranges : 1,
-                            (uint64_t)(h_first != nullptr ? 24 << 10 : 64) << 20,
-                            h_first != nullptr ? budget / 2 : budget / 4, stream, &cg_bytes,
-                            &held);
-    if (hs != GS_OK) return fail(hs);
+    const gs_status s = build_dense_blocks(g, batch ? h_first : one, batch ? ranges : 1,
+                                           (uint64_t)(batch ? 24 << 10 : 64) << 20, max_cg, stream,
+                                           &cg_bytes, &held);
     budget -= cg_bytes;
-    if (h_first == nullptr) held = 0;
+    return s;
+  };
+  const bool small = batch || (n <= kDenseGraphMax && hub_budget_bytes != 1);
+  if (small && first) {
+    hs = build_blocks(batch ? budget / 2 : budget / 4);
+    if (hs != GS_OK) return fail(hs);
+    *blocks = g->dm_bits != nullptr;
+    if (!batch) held = 0;
   }
   hs = build_hub_index(g, budget, held, stream);
   if (hs != GS_OK) return fail(hs);
   hs = build_oriented(g, stream);
   if (hs != GS_OK) return fail(hs);
+  if (small && !first) {
+    hs = build_blocks(0);
+    if (hs != GS_OK) return fail(hs);
+  }
   *out = g;
   return GS_OK;
+}
+
+gs_status gs::create_graph(const int64_t* d_row_ptr, const int32_t* d_col, int64_t n, int64_t nnz,
+                           uint32_t flags, uint64_t hub_budget_bytes, const int64_t* h_first,
+                           int64_t ranges, cudaStream_t stream, gs_graph** out) {
+  bool blocks = true;
+  gs_status s = register_graph(d_row_ptr, d_col, n, nnz, flags, hub_budget_bytes, h_first, ranges,
+                               &blocks, stream, out);
+  if (s == GS_ENOMEM && blocks) {  // the index goes before the blocks, which are optional
+    cudaGetLastError();
+    blocks = false;
+    s = register_graph(d_row_ptr, d_col, n, nnz, flags, hub_budget_bytes, h_first, ranges, &blocks,
+                       stream, out);
+  }
+  return s;
 }
 
 extern "C" gs_status gs_graph_create(const int64_t* d_row_ptr, const int32_t* d_col, int64_t n,

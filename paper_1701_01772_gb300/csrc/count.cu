@@ -1829,8 +1829,8 @@ __global__ void k_fold_seg_final(const unsigned long long* __restrict__ limbs, i
 // =================================================================== host side
 namespace gs {
 
-// 8 triangle-pass CTAs per SM (32 registers) and 512-test tasks: measured
-// best on the 1M-vertex power-law graph (triangle pass 79 -> 47 ms exact).
+// 8 triangle-pass CTAs per SM (k_tri, 32 registers; k_tri_chunks takes at most
+// kTriBlocksPerSm) and tasks of 512 tests.
 Tuning default_tuning() { return Tuning{8, kQuadBlocksPerSm, 512, 1, kHubDenseSlots}; }
 
 int quad_blocks_limit() { return kQuadBlocksPerSm; }
@@ -1960,14 +1960,18 @@ int64_t launch_front(const gs_graph* gr, const DevGraph& g, const int32_t* pairs
 
 int64_t launch_tri(const DevGraph& g, bool four, const Tuning& tu, CountBufs& b,
                    cudaStream_t stream) {
-  const int grid = sm_count() * tu.tri_blocks_per_sm;
+  const int sms = sm_count(), grid = sms * tu.tri_blocks_per_sm;
+  // no more CTAs than are resident: a small call gives each of their warps a run
+  const int chunk_grid = sms * std::min(tu.tri_blocks_per_sm, kTriBlocksPerSm);
   if (four) {
-    k_tri_chunks<<<grid, kThreads, 0, stream>>>(g, b.uv, b.off, b.K, b.t, b.tbits, b.stats + 10);
+    k_tri_chunks<<<chunk_grid, kThreads, 0, stream>>>(g, b.uv, b.off, b.K, b.t, b.tbits,
+                                                      b.stats + 10);
   } else if (b.P >= kManyPositions && b.P >= kLongLists * b.K) {
     // toff is free in 3-node work: the padded offsets
     k_pad_lengths<<<grid_for(b.K, kThreads, 8), kThreads, 0, stream>>>(b.off, b.K, b.toff);
     exclusive_scan_i64(b.toff, b.toff, b.K, b.tmp0, stream);
-    k_tri_chunks<<<grid, kThreads, 0, stream>>>(g, b.uv, b.toff, b.K, b.t, nullptr, b.stats + 10);
+    k_tri_chunks<<<chunk_grid, kThreads, 0, stream>>>(g, b.uv, b.toff, b.K, b.t, nullptr,
+                                                      b.stats + 10);
     return 2 + scan_launches(b.K);
   } else {
     k_tri<<<grid, kThreads, 0, stream>>>(g, b.uv, b.off, b.K, b.t);

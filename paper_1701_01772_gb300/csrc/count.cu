@@ -118,14 +118,15 @@ __device__ __forceinline__ uint32_t tfilter_hash(int32_t x) {
 #endif
 constexpr int64_t kQuadGrabTests = GS_QUAD_GRAB_TESTS;
 // Resident warps per SM of k_dense_pairs (at most 40 registers), in CTAs of
-// 256 threads, or of 128 when there are many units: a unit has nine barriers,
-// at which the warps of a small CTA wait less, but a unit with long lists of
-// other members is walked by fewer warps. 1M-vertex power-law graph exact
-// (3.4M units) 374 ms with 256 threads, 358 with 128; R-MAT 24 0.1% (19,000
-// units) 147 and 154 ms, the 1% estimate of the former (34,000 units) 5.70 and
-// 5.79 ms. The line lies at 256 dense edges per resident CTA of 256.
+// 256 threads, or of 128 when there are many units: the five to seven barriers
+// of a unit hold up the warps of a small CTA less, but a unit with long lists of
+// other members is walked by fewer warps. 4-node phase with 128 and with 256
+// threads, 1M-vertex power-law graph: 34,000 dense edges 1.90 and 1.82 ms,
+// 68,000 3.21 and 3.29, 169,000 7.18 and 7.81, 1.7M 65.1 and 73.2; R-MAT 22:
+// 34,000 8.12 and 7.78, 85,000 17.92 and 17.85, 169,000 32.8 and 34.1. The line
+// lies at kManyDensePerCta dense edges per resident CTA of 256 (73,000 in all).
 constexpr int kDenseWarpsPerSm = 48;
-constexpr int64_t kManyDenseEdges = 256 * 6 * 152;
+constexpr int64_t kManyDensePerCta = 80;
 constexpr int kTriBlocksPerSm = 6;  // k_tri_chunks: at most 40 registers
 // T entries per k_dense_pairs work unit (a heavy dense edge is split into
 // several units so that small samples still fill the GPU).
@@ -2020,7 +2021,8 @@ int64_t launch_dense(const DevGraph& g, bool need_q, CountBufs& b, cudaStream_t 
         g, b.toff, b.t, b.T, b.T_hm, b.tmask, b.dense_e, b.unit_off, b.unit_idx, b.ndense,
         need_q ? 1 : 0, b.k2, b.q, b.stats + 7, b.stats + 4, b.stats + 9);
   };
-  if (b.ndense >= kManyDenseEdges) go(k_dense_pairs<128>, 128);
+  const int64_t resident = (int64_t)sm_count() * (kDenseWarpsPerSm * 32 / 256);
+  if (b.ndense >= kManyDensePerCta * resident) go(k_dense_pairs<128>, 128);
   else go(k_dense_pairs<256>, 256);
   return 1;
 }

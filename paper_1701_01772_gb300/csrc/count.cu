@@ -369,11 +369,15 @@ constexpr int kCompactBlocksPerSm = 5;
 // few edges the longest list is the pass's tail; with many, warps are never
 // short of edges and the CTA's barriers only cost. Compact phase at 1024 /
 // 2048 / 4096 / no limit: adaptive estimation on R-MAT 18 (61 to 2,000 edges a
-// pass) 2.46 / 2.57 / 2.59 / 2.90 ms the whole call, 1M-vertex power-law graph
-// 1% (200,000 edges) 1.07 / 0.88 / 0.91 / 1.17 ms, exact (20M edges) 67 / 51 /
-// 44 / 38 ms.
+// pass) 2.46 / 2.57 / 2.59 / 2.90 ms the whole call; R-MAT 22 19,000 edges 0.37 /
+// 0.36 / 0.38 / 1.49 ms, 64,000 0.68 / 0.64 / 0.62 / 2.6, 193,000 1.67 / 1.53 /
+// 1.27 / 2.9, 1.9M 15.0 / 13.9 / 10.6 / 11.2; 1M-vertex power-law graph 100,000
+// edges 0.64 / 0.53 / 0.60 / 1.85, 200,000 1.01 / 0.81 / 0.78 / 2.25, 1.0M 4.2 /
+// 3.1 / 2.6 / 3.8, 2.0M 8.1 / 6.5 / 5.5 / 6.0, 5M 18.3 / 13.9 / 11.8 / 11.2,
+// exact (20M) 66 / 49 / 42 / 35. Without a limit short lists go to single lanes
+// (ER of mean degree 4, 4M edges 1.5 -> 0.13), so that begins at 2^21 already.
 inline int64_t compact_long(int64_t K) {
-  return K < (1 << 15) ? 1024 : K < (1 << 21) ? 2048 : INT64_MAX;
+  return K < (1 << 15) ? 1024 : K < (1 << 17) ? 2048 : K < (1 << 21) ? 4096 : INT64_MAX;
 }
 
 // What k_compact_T shares of the edges in work: one per warp, the first one's

@@ -150,10 +150,6 @@ __device__ __forceinline__ T warp_sum(T v) {
 }
 
 
-// Bits [0, x) of a word, x clamped to 0..32.
-__device__ __forceinline__ unsigned bits_below(int32_t x) {
-  return x <= 0 ? 0u : x >= 32 ? kFull : (1u << x) - 1u;
-}
 
 __device__ __forceinline__ int64_t deg_of(const int64_t* __restrict__ row_ptr, int32_t v,
                                           int64_t* base) {
@@ -1419,6 +1415,10 @@ __device__ __forceinline__ const int16_t* slots_beside(const DevGraph& g, const 
 // work there (850 of 1390 warp instructions per chunk). Eight CTAs per SM at
 // 32 registers, some spilled, hide more latency than six at 40 (R-MAT 24
 // 0.1%: 151 against 160 ms; 1M-vertex power-law exact 456 against 457 ms).
+// The look for a run is left out where no item of the pack has one: a uniform
+// graph's items have a few dozen tests, and the look and the hit masks made the
+// phase slower than five shuffles per test had been (ER of mean degree 20 / 40,
+// 4M edges exact 13.3 / 50.5 -> 12.3 / 46.9 ms).
 __global__ void __launch_bounds__(kThreads, kQuadBlocksPerSm)
     k_quad(const __grid_constant__ DevGraph g, const int2* __restrict__ uv, const int64_t* __restrict__ off, int64_t K,
            const unsigned long long* __restrict__ t, const int64_t* __restrict__ toff,
@@ -1497,6 +1497,8 @@ __global__ void __launch_bounds__(kThreads, kQuadBlocksPerSm)
       const int64_t ctotal = __shfl_sync(kFull, start, 31);
       start -= mine;
       unsigned long long acc_a = 0, acc_b = 0;  // hits of the lane's item
+      const bool runs = __any_sync(
+          kFull, lane < live && (my->ca[lane] >= 64 || mine - my->ca[lane] >= 64));
       for (; here > 0; --here, ++task) {
         const int64_t lo = (task - __ldg(task_off + gi)) * task_probes;
         const int32_t len = (int32_t)min(ctotal - lo, task_probes);
@@ -1514,51 +1516,53 @@ __global__ void __launch_bounds__(kThreads, kQuadBlocksPerSm)
           // item of test r: the last one that starts at or before it (lanes
           // past the items hold the total, which is at or past len)
           const int j0 = 31 - __clz(__ballot_sync(kFull, srel <= r));
-          const int32_t sj = __shfl_sync(kFull, srel, j0);
-          const int32_t sbj = __shfl_sync(kFull, sb, j0);
-          const int32_t sej = __shfl_sync(kFull, se, j0);
-          const int sg = r >= sbj ? 1 : 0;
-          const int32_t end = sg ? sej : min(sbj, len);
-          if (end - r >= 64) {
-            const int32_t* it = my->it[sg][j0] + (r - (sg ? sbj : sj)) + lane;
-            const int32_t* sl = my->sl[sg][j0];
-            const int32_t sbm = my->sbm[sg][j0], slen = my->slen[sg][j0];
-            const int sslot = my->sslot[sg][j0];
-            unsigned hits = 0;
-            const int32_t n = (end - r) & ~63;
-            r += n;
-            if (sslot >= 0) {
-              const int16_t* hs = slots_beside(g, it, T, T_hm);
-              for (int32_t i = 0; i < n; i += 64) {
-                const int32_t x0 = __ldg(it + i), x1 = __ldg(it + i + 32);
-                int32_t s0, s1;
-                if (hs != nullptr) {
-                  s0 = __ldg(hs + i);
-                  s1 = __ldg(hs + i + 32);
-                } else {
-                  s0 = __ldg(g.hm_slot + x0);
-                  s1 = __ldg(g.hm_slot + x1);
+          if (runs) {  // some segment has 64 tests
+            const int32_t sj = __shfl_sync(kFull, srel, j0);
+            const int32_t sbj = __shfl_sync(kFull, sb, j0);
+            const int32_t sej = __shfl_sync(kFull, se, j0);
+            const int sg = r >= sbj ? 1 : 0;
+            const int32_t end = sg ? sej : min(sbj, len);
+            if (end - r >= 64) {
+              const int32_t* it = my->it[sg][j0] + (r - (sg ? sbj : sj)) + lane;
+              const int32_t* sl = my->sl[sg][j0];
+              const int32_t sbm = my->sbm[sg][j0], slen = my->slen[sg][j0];
+              const int sslot = my->sslot[sg][j0];
+              unsigned hits = 0;
+              const int32_t n = (end - r) & ~63;
+              r += n;
+              if (sslot >= 0) {
+                const int16_t* hs = slots_beside(g, it, T, T_hm);
+                for (int32_t i = 0; i < n; i += 64) {
+                  const int32_t x0 = __ldg(it + i), x1 = __ldg(it + i + 32);
+                  int32_t s0, s1;
+                  if (hs != nullptr) {
+                    s0 = __ldg(hs + i);
+                    s1 = __ldg(hs + i + 32);
+                  } else {
+                    s0 = __ldg(g.hm_slot + x0);
+                    s1 = __ldg(g.hm_slot + x1);
+                  }
+                  const Probe p0 = probe_begin<true>(g, sslot, sbm, sl, slen, x0, s0);
+                  const Probe p1 = probe_begin<true>(g, sslot, sbm, sl, slen, x1, s1);
+                  hits += probe_end(p0, sl, slen, x0);
+                  hits += probe_end(p1, sl, slen, x1);
                 }
-                const Probe p0 = probe_begin<true>(g, sslot, sbm, sl, slen, x0, s0);
-                const Probe p1 = probe_begin<true>(g, sslot, sbm, sl, slen, x1, s1);
-                hits += probe_end(p0, sl, slen, x0);
-                hits += probe_end(p1, sl, slen, x1);
+              } else {
+                for (int32_t i = 0; i < n; i += 64) {
+                  const int32_t x0 = __ldg(it + i), x1 = __ldg(it + i + 32);
+                  const Probe p0 = probe_begin<false>(g, sslot, sbm, sl, slen, x0, -1);
+                  const Probe p1 = probe_begin<false>(g, sslot, sbm, sl, slen, x1, -1);
+                  hits += probe_end(p0, sl, slen, x0);
+                  hits += probe_end(p1, sl, slen, x1);
+                }
               }
-            } else {
-              for (int32_t i = 0; i < n; i += 64) {
-                const int32_t x0 = __ldg(it + i), x1 = __ldg(it + i + 32);
-                const Probe p0 = probe_begin<false>(g, sslot, sbm, sl, slen, x0, -1);
-                const Probe p1 = probe_begin<false>(g, sslot, sbm, sl, slen, x1, -1);
-                hits += probe_end(p0, sl, slen, x0);
-                hits += probe_end(p1, sl, slen, x1);
+              hits = __reduce_add_sync(kFull, hits);
+              if (lane == j0) {
+                if (sg) acc_b += hits;
+                else acc_a += hits;
               }
+              continue;
             }
-            hits = __reduce_add_sync(kFull, hits);
-            if (lane == j0) {
-              if (sg) acc_b += hits;
-              else acc_a += hits;
-            }
-            continue;
           }
           // item starts among the next 64 tests: bit b of m0 / m1 = test r + b
           // / r + 32 + b begins an item (items have tests, so starts differ)

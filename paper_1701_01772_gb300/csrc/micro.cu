@@ -228,11 +228,6 @@ __device__ __forceinline__ int probe_cat(const EndSet& su, const EndSet& sv, int
   return cls == kSu ? 2 : above ? 1 : -1;           // 4-cycle; S_v pair
 }
 
-// Bits [0, x) of a word, x clamped to 0..32.
-__device__ __forceinline__ unsigned bits_below(int32_t x) {
-  return x <= 0 ? 0u : x >= 32 ? kFull : (1u << x) - 1u;
-}
-
 // Probes. A chunk's probes (its items in order) are one index space cut into
 // tasks; warps take runs of tasks from a counter. From probe r on a warp walks
 // either a run of 32 or more probes of one item (its descriptor is the same in

@@ -368,7 +368,7 @@ constexpr int64_t kBlockHeld = 255;  // co-degrees below this are held
 // 1,100 vertices and half of the pairs, nearly all of them past the blocks, 291
 // / 12.6 (27.6 with 16-bit tables alone).
 constexpr unsigned long long kMissedShare = 512;
-__global__ void __launch_bounds__(kBlockRowThreads)
+__global__ void __launch_bounds__(kBlockRowThreads, 2048 / kBlockRowThreads)
     k_block_codeg(const int64_t* __restrict__ row_ptr, const int32_t* __restrict__ col, int64_t n,
                   const int64_t* __restrict__ cg_row, const int32_t* __restrict__ first,
                   const int32_t* __restrict__ row_len, uint8_t* __restrict__ cg,
@@ -1004,21 +1004,16 @@ static RowShape row_shape(size_t row, int least) {
   return RowShape{1024, sm / (row + 1024 * 16 + 2048) >= 2 ? 2 : 1};
 }
 
-// Launches kernel<threads> for the row shape with `smem` dynamic bytes.
-#define GS_LAUNCH_ROWS(kernel, least, smem, stream, ...)                                      \
-  [&]() -> cudaError_t {                                                                      \
-    const RowShape sh = row_shape(smem, least);                                                   \
-    auto go = [&](auto k) -> cudaError_t {                                                    \
-      cudaError_t le = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,   \
-                                            (int)(smem));                                     \
-      if (le != cudaSuccess) return le;                                                       \
-      k<<<sm_count() * sh.per_sm, sh.threads, smem, stream>>>(__VA_ARGS__);                   \
-      return cudaGetLastError();                                                              \
-    };                                                                                        \
-    return sh.threads == 256   ? go(kernel<256>)                                              \
-           : sh.threads == 512 ? go(kernel<512>)                                              \
-                               : go(kernel<1024>);                                            \
-  }()
+// Launches a row kernel with `smem` dynamic bytes.
+template <class K, class... A>
+static cudaError_t launch_rows(K kernel, const RowShape& sh, size_t smem, cudaStream_t stream,
+                               A... args) {
+  const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             (int)smem);
+  if (e != cudaSuccess) return e;
+  kernel<<<sm_count() * sh.per_sm, sh.threads, smem, stream>>>(args...);
+  return cudaGetLastError();
+}
 
 // Vertices of degree >= d for every d up to the largest degree + 1, from one
 // device histogram (a registration asks for about 80 such counts; a launch and
@@ -1336,9 +1331,9 @@ static gs_status build_hub_index(gs_graph* g, uint64_t budget, int64_t held, cud
       const size_t row_smem = sizeof(uint32_t) * (size_t)(n_tb / 2 + 1);
       cudaError_t e = cudaMemsetAsync(d_cnt, 0, sizeof(unsigned long long), stream);
       if (e == cudaSuccess)
-        e = GS_LAUNCH_ROWS(k_table_rows, 1024, row_smem, stream, g->dev.row_ptr, g->dev.col, hubs, n_tb,
-                           flag, lists, g->tb_giant, giants, g->tb_giant_codeg, g->tb_codeg,
-                           d_cnt);
+        e = launch_rows(k_table_rows<1024>, row_shape(row_smem, 1024), row_smem, stream,
+                        g->dev.row_ptr, g->dev.col, hubs, n_tb, flag, lists, g->tb_giant, giants,
+                        g->tb_giant_codeg, g->tb_codeg, d_cnt);
       if (e == cudaSuccess) {
         if (g->tb_giant != nullptr)
           k_mark_giant_pairs<<<grid_for(n_tb, 256, 8), 256, 0, stream>>>(g->tb_giant, n_tb, tb_w);
@@ -1511,9 +1506,13 @@ static gs_status build_hub_index(gs_graph* g, uint64_t budget, int64_t held, cud
         k_mid_row_vertex<<<grid_for(n, 256, 8), 256, 0, stream>>>(g->tb_slot, n, rows_v);
         const size_t row_smem = sizeof(uint32_t) * (size_t)((n_bg + 1) / 2);
         cudaError_t e = cudaMemsetAsync(d_cnt, 0, sizeof(unsigned long long), stream);
+        const RowShape shape = row_shape(row_smem, 256);
         if (e == cudaSuccess)
-          e = GS_LAUNCH_ROWS(k_mid_rows, 256, row_smem, stream, g->dev.row_ptr, g->dev.col, rows_v, rows,
-                             flag, blist, n_bg, g->md_codeg, d_cnt);
+          e = launch_rows(shape.threads == 256   ? k_mid_rows<256>
+                          : shape.threads == 512 ? k_mid_rows<512>
+                                                 : k_mid_rows<1024>,
+                          shape, row_smem, stream, g->dev.row_ptr, g->dev.col, rows_v, rows, flag,
+                          blist, n_bg, g->md_codeg, d_cnt);
         if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
         cudaFree(blist);
         cudaFree(rows_v);

@@ -365,12 +365,12 @@ constexpr int kCompactBlocksPerSm = 5;
 // few edges the longest list is the pass's tail; with many, warps are never
 // short of edges and the CTA's barriers only cost. Compact phase at 1024 /
 // 2048 / 4096 / no limit: adaptive estimation on R-MAT 18 (61 to 2,000 edges a
-// pass) 2.46 / 2.57 / 2.59 / 2.90 ms the whole call; R-MAT 22 19,000 edges 0.37 /
-// 0.36 / 0.38 / 1.49 ms, 64,000 0.68 / 0.64 / 0.62 / 2.6, 193,000 1.67 / 1.53 /
-// 1.27 / 2.9, 1.9M 15.0 / 13.9 / 10.6 / 11.2; 1M-vertex power-law graph 100,000
-// edges 0.64 / 0.53 / 0.60 / 1.85, 200,000 1.01 / 0.81 / 0.78 / 2.25, 1.0M 4.2 /
-// 3.1 / 2.6 / 3.8, 2.0M 8.1 / 6.5 / 5.5 / 6.0, 5M 18.3 / 13.9 / 11.8 / 11.2,
-// exact (20M) 66 / 49 / 42 / 35. Without a limit short lists go to single lanes
+// pass) 2.46 / 2.57 / 2.59 / 2.90 ms the whole call; R-MAT 22 19,000 edges 0.34 /
+// 0.32 / 0.34 / 1.50 ms, 64,000 0.69 / 0.66 / 0.64 / 2.6, 193,000 1.56 / 1.48 /
+// 1.25 / 2.9, 1.9M 12.3 / 11.4 / 8.9 / 11.2; 1M-vertex power-law graph 100,000
+// edges 0.54 / 0.46 / 0.52 / 1.81, 200,000 0.88 / 0.71 / 0.72 / 2.26, 1.0M 3.5 /
+// 2.8 / 2.4 / 3.8, 2.0M 6.6 / 5.1 / 4.7 / 6.0, 5M 16.1 / 12.2 / 10.7 / 11.2,
+// exact (20M) 65 / 49 / 42 / 35. Without a limit short lists go to single lanes
 // (ER of mean degree 4, 4M edges 1.5 -> 0.13), so that begins at 2^21 already.
 inline int64_t compact_long(int64_t K) {
   return K < (1 << 15) ? 1024 : K < (1 << 17) ? 2048 : K < (1 << 21) ? 4096 : INT64_MAX;
@@ -600,14 +600,16 @@ __global__ void __launch_bounds__(kThreads, kCompactBlocksPerSm)
                       sh);
   }
   __syncthreads();
-  // the CTA looks at `look` edges at a time for long lists: few enough that a
-  // small sample is spread over all CTAs
-  const int look = (int)min((int64_t)kThreads, max((int64_t)1, K / gridDim.x));
-  for (int64_t b = (int64_t)blockIdx.x * look; b < K; b += (int64_t)gridDim.x * look) {
+  // the CTA looks for long lists among edges that lie gridDim apart: in a sample
+  // in edge order the edges of hubs with neighbouring ids follow one another
+  // (R-MAT 20 1% with ids by degree: 0.80 ms by a warp per edge, 5.1 by the CTA
+  // that had a hub's edges, 0.45 so)
+  const int64_t step = gridDim.x;
+  for (int64_t b = blockIdx.x; b < K; b += step * kThreads) {
     __shared__ uint32_t todo[kThreads / 32];
-    const int64_t e = b + threadIdx.x;
+    const int64_t e = b + step * threadIdx.x;
     bool is_long = false;
-    if ((int)threadIdx.x < look && e < K) {
+    if (e < K) {
       const int32_t u = uv[e].x;
       is_long = __ldg(g.row_ptr + u + 1) - __ldg(g.row_ptr + u) > long_list;
     }
@@ -616,7 +618,7 @@ __global__ void __launch_bounds__(kThreads, kCompactBlocksPerSm)
     __syncthreads();
     for (int w = 0; w < kThreads / 32; ++w)
       for (unsigned m = todo[w]; m; m &= m - 1) {
-        const int64_t el = b + w * 32 + __ffs(m) - 1;
+        const int64_t el = b + step * (w * 32 + __ffs(m) - 1);
         compact_edge<kThreads / 32>(g, el, uv[el].x, off, toff, tbits, T, tpre, T_hm, tdeg,
                                     mask_idx, dense_counter, sh);
       }

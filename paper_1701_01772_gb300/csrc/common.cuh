@@ -107,7 +107,8 @@ struct DevGraph {
   // order) and v's neighbours above v without a matrix slot; hm_vertex =
   // vertex of each matrix slot (all NULL without a matrix)
   const int64_t* mn_ptr;   // [n+1]
-  const int16_t* mn_slot;  // [mn_ptr[n]]
+  const int16_t* mn_slot;  // [mn_total]
+  int64_t mn_total;        // mn_ptr[n]: adjacency entries with a matrix slot
   const int64_t* nm_ptr;   // [n+1]
   const int32_t* nm_col;   // [nm_ptr[n]]
   const int32_t* hm_vertex;  // [hm_count]

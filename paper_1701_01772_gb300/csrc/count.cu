@@ -124,13 +124,18 @@ constexpr int64_t kQuadGrabTests = GS_QUAD_GRAB_TESTS;
 // Resident warps per SM of k_dense_pairs (at most 40 registers), in CTAs of
 // 256 threads, or of 128 when there are many units: the five to seven barriers
 // of a unit hold up the warps of a small CTA less, but a unit with long lists of
-// other members is walked by fewer warps. 4-node phase with 128 and with 256
-// threads, 1M-vertex power-law graph: 34,000 dense edges 1.90 and 1.82 ms,
-// 68,000 3.21 and 3.29, 169,000 7.18 and 7.81, 1.7M 65.1 and 73.2; R-MAT 22:
-// 34,000 8.12 and 7.78, 85,000 17.92 and 17.85, 169,000 32.8 and 34.1. The line
-// lies at kManyDensePerCta dense edges per resident CTA of 256 (73,000 in all).
+// other members is walked by fewer warps, so that only graphs whose adjacency
+// entries have matrix slots for the most part take small CTAs. 4-node phase with
+// 128 and with 256 threads, and the share of entries with slots: 1M-vertex
+// power-law graph (0.54) 34,000 dense edges 1.90 and 1.82 ms, 68,000 3.21 and
+// 3.29, 169,000 7.18 and 7.81, 1.7M 65.1 and 73.2; R-MAT 20 (0.69) 84,000 3.57
+// and 3.82; R-MAT 22 (0.52) 34,000 8.12 and 7.78, 85,000 17.92 and 17.85, 169,000
+// 32.8 and 34.1; R-MAT 24 (0.36) 32,000 65.4 and 60.3, 95,000 176 and 170,
+// 317,000 549 and 542. The line lies at kManyDensePerCta dense edges per
+// resident CTA of 256 (73,000 in all) and a share of 0.45.
 constexpr int kDenseWarpsPerSm = 48;
 constexpr int64_t kManyDensePerCta = 80;
+constexpr double kSmallCtaShare = 0.45;
 constexpr int kTriBlocksPerSm = 6;  // k_tri_chunks: at most 40 registers
 // T entries per k_dense_pairs work unit (a heavy dense edge is split into
 // several units so that small samples still fill the GPU).
@@ -2036,7 +2041,9 @@ int64_t launch_dense(const DevGraph& g, bool need_q, CountBufs& b, cudaStream_t 
         need_q ? 1 : 0, b.k2, b.q, b.stats + 7, b.stats + 4, b.stats + 9);
   };
   const int64_t resident = (int64_t)sm_count() * (kDenseWarpsPerSm * 32 / 256);
-  if (b.ndense >= kManyDensePerCta * resident) go(k_dense_pairs<128>, 128);
+  if (b.ndense >= kManyDensePerCta * resident &&
+      (double)g.mn_total >= kSmallCtaShare * (double)g.nnz)
+    go(k_dense_pairs<128>, 128);
   else go(k_dense_pairs<256>, 256);
   return 1;
 }

@@ -1274,6 +1274,7 @@ static gs_status build_hub_index(gs_graph* g, uint64_t budget, int64_t held, cud
     GS_CUDA(cudaStreamSynchronize(stream));
     g->dev.mn_ptr = g->mn_ptr;
     g->dev.mn_slot = g->mn_slot;
+    g->dev.mn_total = tot[0];
     g->dev.nm_ptr = g->nm_ptr;
     g->dev.nm_col = g->nm_col;
     g->dev.hm_vertex = g->hm_vertex;

@@ -75,38 +75,47 @@ __global__ void k_orient_count(const int64_t* __restrict__ row_ptr, const int32_
 }
 
 // Out-list (higher-ranked neighbours) and in-list (lower-ranked ones) of
-// every vertex, both in increasing id (one warp per vertex).
-__global__ void k_orient_fill(const int64_t* __restrict__ row_ptr, const int32_t* __restrict__ col,
-                              int64_t n, const int64_t* __restrict__ out_ptr,
-                              const int64_t* __restrict__ in_ptr, int32_t* __restrict__ out_col,
-                              int32_t* __restrict__ in_col) {
+// every vertex, both in increasing id (one warp per vertex). Lists longer than
+// a warp have several steps' loads in flight, as a hub's list is the kernel's
+// tail; the others are one step (2M vertices of mean degree 4: 0.23 ms with one
+// step for all, 0.50 with four, 0.21 so).
+__global__ void __launch_bounds__(kThreads, 8)
+    k_orient_fill(const int64_t* __restrict__ row_ptr, const int32_t* __restrict__ col, int64_t n,
+                  const int64_t* __restrict__ out_ptr, const int64_t* __restrict__ in_ptr,
+                  int32_t* __restrict__ out_col, int32_t* __restrict__ in_col) {
   const int lane = threadIdx.x & 31;
+  const unsigned below = (1u << lane) - 1u;
   const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
   for (int64_t v = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; v < n; v += warps) {
-    const int64_t dv = row_ptr[v + 1] - row_ptr[v];
+    const int64_t begin = row_ptr[v], end = row_ptr[v + 1], dv = end - begin;
     int64_t o = out_ptr[v], i = in_ptr[v];
-    const int64_t end = row_ptr[v + 1];
-    // several steps' loads in flight (a hub's list is the kernel's tail)
+    // one step: x = -1 past the list
+    auto place = [&](int32_t x, bool up) {
+      const unsigned bu = __ballot_sync(kFull, x >= 0 && up);
+      const unsigned bd = __ballot_sync(kFull, x >= 0 && !up);
+      if (x >= 0 && up) out_col[o + __popc(bu & below)] = x;
+      if (x >= 0 && !up) in_col[i + __popc(bd & below)] = x;
+      o += __popc(bu);
+      i += __popc(bd);
+    };
+    auto ranked = [&](int32_t x) {
+      return x >= 0 && ranks_above(__ldg(row_ptr + x + 1) - __ldg(row_ptr + x), x, dv, (int32_t)v);
+    };
+    if (dv <= 32) {
+      const int32_t x = lane < dv ? col[begin + lane] : -1;
+      place(x, ranked(x));
+      continue;
+    }
     constexpr int kDeep = 4;
-    for (int64_t p0 = row_ptr[v] + lane; p0 - lane < end; p0 += 32 * kDeep) {
+    for (int64_t p0 = begin + lane; p0 - lane < end; p0 += 32 * kDeep) {
       int32_t x[kDeep];
-      int64_t d[kDeep];
+      bool up[kDeep];
 #pragma unroll
       for (int h = 0; h < kDeep; ++h) x[h] = p0 + 32 * h < end ? col[p0 + 32 * h] : -1;
 #pragma unroll
-      for (int h = 0; h < kDeep; ++h)
-        d[h] = x[h] >= 0 ? __ldg(row_ptr + x[h] + 1) - __ldg(row_ptr + x[h]) : 0;
+      for (int h = 0; h < kDeep; ++h) up[h] = ranked(x[h]);
 #pragma unroll
-      for (int h = 0; h < kDeep; ++h) {
-        const bool live = x[h] >= 0, up = ranks_above(d[h], x[h], dv, (int32_t)v);
-        const unsigned bu = __ballot_sync(kFull, live && up);
-        const unsigned bd = __ballot_sync(kFull, live && !up);
-        const unsigned below = (1u << lane) - 1u;
-        if (live && up) out_col[o + __popc(bu & below)] = x[h];
-        if (live && !up) in_col[i + __popc(bd & below)] = x[h];
-        o += __popc(bu);
-        i += __popc(bd);
-      }
+      for (int h = 0; h < kDeep; ++h) place(x[h], up[h]);
     }
   }
 }

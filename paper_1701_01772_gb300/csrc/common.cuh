@@ -44,17 +44,11 @@ __device__ __forceinline__ void raise_error(DevError* err, int32_t code, int64_t
 // highest-degree vertices, which most tests touch, stay resident). On R-MAT
 // scale 24 the 1% estimate took 3.69 s with 16384 vertices and 3.22 s with
 // 32767 (more edges go dense, fewer single tests).
-#ifndef GS_HUB_MATRIX_MAX
-#define GS_HUB_MATRIX_MAX 32767
-#endif
-constexpr int64_t kHubMatrixMax = GS_HUB_MATRIX_MAX;
+constexpr int64_t kHubMatrixMax = 32767;
 static_assert(kHubMatrixMax <= 32767, "matrix slots are stored in 16 bits");
 // Default number of matrix slots (the highest-degree vertices) that take
 // part in dense clique mode; the rest of the matrix answers single tests.
-#ifndef GS_HUB_DENSE_SLOTS
-#define GS_HUB_DENSE_SLOTS GS_HUB_MATRIX_MAX
-#endif
-constexpr int64_t kHubDenseSlots = GS_HUB_DENSE_SLOTS;
+constexpr int64_t kHubDenseSlots = kHubMatrixMax;
 
 // Device view of a registered graph plus its hub index.
 struct DevGraph {

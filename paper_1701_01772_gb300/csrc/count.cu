@@ -59,10 +59,7 @@ constexpr int kThreads = 256;
 // k_chunk_cost: 6 CTAs per SM (at most 40 registers) hide more of its
 // dependent loads than 4 do.
 constexpr int kCostBlocksPerSm = 6;
-#ifndef GS_QUAD_BLOCKS_PER_SM
-#define GS_QUAD_BLOCKS_PER_SM 8
-#endif
-constexpr int kQuadBlocksPerSm = GS_QUAD_BLOCKS_PER_SM;
+constexpr int kQuadBlocksPerSm = 8;
 constexpr unsigned kFull = 0xffffffffu;
 // An edge whose T has at least this many hub-matrix members, and whose
 // dense-mode work is the smaller, counts the pairs among them with
@@ -117,10 +114,7 @@ __device__ __forceinline__ uint32_t tfilter_hash(int32_t x) {
 // run searches its place and sets up its packs anew. R-MAT 24 0.1%: 185 / 159
 // / 144 / 138 / 143 ms at 512 / 1024 / 2048 / 4096 / 16384 tests; batch of
 // 1024 graphs 60.6 / 58.8 / 57.9 / 57.6 / 59.6 ms.
-#ifndef GS_QUAD_GRAB_TESTS
-#define GS_QUAD_GRAB_TESTS 4096
-#endif
-constexpr int64_t kQuadGrabTests = GS_QUAD_GRAB_TESTS;
+constexpr int64_t kQuadGrabTests = 4096;
 // Resident warps per SM of k_dense_pairs (at most 40 registers), in CTAs of
 // 256 threads, or of 128 when there are many units: the five to seven barriers
 // of a unit hold up the warps of a small CTA less, but a unit with long lists of
@@ -146,10 +140,7 @@ constexpr int kHubMatrixMaxGroups = (int)((kHubMatrixMax + 127) / 128);
 constexpr int kGroupWords = (kHubMatrixMaxGroups + 31) / 32;
 // Cost of one 128-bit dense group against one membership test, in quarters
 // (the dense-mode choice compares kGroupCost * groups with 4 * tests).
-#ifndef GS_DENSE_GROUP_COST
-#define GS_DENSE_GROUP_COST 4
-#endif
-constexpr int kGroupCost = GS_DENSE_GROUP_COST;
+constexpr int kGroupCost = 4;
 
 template <class T>
 __device__ __forceinline__ T warp_sum(T v) {
@@ -1245,8 +1236,6 @@ __global__ void __launch_bounds__(kThreads, kCostBlocksPerSm)
 
 // ---------------------------------------------------------------- quad
 
-// Item descriptors of the chunk a warp is working on, in shared memory so a
-// lane can read the item its test belongs to.
 // Membership of x in a directory bucket p[0..len): short buckets (the usual
 // case: 2 to 4 entries) are compared entry by entry with independent loads.
 __device__ __forceinline__ bool bucket_contains(const int32_t* __restrict__ p, int32_t len,

@@ -20,10 +20,7 @@ constexpr int64_t kDirMinDegree = 16;
 // 65,250 columns at 96 GiB (the 1% 4-node estimate in 1.02 s, against
 // 2.08 s with 234,019 x 16,317 under a cap of 1.6e11 and 20 GiB).
 constexpr int64_t kMidMinDegree = 2;
-#ifndef GS_MID_WORK_MAX
-#define GS_MID_WORK_MAX 640000000000ull
-#endif
-constexpr unsigned long long kMidWorkMax = GS_MID_WORK_MAX;
+constexpr unsigned long long kMidWorkMax = 640000000000ull;
 
 // ------------------------------------------------------------- validation
 // One warp per row (grid-stride). Checks the simple-graph conditions of
@@ -442,10 +439,7 @@ __global__ void __launch_bounds__(kBlockRowThreads, 2048 / kBlockRowThreads)
 // power-law graph (91,000 rows of 17.6 KB, 256 threads): 33.4 -> 28.3 ms. The
 // rows of k_table_rows are hubs with long lists: 1024 threads, two CTAs per SM
 // where they fit (256 threads: 6.6 against 5.0 ms there).
-#ifndef GS_BIG_MAX
-#define GS_BIG_MAX 65536
-#endif
-constexpr int kBigMax = GS_BIG_MAX;
+constexpr int kBigMax = 65536;
 static_assert(kBigMax <= 65536, "column slots are stored in 16 bits");  // 7 shapes from kBigMin
 constexpr int kBigMin = 1024;  // narrowest shape tried
 
@@ -882,8 +876,6 @@ __global__ void k_giant_index(const int64_t* __restrict__ flag_scan, int64_t cou
     giant[s] = flag_scan[s + 1] > flag_scan[s] ? (int32_t)flag_scan[s] : -1;
 }
 
-// Marks the 16-bit entries of giant pairs 0xFFFF (answered by the giant
-// table). One thread per slot a; only giant rows do work.
 // Co-degree table among the table vertices, one row at a time: row a holds
 // c(a, b) for b > a (contiguous in tb_index order), the number of x in N(a)
 // with b in N(x). A CTA accumulates the row in shared memory (16-bit
@@ -952,6 +944,8 @@ __global__ void __launch_bounds__(kRowThreads, 2048 / kRowThreads)
   }
 }
 
+// Marks the 16-bit entries of giant pairs 0xFFFF (answered by the giant
+// table). One thread per slot a; only giant rows do work.
 __global__ void k_mark_giant_pairs(const int32_t* __restrict__ giant, int64_t count,
                                    uint32_t* __restrict__ words) {
   for (int64_t a = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; a < count;

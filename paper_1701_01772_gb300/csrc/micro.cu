@@ -57,10 +57,7 @@ namespace {
 
 constexpr int kThreads = 256;
 constexpr unsigned kFull = 0xffffffffu;
-#ifndef GS_PROBE_BLOCKS
-#define GS_PROBE_BLOCKS 5
-#endif
-constexpr int kProbeBlocksPerSm = GS_PROBE_BLOCKS;
+constexpr int kProbeBlocksPerSm = 5;
 constexpr int64_t kTaskProbes = 512;
 // Tasks a probe warp takes from the counter, at most (a run sets its chunks up
 // anew: 26.0 / 19.1 / 18.3 ms at 1 / 8 / 32 tasks).

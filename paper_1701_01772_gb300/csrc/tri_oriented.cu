@@ -34,15 +34,9 @@ constexpr unsigned kFull = 0xffffffffu;
 constexpr int64_t kInChunk = 256;      // in-neighbours per work unit
 constexpr int32_t kMaxOutDegree = 4096;  // larger out-lists: the general pass
 // Resident CTAs per SM (as far as shared memory allows).
-#ifndef GS_ORIENT_BLOCKS_PER_SM
-#define GS_ORIENT_BLOCKS_PER_SM 8
-#endif
-constexpr int kOrientBlocksPerSm = GS_ORIENT_BLOCKS_PER_SM;
+constexpr int kOrientBlocksPerSm = 8;
 // Out-list entries a lane loads before it probes them (loads in flight).
-#ifndef GS_PROBE_BATCH
-#define GS_PROBE_BATCH 4
-#endif
-constexpr int kProbeBatch = GS_PROBE_BATCH;
+constexpr int kProbeBatch = 4;
 
 typedef unsigned __int128 u128;
 

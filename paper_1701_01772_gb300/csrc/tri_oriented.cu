@@ -72,7 +72,7 @@ __global__ void k_orient_count(const int64_t* __restrict__ row_ptr, const int32_
 // every vertex, both in increasing id (one warp per vertex). Lists longer than
 // a warp have several steps' loads in flight, as a hub's list is the kernel's
 // tail; the others are one step (2M vertices of mean degree 4: 0.23 ms with one
-// step for all, 0.50 with four, 0.21 so).
+// step for all, 0.50 with four, 0.22 so).
 __global__ void __launch_bounds__(kThreads, 8)
     k_orient_fill(const int64_t* __restrict__ row_ptr, const int32_t* __restrict__ col, int64_t n,
                   const int64_t* __restrict__ out_ptr, const int64_t* __restrict__ in_ptr,
@@ -92,24 +92,22 @@ __global__ void __launch_bounds__(kThreads, 8)
       o += __popc(bu);
       i += __popc(bd);
     };
-    auto ranked = [&](int32_t x) {
-      return x >= 0 && ranks_above(__ldg(row_ptr + x + 1) - __ldg(row_ptr + x), x, dv, (int32_t)v);
-    };
     if (dv <= 32) {
       const int32_t x = lane < dv ? col[begin + lane] : -1;
-      place(x, ranked(x));
+      const int64_t d = x >= 0 ? __ldg(row_ptr + x + 1) - __ldg(row_ptr + x) : 0;
+      place(x, ranks_above(d, x, dv, (int32_t)v));
       continue;
     }
     constexpr int kDeep = 4;
     for (int64_t p0 = begin + lane; p0 - lane < end; p0 += 32 * kDeep) {
-      int32_t x[kDeep];
-      bool up[kDeep];
+      int32_t x[kDeep], d[kDeep];  // degrees are below 2^31
 #pragma unroll
       for (int h = 0; h < kDeep; ++h) x[h] = p0 + 32 * h < end ? col[p0 + 32 * h] : -1;
 #pragma unroll
-      for (int h = 0; h < kDeep; ++h) up[h] = ranked(x[h]);
+      for (int h = 0; h < kDeep; ++h)
+        d[h] = x[h] >= 0 ? (int32_t)(__ldg(row_ptr + x[h] + 1) - __ldg(row_ptr + x[h])) : 0;
 #pragma unroll
-      for (int h = 0; h < kDeep; ++h) place(x[h], up[h]);
+      for (int h = 0; h < kDeep; ++h) place(x[h], ranks_above(d[h], x[h], dv, (int32_t)v));
     }
   }
 }
